@@ -59,7 +59,10 @@ WORKLOAD = ("64^3 lid-driven cavity, Re=1000, u_lid=1, walls on all faces; initi
 #   mg_lap_t   t = L z, (t, s), (t, t): z, s -> t
 #   krylov_C   x += alpha y + omega z, r = s - omega t: x, y, z, s, t, r_hat -> x, r
 WORDS_MG = {"krylov_A": 5, "mg_restrict0": 2.125, "mg_prolong0": 2.125, "mg_lap_v": 3,
-            "krylov_B": 4, "mg_lap_t": 3, "krylov_C": 8}
+            "krylov_B": 4, "mg_lap_t": 3, "krylov_C": 8,
+            # direct solve (boxes without solid cells): a plane's transforms and
+            # the equations along z read and write the field once each
+            "direct_xy": 2, "direct_z": 2}
 # plain BiCGStab: A reads r, p, v, r_hat, writes p, v; B reads r, v, writes t;
 # C reads x, p, r, v, t, r_hat, writes x, r
 WORDS_PLAIN = {"krylov_A": 6, "krylov_B": 3, "krylov_C": 8}
@@ -84,6 +87,7 @@ KERNEL_NAMES = {"krylov_A": "k_mg_src_pair<SRC_P> / k_mg_src<SRC_P> / k_bicg_A",
                 "mg_restrict0": "k_mg_restrict (finest)",
                 "mg_prolong0": "k_mg_prolong_pair / k_mg_prolong (finest)", "predict": "k_predict_tile",
                 "divergence": "k_divergence", "correct": "k_correct_ff",
+                "direct_xy": "k_dir_xy", "direct_z": "k_dir_z",
                 "solve_init": "k_mg_refine_init_ff", "refine": "k_mg_refine_update_ff"}
 
 

@@ -80,6 +80,15 @@ typedef struct {
                                 (NS_PC_NONE) or with one multigrid V-cycle as right
                                 preconditioner (NS_PC_MULTIGRID; falls back to
                                 NS_PC_NONE on grids it cannot coarsen far enough).
+                                With NS_PC_MULTIGRID, a box without solid cells
+                                whose planes fit one SM's shared memory takes its
+                                corrections from a direct solve of L e = r instead
+                                (transforms along x and y, three-point equations
+                                along z; the same stopping tolerances, one
+                                application counted as one iteration), unless its
+                                tolerance is below 1e-14; NS_DIRECT=0 in the
+                                environment at ns_create_grid, or any of the
+                                multigrid's variables below, keeps the V-cycle.
                                 The levels with at most 4096 cells (FP32_REFINE;
                                 512 in FP64) run in one CTA per state; the
                                 environment variable NS_MG_BLOCK_CELLS, read at
@@ -282,7 +291,9 @@ typedef enum {
                               launch (small batches, multigrid preconditioner)    */
     NS_K_MG_CLUSTER = 18,  /* multigrid: the coarse levels on a thread-block cluster
                               per state (everything below the finest level)       */
-    NS_K_KINDS = 19
+    NS_K_DIRECT_XY = 19,   /* direct solve: transforms of the planes along x and y   */
+    NS_K_DIRECT_Z = 20,    /* direct solve: the three-point equations along z        */
+    NS_K_KINDS = 21
 } ns_kernel_kind;
 
 typedef struct {

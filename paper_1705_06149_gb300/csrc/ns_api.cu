@@ -19,6 +19,7 @@
 
 #include "ns.h"
 #include "ns_adjoint.cuh"
+#include "ns_direct.cuh"
 #include "ns_mg.cuh"
 #include "ns_mg_cluster.cuh"
 #include "ns_persist.h"
@@ -96,6 +97,15 @@ struct ns_grid {
     bool cl = false;
     ClPlan cplan{};
     size_t cl_smem = 0;
+    // pressure corrections by the direct solve (boxes without solid cells):
+    // mg stays set (the solves share the multigrid path's start, correction
+    // and graphs), hier tells whether the grid has the hierarchy's levels
+    bool dir = false;
+    bool hier = false;
+    DirPlan<float> dirf{};
+    DirPlan<double> dird{};
+    size_t dir_smem = 0;
+    int dir_hint = 2;  // applications the last solves took
     void* mg_vec[3] = {};                       // Y, Z, S at level 0
     void* mg_B[MG_MAX_LEVELS] = {};             // restricted right sides, levels 1..lc
     void* mg_Y[MG_MAX_LEVELS] = {};             // level iterates, levels 1..lc
@@ -437,6 +447,53 @@ bool cluster_ready(ns_grid* g) {
     return cudaOccupancyMaxActiveClusters(&n, k_mg_cluster<T>, &cfg) == cudaSuccess && n >= 1;
 }
 
+template <typename T>
+ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
+    const Geo& G = g->geo;
+    if (!dir_sizes<T>(G.n, G.bc[2] == BC_PERIODIC, G.n[2] * g->cap, P)) return NS_OK;
+    size_t off[5];
+    const std::vector<T> tab = dir_tables<T>(P, G.bc, G.ih2, off);
+    void* dev = nullptr;
+    NS_TRY(dalloc(g, &dev, tab.size() * sizeof(T)));
+    if (cudaMemcpy(dev, tab.data(), tab.size() * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess)
+        return fail(NS_ERR_CUDA, "ns_create_grid: copy of the direct solve's tables failed");
+    const T* t = (const T*)dev;
+    P.rx[0] = t + off[0];
+    P.rx[1] = t + off[1];
+    P.ly[0] = t + off[2];
+    P.ly[1] = t + off[3];
+    P.col = t + off[4];
+    g->dir_smem = dir_smem_elems(P) * sizeof(T);
+    if (cudaFuncSetAttribute(k_dir_xy<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)DIR_MAX_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(k_dir_xy<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)DIR_MAX_SMEM) != cudaSuccess)
+        return fail(NS_ERR_CUDA, "ns_create_grid: direct solve shared memory attribute");
+    g->dir = true;
+    g->mg = true;
+    return NS_OK;
+}
+
+// Whether the grid's pressure corrections come from the direct solve: a box
+// without solid cells whose planes fit shared memory, conditioned well enough
+// that one application reduces the residual at least about 25 times in the
+// grid's precision (measured: 4e-9 of the residual times the condition number
+// stay in FP32, 1e-17 in FP64), and a tolerance that a residual of that
+// precision can mean (below it the Krylov recursion decides, as it always
+// did).  The environment variables that select a form of the multigrid solve
+// (NS_MG_CLUSTER, NS_MG_BLOCK_CELLS, NS_PERSISTENT), when set, select it;
+// NS_DIRECT=0 turns the direct solve off.
+ns_status setup_direct(ns_grid* g) {
+    for (const char* v : {"NS_MG_CLUSTER", "NS_MG_BLOCK_CELLS", "NS_PERSISTENT"})
+        if (std::getenv(v)) return NS_OK;
+    const char* env = std::getenv("NS_DIRECT");
+    if ((env && std::atoi(env) == 0) || g->geo.solid) return NS_OK;
+    const double rtol = g->fp32 ? g->d.refine_rtol : g->d.poisson_rtol;
+    const double cond = dir_condition(g->geo.n, g->geo.bc, g->geo.ih2);
+    if (!(rtol >= 1e-14) || !(cond <= (g->fp32 ? 1e7 : 1e12))) return NS_OK;
+    return g->fp32 ? setup_direct_of<float>(g, g->dirf) : setup_direct_of<double>(g, g->dird);
+}
+
 ns_status check_state(const ns_grid* g, const ns_state& s, const char* what) {
     if (!s.u || !s.v || !s.w || !s.p)
         return fail(NS_ERR_ARG, std::string(what) + ": null state pointer");
@@ -727,6 +784,55 @@ void mg_apply(ns_grid* g, int batch, MgBuf<T>& mb, T* src, T* src_odd, T* dst) {
                       k_mg_prolong<T><<<dim3(L.ctas, batch), blk, 0, g->stream>>>(
                           L, P.lev[l + 1], g->ctl, y, mb.Yl[l + 1]));
         }
+    }
+}
+
+template <typename T> const DirPlan<T>& dirplan(const ns_grid* g);
+template <> const DirPlan<float>& dirplan<float>(const ns_grid* g) { return g->dirf; }
+template <> const DirPlan<double>& dirplan<double>(const ns_grid* g) { return g->dird; }
+
+// e = L^-1 r for every active state: the residual of the solve in kv[1], the
+// spectral planes in kv[3], e in kv[0] (FP32+refine) or kv[4] (FP64).
+template <typename T>
+void direct_apply(ns_grid* g, int batch) {
+    const DirPlan<T>& P = dirplan<T>(g);
+    const T* r = (const T*)g->kv[1];
+    T* spec = (T*)g->kv[3];
+    T* e = (T*)g->kv[sizeof(T) == 4 ? 0 : 4];
+    const dim3 pg(P.nz * P.xb, batch), zg(ceil_div(P.nx * P.ny, DIR_ZX), batch);
+    const dim3 zb(DIR_ZX, P.zc);
+    const long long units = P.cells * batch;
+    NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+              (k_dir_xy<T, false><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, r, spec)));
+    if (P.zm == DIR_ZC)
+        NS_LAUNCH(g, NS_K_DIRECT_Z, units,
+                  (k_dir_z<T, DIR_ZC><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
+    else
+        NS_LAUNCH(g, NS_K_DIRECT_Z, units,
+                  (k_dir_z<T, DIR_ZC_LONG><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
+    NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+              (k_dir_xy<T, true><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, spec, e)));
+}
+
+// One application of the direct solve and the correction with it (p += e,
+// r -= L e, the decision), on every state still active.
+void direct_correct(ns_grid* g, int batch) {
+    const Lev& L0 = g->plan.lev[0];
+    const dim3 grid(L0.ctas, batch), blk = block_dim();
+    const long long units = L0.cells * batch;
+    if (g->fp32) {
+        direct_apply<float>(g, batch);
+        NS_LAUNCH(g, NS_K_REFINE, units,
+                  k_mg_refine_update_ff<<<grid, blk, 0, g->stream>>>(
+                      L0, mgbuf<float>(g), g->ctl, ffbuf(g), g->geo.n_fluid, g->part_mg,
+                      g->d.refine_rtol * g->d.refine_rtol, g->inner_rtol * g->inner_rtol,
+                      g->maxit, g->max_outer, 0));
+    } else {
+        direct_apply<double>(g, batch);
+        NS_LAUNCH(g, NS_K_REFINE, units,
+                  k_dir_update<<<grid, blk, 0, g->stream>>>(
+                      L0, mgbuf<double>(g), g->ctl, (const double*)g->kv[4], g->part_mg,
+                      g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid));
     }
 }
 
@@ -1123,7 +1229,10 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
         NS_TRY(make_handle(g->stream, &h));
         NS_TRY(loop_cond(g, batch, h, LC_FP64_START, cap_inner));
         return add_while(g, g->body_stream[0], h, [&]() -> ns_status {
-            NS_TRY(mg_iteration<double>(g, batch, tol2, 0));
+            if (g->dir)
+                direct_correct(g, batch);
+            else
+                NS_TRY(mg_iteration<double>(g, batch, tol2, 0));
             return loop_cond(g, batch, h, LC_FP64_ITER, cap_inner);
         });
     }
@@ -1139,6 +1248,10 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
     NS_TRY(make_handle(g->stream, &h));
     NS_TRY(loop_cond(g, batch, h, LC_REFINE_START, cap_refine));
     return add_while(g, g->body_stream[0], h, [&]() -> ns_status {
+        if (g->dir) {
+            direct_correct(g, batch);
+            return loop_cond(g, batch, h, LC_REFINE_ITER, cap_refine);
+        }
         NS_TRY(mg_iteration<float>(g, batch, itol2, 1));
         NS_LAUNCH(g, NS_K_REFINE, 0,
                   k_mg_refine_update_ff<<<grid, blk, 0, g->stream>>>(
@@ -1149,8 +1262,64 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
     });
 }
 
+// The solve by direct corrections on the stream path: as many as the last
+// solves took are issued back to back, then the flags are polled after each.
+ns_status solve_pressure_direct(ns_grid* g, int batch, const double* p_in) {
+    const Lev& L0 = g->plan.lev[0];
+    const dim3 grid(L0.ctas, batch), blk = block_dim();
+    if (g->fp32)
+        launch_refine_init_ff(g, batch, p_in, g->d.refine_rtol * g->d.refine_rtol,
+                              g->inner_rtol * g->inner_rtol);
+    else
+        NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
+                  k_mg_init_warm<double><<<grid, blk, 0, g->stream>>>(
+                      L0, mgbuf<double>(g), g->ctl, g->part_div, g->geo.n_fluid, g->b,
+                      p_in ? p_in : g->p_prev, g->part_mg,
+                      g->d.poisson_rtol * g->d.poisson_rtol, g->maxit));
+    NS_CUDA(cudaGetLastError());
+    const int limit = (g->fp32 ? g->max_outer : g->maxit) + 2;
+    for (int it = 1; it <= limit; ++it) {
+        direct_correct(g, batch);
+        NS_CUDA(cudaGetLastError());
+        if (it < g->dir_hint && it < limit) continue;
+        NS_TRY(poll_ctl(g, batch));
+        bool any = false;
+        for (int s = 0; s < batch; ++s)
+            any |= g->fp32 ? g->h_ctl[s].o_status == OS_REFINE : g->h_ctl[s].status == ST_ITER;
+        if (!any) break;
+    }
+    int mx = 0;
+    double mr = 0.0;
+    ns_status st = NS_OK;
+    for (int s = 0; s < batch; ++s) {
+        const SliceCtl& c = g->h_ctl[s];
+        const int its = g->fp32 ? c.o_steps : c.it_cur;
+        const double rr = g->fp32 ? c.o_rr : c.rr, bb = g->fp32 ? c.o_bb : c.bb;
+        const double rel = bb > 0 ? std::sqrt(rr / bb) : std::sqrt(rr);
+        mx = std::max(mx, its);
+        mr = std::max(mr, rel);
+        g->stats.krylov_iters += its;
+        if (g->fp32) g->stats.refine_steps += its;
+        const bool bad = g->fp32 ? c.o_status == OS_NONFINITE : c.status == ST_NONFINITE;
+        const bool done = g->fp32 ? c.o_status == OS_DONE : c.status == ST_CONV;
+        if (bad)
+            st = fail(NS_ERR_NONFINITE, "non-finite residual in the pressure solve");
+        else if (!done && st == NS_OK)
+            st = fail(NS_ERR_NOT_CONVERGED,
+                      "pressure solve did not reach its tolerance (relative residual " +
+                          std::to_string(rel) + ")");
+    }
+    g->dir_hint = std::max(1, mx);
+    if (st != NS_OK) return st;
+    g->stats.solves += batch;
+    g->stats.last_max_iters = mx;
+    g->stats.last_rel_residual = mr;
+    return NS_OK;
+}
+
 ns_status solve_pressure_mg(ns_grid* g, int batch, const double* p_in) {
     if (g->capturing) return solve_pressure_mg_graph(g, batch, p_in);
+    if (g->dir) return solve_pressure_direct(g, batch, p_in);
     if (g->persist && batch <= g->persist_max_batch) return solve_pressure_persist(g, batch, p_in);
     const Lev& L0 = g->plan.lev[0];
     const dim3 grid(L0.ctas, batch), blk = block_dim();
@@ -1482,6 +1651,7 @@ ns_status parareal_update(ns_grid* g, const void* const fy[4], const void* const
 
 // Kernels one preconditioned iteration launches (mg_apply twice + 3).
 long long mg_iteration_launches(const ns_grid* g) {
+    if (g->dir) return g->fp32 ? 3 : 4;  // the correction counts with FP32+refine's
     const int lc = g->plan.lc;
     const long long apply = 1 + lc + std::max(lc - 1, 0) + 1 + lc;
     return 2 * apply + 3;
@@ -2408,6 +2578,8 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
         const char* env = std::getenv("NS_MG_BLOCK_CELLS");
         const int block_cells = env ? std::max(8, std::atoi(env)) : (g->fp32 ? 4096 : 512);
         g->mg = setup_mg(g, block_cells, ev, d.solid_mask != nullptr);
+        g->hier = g->mg;
+        st = setup_direct(g);
         if (g->mg && d.solid_mask) {
             // solid cells enter the finest level through its face codes
             const std::vector<uint8_t> code = face_codes(g->geo, d.solid_mask);
@@ -2420,8 +2592,8 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
         }
     }
     if (g->mg) {
-        for (int q = 0; q < 3; ++q) A(&g->mg_vec[q], ncell * ev * B);
-        for (int l = 1; l <= g->plan.lc; ++l) {
+        for (int q = 0; q < 3 && !g->dir; ++q) A(&g->mg_vec[q], ncell * ev * B);
+        for (int l = 1; l <= g->plan.lc && !g->dir; ++l) {
             A(&g->mg_B[l], (size_t)g->plan.lev[l].cells * ev * B);
             A(&g->mg_Y[l], (size_t)g->plan.lev[l].cells * ev * B);
         }
@@ -2432,7 +2604,7 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             for (int q = 0; q < 8; ++q) A((void**)&g->ffb[q], ncell * sizeof(float) * B);
         A((void**)&g->part_mg, nparts * 6 * sizeof(double));
     }
-    if (g->mg && st == NS_OK) {
+    if (g->mg && !g->dir && st == NS_OK) {
         // the coarse levels on a thread-block cluster per state, where they
         // split into slabs (NS_MG_CLUSTER=0 turns it off)
         const char* ce = std::getenv("NS_MG_CLUSTER");
@@ -2512,7 +2684,7 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             if (cudaMemsetAsync(g->counter, 0, sizeof(unsigned int) * B, g->stream) !=
                 cudaSuccess)
                 st = fail(NS_ERR_CUDA, "ns_create_grid: memset failed");
-            for (int q = 0; q < 3 && st == NS_OK; ++q)
+            for (int q = 0; q < 3 && !g->dir && st == NS_OK; ++q)
                 if (cudaMemsetAsync(g->mg_vec[q], 0, ncell * ev * B, g->stream) != cudaSuccess)
                     st = fail(NS_ERR_CUDA, "ns_create_grid: memset failed");
             // k_mg_block's shared memory stays within the default 48 KB
@@ -2924,7 +3096,7 @@ ns_status ns_graph_create(ns_grid* const* grids, const ns_state* states, const d
         for (int j = 0; j < i; ++j)
             if (grids[j] == g)
                 return fail(NS_ERR_ARG, "ns_graph_create: a grid appears in two branches");
-        if (!g->mg)
+        if (!g->hier)
             return fail(NS_ERR_ARG,
                         "ns_graph_create: graph-resident solves need the multigrid "
                         "preconditioner (branch " + std::to_string(i) + ")");

@@ -42,6 +42,7 @@ struct SliceCtl {
     float o_fsc;       // FP32+refine: the scale the next correction gives its right side
     float mean_hi, mean_lo;  // FP32+refine: the fluid mean of the iterate, float-float
     float rmean_hi, rmean_lo;  // FP32+refine: the fluid mean of the outer residual
+    double rmean;      // FP64 direct corrections: mean of the residual, 0 outside a solve
     double tol2_in;    // FP32+refine: squared relative tolerance of the inner solve in
                        // progress, when looser than the launch's (else 0)
 };

@@ -1,0 +1,85 @@
+// Driver of the host emulation of the direct solve (test support): builds the
+// plan and tables of a grid as the library does, runs the forward transforms,
+// the columns and the inverse transforms of two states (the second one
+// inactive), every CTA as host threads, and writes e.
+//
+// usage: direct_emu T nx ny nz bcx bcy bcz lx ly lz planes in.bin out.bin
+//   T: f or d; in.bin: r, two states; out.bin: e, two states (the inactive
+//   one's untouched zeros).
+
+#include <functional>
+
+static void launch(int gx, int bx, int by, size_t smem, const std::function<void()>& body) {
+    const int n = bx * by;
+    blockDim = EmuDim3{(unsigned)bx, (unsigned)by, 1};
+    for (int st = 0; st < 2; ++st)
+        for (int c = 0; c < gx; ++c) {
+            std::barrier<> bar(n);
+            emu_cta_barrier = &bar;
+            std::vector<unsigned char> sm(smem + 16, 0xff);  // NaN where nothing is written
+            const size_t mis = (16 - (size_t)sm.data() % 16) % 16;
+            emu_smem = sm.data() + mis;
+            std::vector<std::thread> th;
+            for (int t = 0; t < n; ++t)
+                th.emplace_back([&, t]() {
+                    threadIdx = EmuDim3{(unsigned)(t % bx), (unsigned)(t / bx), 0};
+                    blockIdx = EmuDim3{(unsigned)c, (unsigned)st, 0};
+                    body();
+                    bar.arrive_and_drop();
+                });
+            for (auto& x : th) x.join();
+        }
+}
+
+template <typename T>
+static int run(char** argv) {
+    int n[3], bc[3];
+    double ih2[3];
+    for (int a = 0; a < 3; ++a) {
+        n[a] = atoi(argv[2 + a]);
+        bc[a] = atoi(argv[5 + a]);
+        const double h = atof(argv[8 + a]) / n[a];
+        ih2[a] = 1.0 / (h * h);
+    }
+    DirPlan<T> P;
+    if (!dir_sizes<T>(n, bc[2] == BC_PERIODIC, atoi(argv[11]), P)) return 2;
+    size_t off[5];
+    std::vector<T> tab = dir_tables<T>(P, bc, ih2, off);
+    P.rx[0] = tab.data() + off[0];
+    P.rx[1] = tab.data() + off[1];
+    P.ly[0] = tab.data() + off[2];
+    P.ly[1] = tab.data() + off[3];
+    P.col = tab.data() + off[4];
+    const size_t N = (size_t)P.cells;
+    std::vector<T> r(2 * N), spec(2 * N, T(0)), e(2 * N, T(0));
+    FILE* f = fopen(argv[12], "rb");
+    if (!f || fread(r.data(), sizeof(T), 2 * N, f) != 2 * N) return 3;
+    fclose(f);
+    SliceCtl ctl[2] = {};
+    ctl[0].status = ST_ITER;
+    ctl[0].o_status = OS_REFINE;
+    ctl[1].status = ST_CONV;
+    ctl[1].o_status = OS_DONE;
+    const size_t smem = dir_smem_elems(P) * sizeof(T);
+    launch(P.nz * P.xb, P.nt, 1, smem,
+           [&] { k_dir_xy<T, false>(P, ctl, r.data(), spec.data()); });
+    const int zg = (P.nx * P.ny + DIR_ZX - 1) / DIR_ZX;
+    launch(zg, DIR_ZX, P.zc, 0, [&] {
+        if (P.zm == DIR_ZC)
+            k_dir_z<T, DIR_ZC>(P, ctl, spec.data());
+        else
+            k_dir_z<T, DIR_ZC_LONG>(P, ctl, spec.data());
+    });
+    launch(P.nz * P.xb, P.nt, 1, smem,
+           [&] { k_dir_xy<T, true>(P, ctl, spec.data(), e.data()); });
+    f = fopen(argv[13], "wb");
+    fwrite(e.data(), sizeof(T), 2 * N, f);
+    fclose(f);
+    printf("%d %d %d %d %d\n", P.xb, P.cb, P.nt, P.zm, P.zc);
+    return 0;
+}
+
+int main(int argc, char** argv) {
+    if (argc != 14) return 1;
+    return argv[1][0] == 'f' ? run<float>(argv) : run<double>(argv);
+}

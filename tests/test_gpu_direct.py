@@ -1,0 +1,89 @@
+"""Pressure corrections by the direct solve (boxes without solid cells)
+against the FP64 oracle, at the sizes where its kernels change: odd extents,
+extents below a tile, several column blocks and column chunks, every boundary
+type, grids the multigrid hierarchy cannot halve, and the graph path."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1705_06149_gb300 import Grid, NSError, StepGraph, inputs
+from paper_1705_06149_gb300 import _native as N
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+TOL = {"fp64": 1e-10, "fp32_refine": 1e-5}
+
+CASES = [((6, 3, 5), ("wall", "periodic", "wall")),
+         ((19, 13, 11), ("wall",) * 3),
+         ((45, 37, 21), ("wall", "slip", "wall")),
+         ((33, 10, 9), ("periodic", "periodic", "wall")),
+         ((12, 20, 40), ("wall", "wall", "periodic")),
+         ((10, 6, 150), ("wall",) * 3),
+         ((72, 100, 6), ("slip", "wall", "periodic"))]
+
+
+def rel(a, b):
+    n = np.linalg.norm(np.ravel(b))
+    return np.linalg.norm(np.ravel(a) - np.ravel(b)) / (n if n > 0 else 1.0)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_refine"])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_direct_steps_and_solves_match_the_oracle(case, prec):
+    dims, bc = CASES[case]
+    B = 2
+    box = [d / max(dims) for d in dims]  # cubic cells: cond(L) stays that of the extents
+    og = oracle.Grid(*dims, *box, re=100.0, bc=bc, rtol=1e-13)
+    g = Grid(*dims, *box, re=100.0, bc=bc, precision=prec, batch=B, poisson_rtol=1e-13)
+    inits = [inputs.random_state(*dims, seed=30 + s, sigma=0.2, bc=bc) for s in range(B)]
+    st = g.state_from([np.stack([i[c] for i in inits]) for c in range(4)])
+    g.profile(True)
+    g.step_fine(st, 2e-4, 3)
+    prof = g.profile_read()
+    g.profile(False)
+    assert prof["direct_xy"]["launches"] > 0 and prof["krylov_A"]["launches"] == 0
+    got = st.numpy()
+    for s in range(B):
+        want = oracle.copy_state(inits[s])
+        og.step(want, 2e-4, 3)
+        vg = np.concatenate([np.ravel(got[c][s]) for c in range(3)])
+        vw = np.concatenate([np.ravel(want[c]) for c in range(3)])
+        assert rel(vg, vw) <= TOL[prec], (s, rel(vg, vw))
+        assert rel(got[3][s], want[3]) <= TOL[prec], (s, rel(got[3][s], want[3]))
+    b = np.random.default_rng(case).normal(size=(B,) + og.shape(3))
+    bt = torch.tensor(b, device="cuda")
+    pt = torch.zeros_like(bt)
+    assert g.poisson_solve(bt, pt) >= 1
+    for s in range(B):
+        want, _ = og.poisson(b[s], rtol=1e-13)
+        # both sides stop at a relative residual (FP32+refine 1e-10), which the
+        # condition number of L (at most a few 1e4 here) turns into p's error
+        assert rel(pt[s].cpu().numpy(), want) <= (1e-9 if prec == "fp64" else 1e-6)
+    g.close()
+
+
+def test_a_grid_the_hierarchy_cannot_halve_still_refuses_graphs():
+    g = Grid(45, 37, 21, precision="fp32_refine")
+    with pytest.raises(NSError) as e:
+        StepGraph([(g, g.zeros(1), 1e-3, 1)])
+    assert e.value.status == N.NS_ERR_ARG
+    g.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_refine"])
+def test_direct_solve_off_gives_the_multigrid_result(prec, monkeypatch):
+    dims = (32, 24, 16)
+    init = inputs.random_state(*dims, seed=4, sigma=0.2)
+    out = []
+    for env in ("1", "0"):
+        monkeypatch.setenv("NS_DIRECT", env)
+        g = Grid(*dims, re=200.0, precision=prec, poisson_rtol=1e-13)
+        st = g.state_from(init)
+        g.profile(True)
+        g.step_fine(st, 1e-3, 3)
+        assert (g.profile_read()["direct_xy"]["launches"] > 0) == (env == "1")
+        out.append(st.numpy())
+        g.close()
+    for c in range(4):
+        assert rel(out[0][c], out[1][c]) <= TOL[prec]
