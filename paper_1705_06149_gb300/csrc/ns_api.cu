@@ -106,6 +106,10 @@ struct ns_grid {
     DirPlan<double> dird{};
     size_t dir_smem = 0;
     int dir_hint = 2;  // applications the last solves took
+    DirTile dir_tile{};                         // FP32+refine: tiling of the step kernels
+    float* dir_ring = nullptr;                  // FP32+refine: the last applications
+    double* dir_part = nullptr;                 // [cap][dir_tile.ctas][7]
+    float* dir_base[2] = {nullptr, nullptr};    // warm start of the solve in progress
     void* mg_vec[3] = {};                       // Y, Z, S at level 0
     void* mg_B[MG_MAX_LEVELS] = {};             // restricted right sides, levels 1..lc
     void* mg_Y[MG_MAX_LEVELS] = {};             // level iterates, levels 1..lc
@@ -471,6 +475,13 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
         return fail(NS_ERR_CUDA, "ns_create_grid: direct solve shared memory attribute");
     g->dir = true;
     g->mg = true;
+    if (sizeof(T) == 4) {
+        g->dir_tile = dir_tile_of(G.n, g->cap, g->d.tile_z);
+        NS_TRY(dalloc(g, (void**)&g->dir_ring,
+                      (size_t)G.cnt[3] * g->cap * DIR_RING * sizeof(float)));
+        NS_TRY(dalloc(g, (void**)&g->dir_part,
+                      (size_t)g->dir_tile.ctas * g->cap * 7 * sizeof(double)));
+    }
     return NS_OK;
 }
 
@@ -684,6 +695,9 @@ void launch_refine_init_ff(ns_grid* g, int batch, const double* p_in, double oto
     const Lev& L0 = g->plan.lev[0];
     const dim3 grid(L0.ctas, batch), blk = block_dim();
     MgBuf<float> mb = mgbuf<float>(g);
+    // the direct solve takes the residual's float-float form: its FP32 copies
+    // go to the buffer of the spectral planes, not yet in use
+    if (g->dir) mb.r = mb.rhat = (float*)g->kv[3];
     if (p_in)
         NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
                   k_mg_refine_init_ff<true><<<grid, blk, 0, g->stream>>>(
@@ -791,19 +805,24 @@ template <typename T> const DirPlan<T>& dirplan(const ns_grid* g);
 template <> const DirPlan<float>& dirplan<float>(const ns_grid* g) { return g->dirf; }
 template <> const DirPlan<double>& dirplan<double>(const ns_grid* g) { return g->dird; }
 
-// e = L^-1 r for every active state: the residual of the solve in kv[1], the
-// spectral planes in kv[3], e in kv[0] (FP32+refine) or kv[4] (FP64).
+long long dir_stride(const ns_grid* g) { return (long long)g->geo.cnt[3] * g->cap; }
+
+// e = L^-1 r for every active state: FP32+refine from the residual's high
+// part into the application's slot of the ring, FP64 from kv[1] into kv[4];
+// the spectral planes in kv[3].
 template <typename T>
 void direct_apply(ns_grid* g, int batch) {
     const DirPlan<T>& P = dirplan<T>(g);
-    const T* r = (const T*)g->kv[1];
+    const bool f32 = sizeof(T) == 4;
+    const T* r = f32 ? (const T*)g->ffb[2] : (const T*)g->kv[1];
     T* spec = (T*)g->kv[3];
-    T* e = (T*)g->kv[sizeof(T) == 4 ? 0 : 4];
+    T* e = f32 ? (T*)g->dir_ring : (T*)g->kv[4];
+    const long long ring = f32 ? dir_stride(g) : 0;
     const dim3 pg(P.nz * P.xb, batch), zg(ceil_div(P.nx * P.ny, DIR_ZX), batch);
     const dim3 zb(DIR_ZX, P.zc);
     const long long units = P.cells * batch;
     NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-              (k_dir_xy<T, false><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, r, spec)));
+              (k_dir_xy<T, false><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, r, spec, 0)));
     if (P.zm == DIR_ZC)
         NS_LAUNCH(g, NS_K_DIRECT_Z, units,
                   (k_dir_z<T, DIR_ZC><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
@@ -811,26 +830,25 @@ void direct_apply(ns_grid* g, int batch) {
         NS_LAUNCH(g, NS_K_DIRECT_Z, units,
                   (k_dir_z<T, DIR_ZC_LONG><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
     NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-              (k_dir_xy<T, true><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, spec, e)));
+              (k_dir_xy<T, true><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, spec, e, ring)));
 }
 
-// One application of the direct solve and the correction with it (p += e,
-// r -= L e, the decision), on every state still active.
+// One application of the direct solve and the correction with it, on every
+// state still active.
 void direct_correct(ns_grid* g, int batch) {
     const Lev& L0 = g->plan.lev[0];
-    const dim3 grid(L0.ctas, batch), blk = block_dim();
     const long long units = L0.cells * batch;
     if (g->fp32) {
         direct_apply<float>(g, batch);
         NS_LAUNCH(g, NS_K_REFINE, units,
-                  k_mg_refine_update_ff<<<grid, blk, 0, g->stream>>>(
-                      L0, mgbuf<float>(g), g->ctl, ffbuf(g), g->geo.n_fluid, g->part_mg,
-                      g->d.refine_rtol * g->d.refine_rtol, g->inner_rtol * g->inner_rtol,
-                      g->maxit, g->max_outer, 0));
+                  k_dir_refine<<<dim3(g->dir_tile.ctas, batch), block_dim(), 0, g->stream>>>(
+                      L0, g->dir_tile, g->ctl, g->dir_ring, dir_stride(g), g->dir_base[0],
+                      g->dir_base[1], ffbuf(g), g->dir_part, g->counter,
+                      g->d.refine_rtol * g->d.refine_rtol, g->max_outer));
     } else {
         direct_apply<double>(g, batch);
         NS_LAUNCH(g, NS_K_REFINE, units,
-                  k_dir_update<<<grid, blk, 0, g->stream>>>(
+                  k_dir_update<<<dim3(L0.ctas, batch), block_dim(), 0, g->stream>>>(
                       L0, mgbuf<double>(g), g->ctl, (const double*)g->kv[4], g->part_mg,
                       g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid));
     }
@@ -1229,10 +1247,7 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
         NS_TRY(make_handle(g->stream, &h));
         NS_TRY(loop_cond(g, batch, h, LC_FP64_START, cap_inner));
         return add_while(g, g->body_stream[0], h, [&]() -> ns_status {
-            if (g->dir)
-                direct_correct(g, batch);
-            else
-                NS_TRY(mg_iteration<double>(g, batch, tol2, 0));
+            NS_TRY(mg_iteration<double>(g, batch, tol2, 0));
             return loop_cond(g, batch, h, LC_FP64_ITER, cap_inner);
         });
     }
@@ -1248,10 +1263,6 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
     NS_TRY(make_handle(g->stream, &h));
     NS_TRY(loop_cond(g, batch, h, LC_REFINE_START, cap_refine));
     return add_while(g, g->body_stream[0], h, [&]() -> ns_status {
-        if (g->dir) {
-            direct_correct(g, batch);
-            return loop_cond(g, batch, h, LC_REFINE_ITER, cap_refine);
-        }
         NS_TRY(mg_iteration<float>(g, batch, itol2, 1));
         NS_LAUNCH(g, NS_K_REFINE, 0,
                   k_mg_refine_update_ff<<<grid, blk, 0, g->stream>>>(
@@ -1262,21 +1273,21 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
     });
 }
 
-// The solve by direct corrections on the stream path: as many as the last
-// solves took are issued back to back, then the flags are polled after each.
-ns_status solve_pressure_direct(ns_grid* g, int batch, const double* p_in) {
-    const Lev& L0 = g->plan.lev[0];
-    const dim3 grid(L0.ctas, batch), blk = block_dim();
-    if (g->fp32)
-        launch_refine_init_ff(g, batch, p_in, g->d.refine_rtol * g->d.refine_rtol,
-                              g->inner_rtol * g->inner_rtol);
-    else
-        NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
-                  k_mg_init_warm<double><<<grid, blk, 0, g->stream>>>(
-                      L0, mgbuf<double>(g), g->ctl, g->part_div, g->geo.n_fluid, g->b,
-                      p_in ? p_in : g->p_prev, g->part_mg,
-                      g->d.poisson_rtol * g->d.poisson_rtol, g->maxit));
+// The corrections of a started solve.  On the stream path as many as the last
+// solves took are issued back to back, then the flags are polled after each;
+// captured, they are a while loop on the device.
+ns_status direct_loop(ns_grid* g, int batch) {
     NS_CUDA(cudaGetLastError());
+    if (g->capturing) {
+        const int cap = (g->fp32 ? g->max_outer : g->maxit) + 2;
+        cudaGraphConditionalHandle h;
+        NS_TRY(make_handle(g->stream, &h));
+        NS_TRY(loop_cond(g, batch, h, g->fp32 ? LC_REFINE_START : LC_FP64_START, cap));
+        return add_while(g, g->body_stream[0], h, [&]() -> ns_status {
+            direct_correct(g, batch);
+            return loop_cond(g, batch, h, g->fp32 ? LC_REFINE_ITER : LC_FP64_ITER, cap);
+        });
+    }
     const int limit = (g->fp32 ? g->max_outer : g->maxit) + 2;
     for (int it = 1; it <= limit; ++it) {
         direct_correct(g, batch);
@@ -1317,9 +1328,96 @@ ns_status solve_pressure_direct(ns_grid* g, int batch, const double* p_in) {
     return NS_OK;
 }
 
+// A gauged solve as solve_pressure describes it, by direct corrections.
+ns_status solve_pressure_direct(ns_grid* g, int batch, const double* p_in) {
+    const Lev& L0 = g->plan.lev[0];
+    if (g->fp32) {
+        launch_refine_init_ff(g, batch, p_in, g->d.refine_rtol * g->d.refine_rtol,
+                              g->inner_rtol * g->inner_rtol);
+        g->dir_base[0] = g->ffb[0];
+        g->dir_base[1] = g->ffb[1];
+    } else {
+        NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
+                  k_mg_init_warm<double><<<dim3(L0.ctas, batch), block_dim(), 0, g->stream>>>(
+                      L0, mgbuf<double>(g), g->ctl, g->part_div, g->geo.n_fluid, g->b,
+                      p_in ? p_in : g->p_prev, g->part_mg,
+                      g->d.poisson_rtol * g->d.poisson_rtol, g->maxit));
+    }
+    return direct_loop(g, batch);
+}
+
+// The velocity correction after a solve by direct corrections (FP32+refine):
+// u, v, w from F* or the increments fs, p (may be null); with w_next the next
+// warm start goes there.
+template <bool INCR>
+void direct_velocity(ns_grid* g, int batch, float* const fs[3], float* const vel[3], double* p,
+                     double dt, float* const w_next[2]) {
+    const Geo& G = g->geo;
+    NS_LAUNCH(g, NS_K_CORRECT, G.cnt[3] * batch,
+              k_dir_correct<INCR><<<dim3(g->dir_tile.ctas, batch), block_dim(), 0, g->stream>>>(
+                  g->plan.lev[0], g->dir_tile, g->ctl, fs[0], fs[1], fs[2], vel[0], vel[1],
+                  vel[2], ffbuf(g), g->dir_base[0], g->dir_base[1], g->dir_ring, dir_stride(g),
+                  w_next ? w_next[0] : nullptr, w_next ? w_next[1] : nullptr, p, dt_ih(G, dt),
+                  G.cnt[0], G.cnt[1], G.cnt[2]));
+}
+
+// The caller's FP64 pressure as warm start (ffb[4..5]) and last pressure.
+void direct_load_p(ns_grid* g, int batch, const double* p) {
+    const long long cells = g->geo.cnt[3] * batch;
+    NS_LAUNCH(g, NS_K_INNER_INIT, cells,
+              k_dir_load_p<<<(unsigned)((cells + NTHREADS - 1) / NTHREADS), block_dim(), 0,
+                             g->stream>>>(cells, p, ffbuf(g)));
+}
+
+// Start of an FP32+refine solve: b = D fs / dt (with vel: D (vel + fs) / dt),
+// r = b - L warm.
+void direct_start(ns_grid* g, int batch, float* const fs[3], float* const vel[3],
+                  float* const warm[2], double dt) {
+    const Geo& G = g->geo;
+    auto ff = [](double d) { return FF{(float)d, (float)(d - (double)(float)d)}; };
+    const FF idt = ff(1.0 / dt), ihx = ff(G.ih[0]), ihy = ff(G.ih[1]), ihz = ff(G.ih[2]);
+    const double otol2 = g->d.refine_rtol * g->d.refine_rtol;
+    const dim3 grid(g->dir_tile.ctas, batch), blk = block_dim();
+    if (vel)
+        NS_LAUNCH(g, NS_K_SOLVE_INIT, G.cnt[3] * batch,
+                  k_dir_start<true><<<grid, blk, 0, g->stream>>>(
+                      g->plan.lev[0], g->dir_tile, g->ctl, fs[0], fs[1], fs[2], vel[0], vel[1],
+                      vel[2], warm[0], warm[1], ffbuf(g), idt, ihx, ihy, ihz, G.cnt[0], G.cnt[1],
+                      G.cnt[2], g->dir_part, g->counter, otol2, g->max_outer));
+    else
+        NS_LAUNCH(g, NS_K_SOLVE_INIT, G.cnt[3] * batch,
+                  k_dir_start<false><<<grid, blk, 0, g->stream>>>(
+                      g->plan.lev[0], g->dir_tile, g->ctl, fs[0], fs[1], fs[2], nullptr, nullptr,
+                      nullptr, warm[0], warm[1], ffbuf(g), idt, ihx, ihy, ihz, G.cnt[0], G.cnt[1],
+                      G.cnt[2], g->dir_part, g->counter, otol2, g->max_outer));
+    g->dir_base[0] = warm[0];
+    g->dir_base[1] = warm[1];
+}
+
+// One FP32+refine step by direct corrections, n-th of a call of nsteps: the
+// warm start alternates between the buffers ffb[4..5] (even n) and ffb[0..1].
+// The FP64 pressure is written by the call's last step only.
+ns_status direct_step(ns_grid* g, const ns_state& io, double dt, int n, int nsteps) {
+    const int B = io.batch;
+    float* vel[3] = {(float*)io.u, (float*)io.v, (float*)io.w};
+    float* fs[3] = {(float*)g->fs[0], (float*)g->fs[1], (float*)g->fs[2]};
+    float* even[2] = {g->ffb[4], g->ffb[5]};
+    float* odd[2] = {g->ffb[0], g->ffb[1]};
+    float** cur = n % 2 ? odd : even;
+    float** next = n % 2 ? even : odd;
+    if (n == 0) direct_load_p(g, B, (const double*)io.p);
+    direct_start(g, B, fs, n == 0 ? vel : nullptr, cur, dt);
+    NS_TRY(direct_loop(g, B));
+    const bool last = n + 1 == nsteps;
+    direct_velocity<true>(g, B, fs, vel, last ? (double*)io.p : nullptr, dt,
+                          last ? nullptr : next);
+    NS_CUDA(cudaGetLastError());
+    return NS_OK;
+}
+
 ns_status solve_pressure_mg(ns_grid* g, int batch, const double* p_in) {
-    if (g->capturing) return solve_pressure_mg_graph(g, batch, p_in);
     if (g->dir) return solve_pressure_direct(g, batch, p_in);
+    if (g->capturing) return solve_pressure_mg_graph(g, batch, p_in);
     if (g->persist && batch <= g->persist_max_batch) return solve_pressure_persist(g, batch, p_in);
     const Lev& L0 = g->plan.lev[0];
     const dim3 grid(L0.ctas, batch), blk = block_dim();
@@ -1537,6 +1635,11 @@ ns_status step_impl(ns_grid* g, const ns_state& io, double dt, int nsteps) {
     const long long cells = G.cnt[3] * B;
     for (int n = 0; n < nsteps; ++n) {
         NS_LAUNCH(g, NS_K_PREDICT, cells, launch_predict<T, INCR>(g, B, u, v, w, fu, fv, fw, dt));
+        if (INCR && g->dir) {
+            NS_TRY(direct_step(g, io, dt, n, nsteps));
+            if (!g->capturing) g->stats.steps += B;
+            continue;
+        }
         const bool with_u = INCR && n == 0;
         NS_LAUNCH(g, NS_K_DIVERGENCE, cells,
                   k_divergence<T><<<gcell, block_dim(), 0, g->stream>>>(
@@ -1588,6 +1691,20 @@ ns_status project_impl(ns_grid* g, const ns_state& io, double* phi = nullptr) {
     T* v = (T*)io.v;
     T* w = (T*)io.w;
     g->prof.active = B >= g->prof.min_batch;
+    if (g->fp32 && g->dir) {
+        float* vel[3] = {(float*)io.u, (float*)io.v, (float*)io.w};
+        float* warm[2] = {g->ffb[4], g->ffb[5]};
+        if (phi)
+            direct_load_p(g, B, phi);
+        else
+            for (float* q : warm)
+                NS_CUDA(cudaMemsetAsync(q, 0, sizeof(float) * G.cnt[3] * B, g->stream));
+        direct_start(g, B, vel, nullptr, warm, 1.0);
+        NS_TRY(direct_loop(g, B));
+        direct_velocity<false>(g, B, vel, vel, phi, 1.0, nullptr);
+        NS_CUDA(cudaGetLastError());
+        return NS_OK;
+    }
     NS_LAUNCH(g, NS_K_DIVERGENCE, G.cnt[3] * B,
               k_divergence<T><<<gcell, block_dim(), 0, g->stream>>>(
                   G, u, v, w, nullptr, nullptr, nullptr, g->b, g->part_div, 1.0));
@@ -1673,7 +1790,7 @@ ns_status account_graph(ns_grid* g, int B, long long state_steps, long long step
     g->stats.steps += state_steps;
     // per step: predict, divergence, solve start, loop condition, correction;
     // per loop body: one iteration, (FP32) the outer correction, the condition
-    g->stats.launches += step_groups * 5 +
+    g->stats.launches += step_groups * (g->dir && g->fp32 ? 4 : 5) +
                          bodies * (mg_iteration_launches(g) + (g->fp32 ? 2 : 1)) +
                          extra_launches;
     ns_status result = NS_OK;
@@ -2551,7 +2668,6 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
     };
     for (int c = 0; c < 3; ++c) A(&g->fs[c], (size_t)G.cnt[c] * ev * B);
     A((void**)&g->b, ncell * sizeof(double) * B);
-    for (int q = 0; q < 8; ++q) A(&g->kv[q], ncell * ev * B);
     A((void**)&g->p64[0], ncell * sizeof(double) * B);
     A((void**)&g->p64[1], ncell * sizeof(double) * B);
     const size_t nparts = (size_t)G.ctas * B;
@@ -2591,6 +2707,10 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             g->plan.lev[0].fcode = (const uint8_t*)fc;
         }
     }
+    // the direct solve needs the spectral planes (kv[3]), in FP64 also x, r,
+    // the start's copy of r and e; BiCGStab all eight vectors
+    for (int q = 0; q < 8; ++q)
+        if (!g->dir || q == 3 || (!g->fp32 && q < 5)) A(&g->kv[q], ncell * ev * B);
     if (g->mg) {
         for (int q = 0; q < 3 && !g->dir; ++q) A(&g->mg_vec[q], ncell * ev * B);
         for (int l = 1; l <= g->plan.lc && !g->dir; ++l) {
@@ -2664,7 +2784,7 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             if (cudaMemsetAsync(g->fs[c], 0, (size_t)G.cnt[c] * ev * B, g->stream) != cudaSuccess)
                 st = fail(NS_ERR_CUDA, "ns_create_grid: memset failed");
         for (int q = 0; q < 8 && st == NS_OK; ++q)
-            if (cudaMemsetAsync(g->kv[q], 0, ncell * ev * B, g->stream) != cudaSuccess)
+            if (g->kv[q] && cudaMemsetAsync(g->kv[q], 0, ncell * ev * B, g->stream) != cudaSuccess)
                 st = fail(NS_ERR_CUDA, "ns_create_grid: memset failed");
         if (st == NS_OK &&
             cudaMemsetAsync(g->ctl, 0, sizeof(SliceCtl) * B, g->stream) != cudaSuccess)
@@ -2797,7 +2917,10 @@ ns_status ns_poisson_solve(ns_grid* grid, const double* b, double* p, int batch,
     // the face part pointed at the (unused) F* buffers
     const double* x0 = grid->fp32 ? grid->p64[0] : (const double*)grid->kv[0];
     const double* x1 = grid->fp32 ? grid->p64[1] : (const double*)grid->kv[0];
-    if (grid->fp32 && grid->mg)
+    if (grid->fp32 && grid->dir) {
+        float* fs[3] = {(float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2]};
+        direct_velocity<false>(grid, batch, fs, fs, p, 0.0, nullptr);
+    } else if (grid->fp32 && grid->mg)
         NS_LAUNCH(grid, NS_K_CORRECT, G.cnt[3] * batch,
                   k_correct_ff<false><<<gface, block_dim(), 0, grid->stream>>>(
                       G, grid->ctl, (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2],

@@ -67,6 +67,25 @@ template <> __device__ __forceinline__ bool dir_active<double>(const SliceCtl* c
     return c->status == ST_ITER;
 }
 
+// FP32 corrections live in a ring of DIR_RING buffers, one per application;
+// the pressure is the warm start plus the applications not yet folded into it
+// (the last three at most).  The residual is scaled by a power of two on its
+// way into the transforms and e unscaled on its way out, so that neither
+// underflows however far the refinement has come.
+constexpr int DIR_RING = 4;
+template <typename T> __device__ __forceinline__ T dir_scale(const SliceCtl* c, bool inv);
+template <> __device__ __forceinline__ float dir_scale<float>(const SliceCtl* c, bool inv) {
+    return inv ? 1.0f / c->o_fsc : c->o_fsc;
+}
+template <> __device__ __forceinline__ double dir_scale<double>(const SliceCtl*, bool) {
+    return 1.0;
+}
+template <typename T> __device__ __forceinline__ int dir_slot(const SliceCtl* c);
+template <> __device__ __forceinline__ int dir_slot<float>(const SliceCtl* c) {
+    return c->o_steps & (DIR_RING - 1);
+}
+template <> __device__ __forceinline__ int dir_slot<double>(const SliceCtl*) { return 0; }
+
 // acc[i][j] += sum_k L[i rs][k] R[k][j], i, j < 4, k ascending (K a multiple
 // of 4; rows of L are rs apart so that neighbouring threads read
 // neighbouring rows).
@@ -97,15 +116,17 @@ inline size_t dir_smem_elems(const DirPlan<T>& P) {
 }
 
 // Forward (INV false): src [nz][ny][nx] cells -> dst [nz][ky][kx].  Inverse:
-// src [nz][ky][kx] -> dst cells.  blockIdx.x = plane and column block,
+// src [nz][ky][kx] -> dst cells (FP32: the application's slot of the ring,
+// slots `ring` elements apart).  blockIdx.x = plane and column block,
 // blockIdx.y = state.
 template <typename T, bool INV>
 __global__ void __launch_bounds__(DIR_MAX_THREADS)
     k_dir_xy(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const T* __restrict__ src,
-             T* __restrict__ dst) {
+             T* __restrict__ dst, long long ring) {
     pdl_wait();
     const long long s = blockIdx.y;
     if (!dir_active<T>(ctl + s)) return;
+    const T scale = dir_scale<T>(ctl + s, INV);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, ny = P.ny, hx = P.hx, hy = P.hy, hxp = P.hxp, hyp = P.hyp;
     const int ldx = P.ldx, ldy = P.ldy, cb = P.cb;
@@ -117,7 +138,8 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const int c0 = ((int)blockIdx.x - z * P.xb) * cb;
     const int t = (int)threadIdx.x, nt = (int)blockDim.x;
     const T* __restrict__ a = src + s * P.cells + (long long)z * nx * ny;
-    T* __restrict__ o = dst + s * P.cells + (long long)z * nx * ny;
+    T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s) * ring : 0) + s * P.cells +
+                        (long long)z * nx * ny;
     {
         // the plane: thread (row, column j) of a pass; rows and columns beyond
         // the halves are zero
@@ -150,7 +172,8 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
                     if (yo && xo) q[3] = a[(hy + y) * nx + hx + j];
                 }
 #pragma unroll
-                for (int h = 0; h < 4; ++h) F[(h * hyp + y) * ldx + j] = q[h];
+                for (int h = 0; h < 4; ++h)
+                    F[(h * hyp + y) * ldx + j] = INV ? q[h] : q[h] * scale;
             }
         }
         // the matrices
@@ -221,8 +244,9 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
             const int x = c0 + j, xm = nx - 1 - x;
             for (int y = y0; y < hy; y += rpp) {
                 const int ym = ny - 1 - y;
-                const T ee = F[y * cb + j], eo = F[(hyp + y) * cb + j];
-                const T oe = F[(2 * hyp + y) * cb + j], oo = F[(3 * hyp + y) * cb + j];
+                const T ee = scale * F[y * cb + j], eo = scale * F[(hyp + y) * cb + j];
+                const T oe = scale * F[(2 * hyp + y) * cb + j];
+                const T oo = scale * F[(3 * hyp + y) * cb + j];
                 const T pe = ee + oe, po = eo + oo, me = ee - oe, mo = eo - oo;
                 o[y * nx + x] = pe + po;
                 if (xm != x) o[y * nx + xm] = pe - po;
@@ -283,6 +307,15 @@ __global__ void __launch_bounds__(dir_z_threads<T>(ZM))
     // mode has c1 = 0: the sums of a mean-free column start from 0)
     const T first = P.per_z ? c1 * Y : c1 * fma(rn, Y, Lt);
     T prev = fma(below, first, carry);
+    if (q == 0) {
+        // the constant (kx, ky) mode: the column's mean is out of L's range;
+        // without it the sums end at zero
+        const T mean = Y / T(nz);
+        prev -= mean * T(k0);
+#pragma unroll
+        for (int i = 0; i < ZM; ++i)
+            if (i < len) f[i] -= mean;
+    }
 #pragma unroll
     for (int i = 0; i < ZM; ++i)
         if (i < len) {
@@ -331,6 +364,390 @@ __global__ void __launch_bounds__(dir_z_threads<T>(ZM))
     }
 }
 
+// ---------------------------------------------------------------------------
+// the FP32+refine step around the direct solve (boxes without solid cells):
+// start of the solve, outer correction, velocity correction.  Everything per
+// cell runs in FP32 and float-float: GB300's FP64 pipe is 1/64 of its FP32
+// one, and a handful of conversions and FP64 sums per cell made each of these
+// passes FP64-bound.
+// ---------------------------------------------------------------------------
+
+// Tiling: a CTA of 128 threads covers w x r columns (w the width of the x
+// tiles, r = 128 / w rows) and lz cells along z, in batches of DIR_ZB whose
+// loads are issued together.
+struct DirTile {
+    int w, r, bx, by, lz, ctas;
+};
+constexpr int DIR_ZB = 4;
+
+__device__ __forceinline__ bool dir_origin(const DirTile& t, const int* n, int& i, int& j,
+                                           int& k0) {
+    const int cta = (int)blockIdx.x;
+    const int q = cta / t.bx, tx = cta - q * t.bx;
+    const int tz = q / t.by, ty = q - tz * t.by;
+    const int th = tid_flat(), y = th / t.w, x = th - y * t.w;
+    i = tx * t.w + x;
+    j = ty * t.r + y;
+    k0 = tz * t.lz;
+    return y < t.r && i < n[0] && j < n[1];
+}
+
+// DIR_ZB cells of a column with their neighbours: c[1 + q] cell q, c[0] the
+// one below the first, c[DIR_ZB + 1] the one above the last (cells beyond the
+// tile repeat its last neighbour and are not used).
+struct DirSlab {
+    float c[DIR_ZB + 2], xl[DIR_ZB], xh[DIR_ZB], yl[DIR_ZB], yh[DIR_ZB];
+};
+
+__device__ __forceinline__ int dir_zwrap(const Lev& L, int k) {
+    if (k < 0) return L.bc[2] == BC_PERIODIC ? L.n[2] - 1 : 0;
+    if (k >= L.n[2]) return L.bc[2] == BC_PERIODIC ? 0 : L.n[2] - 1;
+    return k;
+}
+
+__device__ __forceinline__ void dir_load(const Lev& L, const NbrXY& xy, int kb, int k1,
+                                         const float* __restrict__ a, DirSlab& v) {
+    const int plane = L.n[0] * L.n[1];
+#pragma unroll
+    for (int q = 0; q < DIR_ZB + 2; ++q)
+        v.c[q] = a[dir_zwrap(L, min(kb + q - 1, k1)) * plane + xy.base];
+#pragma unroll
+    for (int q = 0; q < DIR_ZB; ++q) {
+        const float* __restrict__ p = a + min(kb + q, k1 - 1) * plane + xy.base;
+        v.xl[q] = p[xy.xl];
+        v.xh[q] = p[xy.xh];
+        v.yl[q] = p[xy.yl];
+        v.yh[q] = p[xy.yh];
+    }
+}
+
+__device__ __forceinline__ FF dir_lap_ff(const Lev& L, const DirSlab& v, int q) {
+    const float eh[3] = {v.xh[q], v.yh[q], v.c[q + 2]};
+    const float el[3] = {v.xl[q], v.yl[q], v.c[q]};
+    return lap_ff6(L, eh, el, v.c[q + 1]);
+}
+
+// a b with a float, b float-float; both float-float.
+__device__ __forceinline__ FF ff_mul_f(float a, FF b) {
+    const float p = a * b.hi;
+    return ff_norm(p, fmaf(a, b.hi, -p) + a * b.lo);
+}
+__device__ __forceinline__ FF ff_mul(FF a, FF b) {
+    const float p = a.hi * b.hi;
+    return ff_norm(p, fmaf(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi));
+}
+
+// The last CTA of the start or of an outer correction: target met, out of
+// corrections, or on.
+__device__ __forceinline__ void dir_decide(SliceCtl* c, double rr, double otol2, long long cells,
+                                           int max_outer) {
+    c->o_rr = rr;
+    c->p_final = 0;
+    c->o_fsc = float(pow2_scale(rr, cells));
+    c->status = ST_IDLE;
+    if (!isfinite(rr)) {
+        c->o_status = OS_NONFINITE;
+    } else if (rr <= otol2 * c->o_bb) {
+        c->o_status = OS_DONE;
+    } else if (c->o_steps >= max_outer) {
+        c->o_status = OS_FAIL;
+    } else {
+        c->o_status = OS_REFINE;
+        c->status = ST_ITER;
+    }
+}
+
+// The pressure of the caller (FP64) as warm start and as last pressure.
+__global__ void __launch_bounds__(NTHREADS)
+    k_dir_load_p(long long n, const double* __restrict__ p, FFBuf f) {
+    pdl_wait();
+    const long long q = (long long)blockIdx.x * NTHREADS + tid_flat();
+    if (q >= n) return;
+    const FF v = ff_from_double(p[q]);
+    f.w_hi[q] = v.hi;
+    f.w_lo[q] = v.lo;
+    f.q_hi[q] = v.hi;
+    f.q_lo[q] = v.lo;
+}
+
+// Start of a step's solve: b = D F* / dt (WITH_U: of u + increment, the
+// stored u differenced exactly), r = b - L w.  The mean of r (rounding, the
+// fluxes of b cancel) is left in r and taken out by the next residual.
+template <bool WITH_U>
+__global__ void __launch_bounds__(NTHREADS)
+    k_dir_start(Lev L, DirTile t, SliceCtl* __restrict__ ctl, const float* __restrict__ fu,
+                const float* __restrict__ fv, const float* __restrict__ fw,
+                const float* __restrict__ u, const float* __restrict__ v,
+                const float* __restrict__ w, const float* __restrict__ w_hi,
+                const float* __restrict__ w_lo, FFBuf f, FF inv_dt, FF ihx, FF ihy, FF ihz,
+                long long cu, long long cv, long long cw, double* __restrict__ part,
+                unsigned int* __restrict__ counter, double otol2, int max_outer) {
+    pdl_wait();
+    const long long s = blockIdx.y;
+    SliceCtl* c = ctl + s;
+    const long long off = s * L.cells;
+    const int ex = L.n[0] + (L.bc[0] != BC_PERIODIC), ey = L.n[1] + (L.bc[1] != BC_PERIODIC);
+    int i, j, k0;
+    SqAcc arr, abb;
+    float sb = 0.0f;
+    FF sr{0.0f, 0.0f}, sw{0.0f, 0.0f};
+    if (dir_origin(t, L.n, i, j, k0)) {
+        const int k1 = min(k0 + t.lz, L.n[2]);
+        const NbrXY xy = make_nbr_xy(L, i, j);
+        const int plane = L.n[0] * L.n[1];
+        const int ip = i + 1 == ex ? 0 : i + 1, jp = j + 1 == ey ? 0 : j + 1;
+        // faces of the cell: u at (i, ip), v at (j, jp), w at (k, k + 1)
+        const long long u0 = (long long)j * ex, v0 = (long long)j * L.n[0] + i,
+                        v1 = (long long)jp * L.n[0] + i;
+        const long long pu = (long long)L.n[1] * ex, pv = (long long)ey * L.n[0];
+        const int ez = L.n[2] + (L.bc[2] != BC_PERIODIC);
+        auto div3 = [&](const float* __restrict__ a, const float* __restrict__ b,
+                        const float* __restrict__ d, int k, float (&q)[6]) {
+            const int kp = k + 1 == ez ? 0 : k + 1;
+            q[0] = a[s * cu + k * pu + u0 + ip];
+            q[1] = a[s * cu + k * pu + u0 + i];
+            q[2] = b[s * cv + k * pv + v1];
+            q[3] = b[s * cv + k * pv + v0];
+            q[4] = d[s * cw + (long long)kp * plane + xy.base];
+            q[5] = d[s * cw + (long long)k * plane + xy.base];
+        };
+        for (int kb = k0; kb < k1; kb += DIR_ZB) {
+            DirSlab wh, wl;
+            float fa[DIR_ZB][6];
+            dir_load(L, xy, kb, k1, w_hi + off, wh);
+            dir_load(L, xy, kb, k1, w_lo + off, wl);
+#pragma unroll
+            for (int q = 0; q < DIR_ZB; ++q) div3(fu, fv, fw, min(kb + q, k1 - 1), fa[q]);
+#pragma unroll
+            for (int q = 0; q < DIR_ZB; ++q) {
+                if (kb + q >= k1) break;
+                // the increment's divergence in FP32 (its differences carry no
+                // cancellation against u)
+                float dv = (fa[q][0] - fa[q][1]) * ihx.hi;
+                dv += (fa[q][2] - fa[q][3]) * ihy.hi;
+                dv += (fa[q][4] - fa[q][5]) * ihz.hi;
+                FF b;
+                if (WITH_U) {
+                    float ua[6];
+                    div3(u, v, w, kb + q, ua);
+                    FF d{dv, 0.0f};
+                    const FF ih[3] = {ihx, ihy, ihz};
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        FF g;
+                        two_sum(ua[2 * a], -ua[2 * a + 1], g.hi, g.lo);
+                        d = ff_add(d, ff_mul(g, ih[a]));
+                    }
+                    b = ff_mul(d, inv_dt);
+                } else {
+                    b = ff_mul_f(dv, inv_dt);
+                }
+                const float ll = lap7<float>(L, wl.xh[q], wl.xl[q], wl.yh[q], wl.yl[q],
+                                             wl.c[q + 2], wl.c[q], wl.c[q + 1]);
+                const FF lp = ff_add_f(dir_lap_ff(L, wh, q), ll);
+                const FF r = ff_add(b, ff_neg(lp));
+                const long long id = off + (long long)(kb + q) * plane + xy.base;
+                f.r_hi[id] = r.hi;
+                f.r_lo[id] = r.lo;
+                arr.add(r.hi);
+                abb.add(b.hi);
+                sb += b.hi;
+                sr = ff_add(sr, r);
+                sw = ff_add(sw, FF{wh.c[q + 1], wl.c[q + 1]});
+            }
+        }
+    }
+    float acc[5] = {arr.big, arr.small, abb.big, abb.small, sb};
+    const FF ffs[2] = {sr, sw};
+    double tot[7];
+    if (partials_arrive_ff<5, 2>(acc, ffs, part + s * t.ctas * 7, counter + s, t.ctas, tot) &&
+        tid_flat() == 0) {
+        const double n = (double)L.cells;
+        const double rr = tot[0] + tot[1] * 0x1p-128, bb = tot[2] + tot[3] * 0x1p-128;
+        const FF rm = ff_from_double(tot[5] / n);
+        c->rmean_hi = rm.hi;
+        c->rmean_lo = rm.lo;
+        c->sx = tot[6];
+        const FF mean = ff_from_double(tot[6] / n);
+        c->mean_hi = mean.hi;
+        c->mean_lo = mean.lo;
+        c->o_steps = 0;
+        c->o_bb = fmax(bb - tot[4] * tot[4] / n, 0.0);
+        // a NaN stays one
+        const double r0 = rr - tot[5] * tot[5] / n;
+        dir_decide(c, r0 < 0.0 ? 0.0 : r0, otol2, L.cells, max_outer);
+    }
+}
+
+// Outer correction with the application e just made: r <- r - mean(r) - L e
+// (L e in float-float), its norm, the decision.  p is not touched: the warm
+// start `base` and the last applications together are the pressure (from the
+// fourth application on the oldest one still apart is folded into base).
+__global__ void __launch_bounds__(NTHREADS)
+    k_dir_refine(Lev L, DirTile t, SliceCtl* __restrict__ ctl, const float* __restrict__ ring,
+                 long long stride, float* __restrict__ base_hi, float* __restrict__ base_lo,
+                 FFBuf f, double* __restrict__ part, unsigned int* __restrict__ counter,
+                 double otol2, int max_outer) {
+    pdl_wait();
+    const long long s = blockIdx.y;
+    SliceCtl* c = ctl + s;
+    if (!dir_active<float>(c)) return;
+    const long long off = s * L.cells;
+    const int step = c->o_steps;
+    const float* __restrict__ e = ring + (step & (DIR_RING - 1)) * stride + off;
+    const float* __restrict__ old = ring + ((step + 1) & (DIR_RING - 1)) * stride + off;
+    const FF neg_rmean{-c->rmean_hi, -c->rmean_lo};
+    int i, j, k0;
+    SqAcc arr;
+    FF sr{0.0f, 0.0f}, se{0.0f, 0.0f};
+    if (dir_origin(t, L.n, i, j, k0)) {
+        const int k1 = min(k0 + t.lz, L.n[2]);
+        const NbrXY xy = make_nbr_xy(L, i, j);
+        const int plane = L.n[0] * L.n[1];
+        for (int kb = k0; kb < k1; kb += DIR_ZB) {
+            DirSlab ev;
+            FF ro[DIR_ZB];
+            dir_load(L, xy, kb, k1, e, ev);
+#pragma unroll
+            for (int q = 0; q < DIR_ZB; ++q) {
+                const long long id = off + (long long)min(kb + q, k1 - 1) * plane + xy.base;
+                ro[q] = FF{f.r_hi[id], f.r_lo[id]};
+            }
+#pragma unroll
+            for (int q = 0; q < DIR_ZB; ++q) {
+                if (kb + q >= k1) break;
+                const long long id = off + (long long)(kb + q) * plane + xy.base;
+                const FF le = dir_lap_ff(L, ev, q);
+                const FF r = ff_add(ff_add(ro[q], neg_rmean), ff_neg(le));
+                f.r_hi[id] = r.hi;
+                f.r_lo[id] = r.lo;
+                arr.add(r.hi);
+                sr = ff_add(sr, r);
+                se = ff_add_f(se, ev.c[q + 1]);
+                if (step >= DIR_RING - 1) {
+                    const FF b = ff_add_f(FF{base_hi[id], base_lo[id]}, old[id - off]);
+                    base_hi[id] = b.hi;
+                    base_lo[id] = b.lo;
+                }
+            }
+        }
+    }
+    float acc[2] = {arr.big, arr.small};
+    const FF ffs[2] = {sr, se};
+    double tot[4];
+    if (partials_arrive_ff<2, 2>(acc, ffs, part + s * t.ctas * 4, counter + s, t.ctas, tot) &&
+        tid_flat() == 0) {
+        const double n = (double)L.cells;
+        const FF rm = ff_from_double(tot[2] / n);
+        c->rmean_hi = rm.hi;
+        c->rmean_lo = rm.lo;
+        c->sx += tot[3];
+        const FF mean = ff_from_double(c->sx / n);
+        c->mean_hi = mean.hi;
+        c->mean_lo = mean.lo;
+        c->o_steps = step + 1;
+        const double r0 = tot[0] + tot[1] * 0x1p-128 - tot[2] * tot[2] / n;
+        dir_decide(c, r0 < 0.0 ? 0.0 : r0, otol2, L.cells, max_outer);
+    }
+}
+
+// Velocity correction u = u + (increment - dt G p) (INCR) or F* - dt G p, p =
+// base + the applications still apart; p_out (may be null) = p - mean in FP64;
+// with w_hi given the next warm start w = 2 (p - mean) - q (not in base's
+// buffers, which neighbouring cells still read) and q = p - mean.
+template <bool INCR>
+__global__ void __launch_bounds__(NTHREADS)
+    k_dir_correct(Lev L, DirTile t, const SliceCtl* __restrict__ ctl, const float* fu,
+                  const float* fv, const float* fw, float* u, float* v, float* w, FFBuf f,
+                  const float* base_hi, const float* base_lo, const float* __restrict__ ring,
+                  long long stride, float* __restrict__ w_hi, float* __restrict__ w_lo,
+                  double* __restrict__ p_out, float3 dt_ih, long long cu, long long cv,
+                  long long cw) {
+    pdl_wait();
+    const long long s = blockIdx.y;
+    const SliceCtl* c = ctl + s;
+    const long long off = s * L.cells;
+    const int step = c->o_steps, ne = min(step, DIR_RING - 1);
+    const float* __restrict__ e0 = ring + ((step - 1) & (DIR_RING - 1)) * stride + off;
+    const float* __restrict__ e1 = ring + ((step - 2) & (DIR_RING - 1)) * stride + off;
+    const float* __restrict__ e2 = ring + ((step - 3) & (DIR_RING - 1)) * stride + off;
+    const float* bh = base_hi + off;
+    const float* bl = base_lo + off;
+    const FF neg_mean{-c->mean_hi, -c->mean_lo};
+    const bool keep = w_hi != nullptr;
+    int i, j, k0;
+    if (!dir_origin(t, L.n, i, j, k0)) return;
+    const int nx = L.n[0], ny = L.n[1], nz = L.n[2], plane = nx * ny;
+    const int wx = L.bc[0] != BC_PERIODIC, wy = L.bc[1] != BC_PERIODIC, wz = L.bc[2] != BC_PERIODIC;
+    const int k1 = min(k0 + t.lz, nz);
+    const int base = j * nx + i;
+    const int xl = i > 0 ? base - 1 : (wx ? base : base + nx - 1);
+    const int yl = j > 0 ? base - nx : (wy ? base : base + (ny - 1) * nx);
+    // p at a cell: the newest application is the smallest, so it is added last
+    auto pat = [&](int q) -> FF {
+        FF p{bh[q], bl[q]};
+        if (ne > 2) p = ff_add_f(p, e2[q]);
+        if (ne > 1) p = ff_add_f(p, e1[q]);
+        if (ne > 0) p = ff_add_f(p, e0[q]);
+        return p;
+    };
+    FF pz = pat((k0 > 0 ? k0 - 1 : (wz ? 0 : nz - 1)) * plane + base);
+    const long long ru = s * cu + (long long)j * (nx + wx) + i, pu = (long long)ny * (nx + wx);
+    const long long rv = s * cv + (long long)j * nx + i, pv = (long long)(ny + wy) * nx;
+    const long long rw = s * cw + base;
+    const bool ax = i > 0 || !wx, ay = j > 0 || !wy;
+    constexpr int ZB = 2;
+    for (int kb = k0; kb < k1; kb += ZB) {
+        FF pc[ZB], px[ZB], py[ZB], qv[ZB];
+        float fa[ZB][3], oa[ZB][3];
+#pragma unroll
+        for (int q = 0; q < ZB; ++q) {
+            const int k = min(kb + q, k1 - 1);
+            pc[q] = pat(k * plane + base);
+            px[q] = pat(k * plane + xl);
+            py[q] = pat(k * plane + yl);
+            fa[q][0] = fu[ru + k * pu];
+            fa[q][1] = fv[rv + k * pv];
+            fa[q][2] = fw[rw + (long long)k * plane];
+            if (INCR) {
+                oa[q][0] = u[ru + k * pu];
+                oa[q][1] = v[rv + k * pv];
+                oa[q][2] = w[rw + (long long)k * plane];
+            }
+            if (keep) {
+                const long long id = off + (long long)k * plane + base;
+                qv[q] = FF{f.q_hi[id], f.q_lo[id]};
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < ZB; ++q) {
+            const int k = kb + q;
+            if (k >= k1) break;
+            auto corr = [&](int d, FF lo, float dt_h) -> float {
+                const float dgp = ((pc[q].hi - lo.hi) + (pc[q].lo - lo.lo)) * dt_h;
+                return INCR ? oa[q][d] + (fa[q][d] - dgp) : fa[q][d] - dgp;
+            };
+            u[ru + k * pu] = ax ? corr(0, px[q], dt_ih.x) : 0.0f;
+            v[rv + k * pv] = ay ? corr(1, py[q], dt_ih.y) : 0.0f;
+            w[rw + (long long)k * plane] = (k > 0 || !wz) ? corr(2, pz, dt_ih.z) : 0.0f;
+            // the high wall faces hold zero
+            if (wx && i == nx - 1) u[ru + k * pu + 1] = 0.0f;
+            if (wy && j == ny - 1) v[rv + k * pv + nx] = 0.0f;
+            if (wz && k == nz - 1) w[rw + (long long)nz * plane] = 0.0f;
+            const long long id = off + (long long)k * plane + base;
+            const FF pg = ff_add(pc[q], neg_mean);
+            if (p_out) p_out[id] = ff_to_double(pg);
+            if (keep) {
+                const FF wn = ff_add(FF{2.0f * pg.hi, 2.0f * pg.lo}, ff_neg(qv[q]));
+                w_hi[id] = wn.hi;
+                w_lo[id] = wn.lo;
+                f.q_hi[id] = pg.hi;
+                f.q_lo[id] = pg.lo;
+            }
+            pz = pc[q];
+        }
+    }
+}
 // FP64: x += e, r -= L e + mean(r), (r, r), sum x; the last CTA decides.  The
 // mean of the residual, made by rounding, is out of every correction's reach
 // (L has no range there): it is taken out of the next residual, or it would
@@ -519,6 +936,22 @@ inline std::vector<T> dir_tables(const DirPlan<T>& P, const int bc[3], const dou
             c[4 * cols + q] = (T)(-rho / ih2[2]);
         }
     return v;
+}
+
+// Tiling of the step kernels: x tiles of about 32 columns, 8 cells of the
+// march per thread (4 where a call would not fill the SMs eight CTAs deep;
+// tile_z where given).
+inline DirTile dir_tile_of(const int n[3], int cap, int tile_z) {
+    DirTile t;
+    const int xt = (n[0] + 31) / 32;
+    t.w = (n[0] + xt - 1) / xt;
+    t.r = NTHREADS / t.w;
+    t.bx = (n[0] + t.w - 1) / t.w;
+    t.by = (n[1] + t.r - 1) / t.r;
+    const long long full = (long long)t.bx * t.by * ((n[2] + 7) / 8) * cap;
+    t.lz = tile_z > 0 ? (tile_z < n[2] ? tile_z : n[2]) : (full < 152 * 8 ? 4 : 8);
+    t.ctas = t.bx * t.by * ((n[2] + t.lz - 1) / t.lz);
+    return t;
 }
 
 // Condition number of L on its range (its largest over its smallest nonzero

@@ -58,11 +58,13 @@ static int run(char** argv) {
     SliceCtl ctl[2] = {};
     ctl[0].status = ST_ITER;
     ctl[0].o_status = OS_REFINE;
+    ctl[0].o_fsc = 4.0f;  // the scale FP32 residuals carry through the transforms
+    ctl[1].o_fsc = 4.0f;
     ctl[1].status = ST_CONV;
     ctl[1].o_status = OS_DONE;
     const size_t smem = dir_smem_elems(P) * sizeof(T);
     launch(P.nz * P.xb, P.nt, 1, smem,
-           [&] { k_dir_xy<T, false>(P, ctl, r.data(), spec.data()); });
+           [&] { k_dir_xy<T, false>(P, ctl, r.data(), spec.data(), 0); });
     const int zg = (P.nx * P.ny + DIR_ZX - 1) / DIR_ZX;
     launch(zg, DIR_ZX, P.zc, 0, [&] {
         if (P.zm == DIR_ZC)
@@ -71,7 +73,7 @@ static int run(char** argv) {
             k_dir_z<T, DIR_ZC_LONG>(P, ctl, spec.data());
     });
     launch(P.nz * P.xb, P.nt, 1, smem,
-           [&] { k_dir_xy<T, true>(P, ctl, spec.data(), e.data()); });
+           [&] { k_dir_xy<T, true>(P, ctl, spec.data(), e.data(), 0); });
     f = fopen(argv[13], "wb");
     fwrite(e.data(), sizeof(T), 2 * N, f);
     fclose(f);
