@@ -122,10 +122,9 @@ typedef struct {
     int predict_tile_z;      /* 32 x predict_tile_y x predict_tile_z cells, one
                                 thread per (x, y) column marching z; (y, z) one of
                                 (4,4) (4,8) (8,2) (8,4) (8,8) (16,4), else
-                                NS_ERR_ARG; (0, 0): (8, 4).  Every face takes the
-                                same operands whatever the tile; results move only
-                                at rounding level (the compiler may fuse products
-                                into multiply-adds differently per shape).        */
+                                NS_ERR_ARG; (0, 0): chosen by size and batch.
+                                Every face takes the same operations whatever the
+                                tile, so the results do not depend on it.         */
     int coarse_tile_z;       /* tile_z of the batch-1 companion grid on which
                                 ns_parareal_iterate evaluates the coarse
                                 propagator (every G of a grid, so G_new and G_old

@@ -262,6 +262,26 @@ void free_all(ns_grid* g) {
 
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
+// Default predictor tile of a grid: 16 columns wide where that leaves an
+// eighth fewer columns idle than 32, and of the shapes below the longest march
+// that still gives the call about 1500 warps (ten per SM): a longer march
+// stages fewer halo planes per cell (64^3 x 32 states, FP32: 399 us with one
+// plane, 225 with 4, 156 with 32), too few warps leave SMs idle (one 16^3
+// state, FP64: 16 us with one plane, 154 with 16).
+void predict_tile_auto(const int n[3], int cap, int& px, int& py, int& pz) {
+    static const int shapes[2][7][2] = {
+        {{8, 32}, {8, 16}, {8, 8}, {8, 4}, {4, 4}, {4, 2}, {4, 1}},
+        {{8, 32}, {8, 8}, {8, 8}, {4, 4}, {4, 4}, {4, 2}, {4, 1}}};
+    px = 8 * ceil_div(n[0], 16) <= 14 * ceil_div(n[0], 32) ? 16 : 32;
+    for (const auto& s : shapes[px == 16]) {
+        py = s[0];
+        pz = s[1];
+        const long long warps = (long long)cap * ceil_div(n[0], px) * ceil_div(n[1], py) *
+                                ceil_div(n[2], pz) * (px * py / 32);
+        if (warps >= 1500) return;
+    }
+}
+
 void setup_geo(ns_grid* g) {
     Geo& G = g->geo;
     const ns_grid_desc& d = g->d;
@@ -303,8 +323,10 @@ void setup_geo(ns_grid* g) {
     G.fctas = G.fbx * G.fby * G.fbz;
     G.n_fluid = G.n[0] * G.n[1] * G.n[2];
     const bool deflt = d.predict_tile_y == 0 && d.predict_tile_z == 0;
-    G.pty = deflt ? PT_Y : d.predict_tile_y;
-    G.ptz = deflt ? PT_Z : d.predict_tile_z;
+    G.ptx = PT_X;
+    G.pty = d.predict_tile_y;
+    G.ptz = d.predict_tile_z;
+    if (deflt) predict_tile_auto(G.n, g->cap, G.ptx, G.pty, G.ptz);
 }
 
 // Face codes of the finest level with solid cells (FC_FLUID and one bit per
@@ -1546,6 +1568,32 @@ ns_status solve_pressure(ns_grid* g, int batch, const double* p_in) {
     return NS_OK;
 }
 
+// Calls f with the predictor tile (px, py, pz) as constants.
+template <typename F>
+auto with_predict_tile(int px, int py, int pz, F&& f) {
+    using std::integral_constant;
+#define NS_TILE(X, Y, Z) \
+    f(integral_constant<int, X>{}, integral_constant<int, Y>{}, integral_constant<int, Z>{})
+    switch (px * 10000 + py * 100 + pz) {
+        case 160401: return NS_TILE(16, 4, 1);
+        case 160402: return NS_TILE(16, 4, 2);
+        case 160404: return NS_TILE(16, 4, 4);
+        case 160808: return NS_TILE(16, 8, 8);
+        case 160832: return NS_TILE(16, 8, 32);
+        case 320401: return NS_TILE(32, 4, 1);
+        case 320402: return NS_TILE(32, 4, 2);
+        case 320404: return NS_TILE(32, 4, 4);
+        case 320408: return NS_TILE(32, 4, 8);
+        case 320802: return NS_TILE(32, 8, 2);
+        case 320808: return NS_TILE(32, 8, 8);
+        case 320816: return NS_TILE(32, 8, 16);
+        case 320832: return NS_TILE(32, 8, 32);
+        case 321604: return NS_TILE(32, 16, 4);
+        default: return NS_TILE(32, 8, 4);
+    }
+#undef NS_TILE
+}
+
 template <typename T, bool INCR>
 void launch_predict(ns_grid* g, int batch, const T* u, const T* v, const T* w, T* fu, T* fv, T* fw,
                     double dt) {
@@ -1555,52 +1603,28 @@ void launch_predict(ns_grid* g, int batch, const T* u, const T* v, const T* w, T
             G, u, v, w, fu, fv, fw, dt);
         return;
     }
-    auto go = [&](auto py_c, auto pz_c) {
-        constexpr int PY = decltype(py_c)::value, PZ = decltype(pz_c)::value;
-        const int tbx = ceil_div(G.n[0], PT_X), tby = ceil_div(G.n[1], PY),
+    with_predict_tile(G.ptx, G.pty, G.ptz, [&](auto px, auto py, auto pz) {
+        constexpr int PX = decltype(px)::value, PY = decltype(py)::value,
+                      PZ = decltype(pz)::value;
+        const int tbx = ceil_div(G.n[0], PX), tby = ceil_div(G.n[1], PY),
                   tbz = ceil_div(G.n[2], PZ);
-        const size_t smem = 3 * (size_t)ptile_elems<PY, PZ>() * sizeof(T);
-        k_predict_tile<T, INCR, PY, PZ><<<dim3(tbx * tby * tbz, batch), PT_X * PY, smem,
-                                          g->stream>>>(G, u, v, w, fu, fv, fw, dt, tbx, tby);
-    };
-    using I2 = std::integral_constant<int, 2>;
-    using I4 = std::integral_constant<int, 4>;
-    using I8 = std::integral_constant<int, 8>;
-    using I16 = std::integral_constant<int, 16>;
-    const int key = G.pty * 100 + G.ptz;
-    switch (key) {
-        case 404: go(I4{}, I4{}); break;
-        case 408: go(I4{}, I8{}); break;
-        case 802: go(I8{}, I2{}); break;
-        case 808: go(I8{}, I8{}); break;
-        case 1604: go(I16{}, I4{}); break;
-        default: go(I8{}, I4{}); break;
-    }
+        const size_t smem = 3 * (size_t)ptile_elems<PY, PZ, PX>() * sizeof(T);
+        k_predict_tile<T, INCR, PY, PZ, PX><<<dim3(tbx * tby * tbz, batch), PX * PY, smem,
+                                              g->stream>>>(G, u, v, w, fu, fv, fw, dt, tbx, tby);
+    });
 }
 
 // Shared memory limit of the predictor instantiation the grid uses (a value
 // fixed per instantiation, so grids never lower each other's).
 template <typename T, bool INCR>
-cudaError_t predict_smem_attr(int pty, int ptz) {
-    auto set = [](auto py_c, auto pz_c) {
-        constexpr int PY = decltype(py_c)::value, PZ = decltype(pz_c)::value;
-        const int bytes = 3 * ptile_elems<PY, PZ>() * (int)sizeof(T);
-        if (bytes <= 48 * 1024) return cudaSuccess;
-        return cudaFuncSetAttribute(k_predict_tile<T, INCR, PY, PZ>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    };
-    using I2 = std::integral_constant<int, 2>;
-    using I4 = std::integral_constant<int, 4>;
-    using I8 = std::integral_constant<int, 8>;
-    using I16 = std::integral_constant<int, 16>;
-    switch (pty * 100 + ptz) {
-        case 404: return set(I4{}, I4{});
-        case 408: return set(I4{}, I8{});
-        case 802: return set(I8{}, I2{});
-        case 808: return set(I8{}, I8{});
-        case 1604: return set(I16{}, I4{});
-        default: return set(I8{}, I4{});
-    }
+cudaError_t predict_smem_attr(const Geo& G) {
+    return with_predict_tile(G.ptx, G.pty, G.ptz, [](auto px, auto py, auto pz) {
+        constexpr int PX = decltype(px)::value, PY = decltype(py)::value,
+                      PZ = decltype(pz)::value;
+        return cudaFuncSetAttribute(k_predict_tile<T, INCR, PY, PZ, PX>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    3 * ptile_elems<PY, PZ, PX>() * (int)sizeof(T));
+    });
 }
 
 bool predict_tile_ok(int y, int z) {
@@ -2793,11 +2817,11 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             cudaMemsetAsync(g->loopc, 0, sizeof(LoopCount), g->stream) != cudaSuccess)
             st = fail(NS_ERR_CUDA, "ns_create_grid: memset failed");
         if (st == NS_OK) {
-            const int py = g->geo.pty, pz = g->geo.ptz;
-            const bool ok = g->fp32 ? (predict_smem_attr<float, false>(py, pz) == cudaSuccess &&
-                                       predict_smem_attr<float, true>(py, pz) == cudaSuccess)
-                                    : (predict_smem_attr<double, false>(py, pz) == cudaSuccess &&
-                                       predict_smem_attr<double, true>(py, pz) == cudaSuccess);
+            const Geo& G = g->geo;
+            const bool ok = g->fp32 ? (predict_smem_attr<float, false>(G) == cudaSuccess &&
+                                       predict_smem_attr<float, true>(G) == cudaSuccess)
+                                    : (predict_smem_attr<double, false>(G) == cudaSuccess &&
+                                       predict_smem_attr<double, true>(G) == cudaSuccess);
             if (!ok) st = fail(NS_ERR_CUDA, "ns_create_grid: predictor shared memory attribute");
         }
         if (st == NS_OK && g->mg) {

@@ -71,7 +71,7 @@ struct Geo {
     int n_fluid;         // fluid cells per state
     const uint8_t* solid;  // device cell mask (1 = solid), nullptr without obstacles
     float fih[3], fih2[3], finv_re;  // FP32 copies (no FP64 conversions in FP32 kernels)
-    int pty, ptz;        // predictor tile: 32 x pty x ptz cells
+    int ptx, pty, ptz;   // predictor tile: ptx x pty x ptz cells
 };
 
 // h^-1, h^-2 and 1/Re in the kernel's precision
@@ -173,25 +173,83 @@ __device__ __forceinline__ T smart_flux(T uf, T bb, T b, T f, T ff) {
     return T(0);
 }
 
-// The same flux without branches (for warps whose faces take different
-// SMART branches): pick the upwind triple, evaluate every branch, select.
-// uf = 0 gives 0 as above (the face value is finite).
+// phi_face of a face between b and f as above, transported by tr (twice the
+// velocity; of a transport of zero any finite value serves), from differences: with k = C - U and g = D - C the SMART
+// value is C + min(2 |k|, |k|/8 + 3|g|/8, |g|) in g's direction where k and g
+// have the same sign (C between U and D), else C -- the three branches are the
+// three arguments, each the smallest on its range of cc/dd.
 template <typename T>
-__device__ __forceinline__ T smart_flux_sel(T uf, T bb, T b, T f, T ff) {
-    const bool pos = uf > T(0);
-    const T U = pos ? bb : ff;
+__device__ __forceinline__ T smart_phi(T tr, T bb, T b, T f, T ff) {
+    const bool pos = tr > T(0);
     const T C = pos ? b : f;
-    const T D = pos ? f : b;
-    const T dd = D - U;
-    const T cc = C - U;
-    const T a = dd > T(0) ? cc : -cc;
-    const T bd = fabs(dd);
-    const T quick = fma(T(0.75), cc, fma(T(0.375), dd, U));
-    const T steep = fma(T(3), cc, U);
-    T phi = (T(6) * a <= bd) ? steep : ((T(6) * a <= T(5) * bd) ? quick : D);
-    phi = (dd == T(0) || a < T(0) || a > bd) ? C : phi;
-    return uf * phi;
+    const T k = (pos ? b : ff) - (pos ? bb : f);  // (of the x-ordered line)
+    const T g = f - b;
+    const T ks = g < T(0) ? -k : k, ag = fabs(g);
+    const T q = fma(T(0.375), ag, T(0.125) * ks);
+    const T m = max(min(min(ks + ks, q), ag), T(0));
+    return C + ((g < T(0)) == pos ? -m : m);
 }
+#ifdef __CUDA_ARCH__
+// FP32: differences (FMA pipe) rather than selects (the ALU has half its
+// rate); the signs as bits.
+template <>
+__device__ __forceinline__ float smart_phi<float>(float tr, float bb, float b, float f,
+                                                    float ff) {
+    const bool pos = tr > 0.0f;
+    const float C = pos ? b : f;
+    const float kl = b - bb, kr = ff - f, g = f - b;
+    const float k = pos ? kl : kr;
+    const float q = fmaf(0.375f, g, 0.125f * k);
+    float m = fminf(fminf(fabsf(k + k), fabsf(q)), fabsf(g));
+    m = ((__float_as_uint(k) ^ __float_as_uint(g)) & 0x80000000u) != 0 ? 0.0f : m;
+    const unsigned flip = (__float_as_uint(g) ^ __float_as_uint(tr)) & 0x80000000u;
+    return C + __uint_as_float(__float_as_uint(m) ^ flip);
+}
+// FP64: the comparisons, signs and powers of two on the integer pipe (the
+// order of nonnegative doubles is that of their bits; a scaled |k| below
+// 2^-1019 counts as 0, a |k| of 0 as 2^-1022 in the comparison).
+template <>
+__device__ __forceinline__ double smart_phi<double>(double tr, double bb, double b, double f,
+                                                      double ff) {
+    const int ht = __double2hiint(tr);
+    const bool pos = ht >= 0;
+    const double C = pos ? b : f;
+    const double k = (pos ? b : ff) - (pos ? bb : f);
+    const double g = f - b;
+    const int hk = __double2hiint(k), hg = __double2hiint(g);
+    const int ak = hk & 0x7fffffff, ah = hg & 0x7fffffff;
+    const double k8 = ak >= 0x00400000 ? __hiloint2double(ak - 0x00300000, __double2loint(k)) : 0.0;
+    const double ag = __hiloint2double(ah, __double2loint(g));
+    const double q = fma(0.375, ag, k8);
+    const unsigned long long K = (unsigned long long)__double_as_longlong(
+                                     __hiloint2double(ak, __double2loint(k))) +
+                                 (1ull << 52);
+    const unsigned long long Q = (unsigned long long)__double_as_longlong(q);
+    const unsigned long long A = (unsigned long long)__double_as_longlong(ag);
+    // C + 2 |k|, C + q or C + |g|, with g's direction seen from C
+    const bool steep = K <= Q && K < A;
+    const bool down = !steep && A <= Q;
+    int hx = steep ? ak : (down ? ah : __double2hiint(q));
+    int lx = steep ? __double2loint(k) : (down ? __double2loint(g) : __double2loint(q));
+    const bool same = (hk ^ hg) >= 0;
+    hx ^= (hg ^ ht) & 0x80000000;
+    hx = same ? hx : 0;
+    lx = same ? lx : 0;
+    const double w = __hiloint2double(steep ? 0x40000000 : 0x3ff00000, 0);
+    return fma(w, __hiloint2double(hx, lx), C);
+}
+#endif
+
+// a b rounded: not contracted with a sum it enters.
+template <typename T> __device__ __forceinline__ T mul_rounded(T a, T b) { return a * b; }
+#ifdef __CUDA_ARCH__
+template <> __device__ __forceinline__ float mul_rounded<float>(float a, float b) {
+    return __fmul_rn(a, b);
+}
+template <> __device__ __forceinline__ double mul_rounded<double>(double a, double b) {
+    return __dmul_rn(a, b);
+}
+#endif
 
 __device__ __forceinline__ bool cell_solid(const Geo& g, int i, int j, int k) {
     return g.solid != nullptr && g.solid[cindex(g, i, j, k)] != 0;

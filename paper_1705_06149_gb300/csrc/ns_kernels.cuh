@@ -61,160 +61,271 @@ struct KBuf {       // Krylov vectors of all states, [batch][cells]
 // predictor  F* = u + dt (Re^-1 lap u - div(u u))
 // ---------------------------------------------------------------------------
 
-// Tiled predictor: a CTA of PT_X x PT_Y x PT_Z cells stages u, v, w on its
-// tile and a halo of two positions (ghost values applied while staging), then
-// evaluates every face of the tile from shared memory with constant strides.
+// Tiled predictor: a CTA owns PX x PY columns and PZ cells along z.  It marches
+// in z with a ring of PT_RING planes of u, v, w in shared memory (tile and a
+// halo of two positions, ghost values applied while staging; the plane three
+// ahead is loaded during a step and stored at its end) and evaluates every face
+// flux once: a thread owns the column (x, y) and computes the fluxes through
+// its cell's high faces; the low ones are the left lane's (a shuffle), the
+// lower row's (through shared memory; one barrier per z step) and the ones of
+// the cell below (carried).  The fluxes through the tile's low x and y faces
+// are computed by other threads in turn.
 // Faces owned by the tile: the low face of each of its cells along each
 // component's axis, plus the high wall face of the last cell of the domain.
-// The tile is PT_X x PY x PZ cells (PT_X x PY threads); the default is
-// 32 x 8 x 4, and the tile autotuner chooses among the instantiated shapes.
+// predict_tile_auto chooses the tile, or the tile autotuner among the shapes
+// of PT_X columns.
+// Bound: FP64, the FP64 pipe (a warp instruction holds it 16 cycles, so the
+// face value is selected by integer comparisons and costs four FP64
+// operations); FP32, instruction issue (hence the march: staging a tile with
+// its z halo at once took half of all instructions) with 16 warps per SM (24
+// with a third of the registers less: 168 us against 156 below).
+// Measured against evaluating every y flux twice and the face value by
+// comparisons, from 32 x 8 x 4 tiles staged at once: 64^3 x 32 states FP32
+// 280 -> 156 us, 64^3 FP32 27 -> 12 us, 64^3 x 4 FP64 747 -> 294 us, 16^3 FP64
+// 121 -> 16 us.
 constexpr int PT_X = 32, PT_Y = 8, PT_Z = 4;
 constexpr int PT_THREADS = PT_X * PT_Y;
-constexpr int PH = 2;  // halo
-constexpr int PS_X = PT_X + 2 * PH, PS_Y = PT_Y + 2 * PH, PS_Z = PT_Z + 2 * PH;
-constexpr int PS_N = PS_X * PS_Y * PS_Z;
+constexpr int PH = 2;       // halo
+#ifdef __CUDACC__
+#define NS_MIN_CTAS(...) , __VA_ARGS__
+#else
+#define NS_MIN_CTAS(...)
+#endif
+constexpr int PT_RING = 5;  // planes z-1 .. z+2 in use, z+3 being stored
 
-// Staged elements of one component for a PT_X x PY x PZ tile.
-template <int PY, int PZ>
+// Staged elements of one component for a PX x PY x PZ tile (whatever PZ).
+template <int PY, int PZ, int PX = PT_X>
 constexpr int ptile_elems() {
-    return (PT_X + 2 * PH) * (PY + 2 * PH) * (PZ + 2 * PH);
+    return (PX + 2 * PH) * (PY + 2 * PH) * PT_RING;
 }
 
-template <typename T, bool INCR, int PY = PT_Y, int PZ = PT_Z>
-__global__ void __launch_bounds__(PT_X * PY)
+template <typename T, bool INCR, int PY = PT_Y, int PZ = PT_Z, int PX = PT_X>
+__global__ void __launch_bounds__(PX * PY NS_MIN_CTAS(512 / (PX * PY)))
     k_predict_tile(Geo g, const T* __restrict__ u, const T* __restrict__ v,
                    const T* __restrict__ w, T* __restrict__ fu, T* __restrict__ fv,
                    T* __restrict__ fw, double dt, int tbx, int tby) {
     pdl_wait();
-    constexpr int PT_Y = PY, PT_Z = PZ;
-    constexpr int PT_THREADS = PT_X * PY;
-    constexpr int PS_Y = PY + 2 * PH, PS_Z = PZ + 2 * PH;
-    constexpr int PS_N = PS_X * PS_Y * PS_Z;
+    constexpr int NT = PX * PY;
+    constexpr int SX = PX + 2 * PH, SY = PY + 2 * PH;
+    constexpr int PLANE = SX * SY, SN = PLANE * PT_RING;
+    constexpr int PER = (PLANE + NT - 1) / NT;
+    static_assert(PER <= 5, "two flag bits per staged position and component");
     extern __shared__ __align__(16) unsigned char psm_raw[];
-    T* sm = reinterpret_cast<T*>(psm_raw);  // [3][PS_Z][PS_Y][PS_X]
+    T* sm = reinterpret_cast<T*>(psm_raw);  // [3][PT_RING][SY][SX]
+    // fluxes through the tile's low x / y faces and the rows' high y faces, by
+    // parity of the z step
+    __shared__ T xlo[2][3][PY], ylo[2][3][PX], yex[2][3][PY][PX];
+    __shared__ T coef[6];  // dt / (2 h) (the fluxes are twice the convective ones), dt / (Re h^2)
+    __shared__ int zsrc[3][PZ + 4];  // z index a staged plane comes from, ~ of it: sign -1
     const long long s = blockIdx.y;
     const T* vel3[3] = {u + s * g.cnt[0], v + s * g.cnt[1], w + s * g.cnt[2]};
     T* out[3] = {fu + s * g.cnt[0], fv + s * g.cnt[1], fw + s * g.cnt[2]};
     const int cta = blockIdx.x;
-    const int i0 = (cta % tbx) * PT_X;
-    const int j0 = ((cta / tbx) % tby) * PT_Y;
-    const int k0 = (cta / (tbx * tby)) * PT_Z;
+    const int tyz = cta / tbx, tz = tyz / tby;
+    const int i0 = (cta - tyz * tbx) * PX;
+    const int j0 = (tyz - tz * tby) * PY;
+    const int k0 = tz * PZ;
     const int t = threadIdx.x;
-    // Stage positions (i0-2 .. i0+PT_X+1) etc. of every component, ghost
-    // values applied (the rules act on each axis separately).  The z part of
-    // the rules is the same for the whole CTA and the x / y part is fixed per
-    // plane position, so each is evaluated once; every element then costs a
-    // load and at most a multiply-add.
-    constexpr int PLANE = PS_X * PS_Y;
-    constexpr int PER = (PLANE + PT_THREADS - 1) / PT_THREADS;
+    const int zn = min(PZ, g.n[2] - k0);
+    // (one warp: a warp's FP64 operation holds the pipe whatever its lanes)
+    if (t < 6) {
+        const int d = t < 3 ? t : t - 3;
+        coef[t] = T(dt * (t < 3 ? 0.5 * g.ih[d] : g.inv_re * g.ih2[d]));
+    }
+    for (int q = t; q < 3 * (PZ + 4); q += NT) {
+        const int c = q / (PZ + 4), gk = k0 - PH + q - c * (PZ + 4);
+        int qk = gk;
+        T sign = T(1), add = T(0);
+        ghost_axis(g, c, 2, qk, sign, add);
+        // (positions further out are staged from anywhere and not used)
+        if (gk >= g.ext[c][2] + PH) qk = 0;
+        zsrc[c][q - c * (PZ + 4)] = sign < T(0) ? ~qk : qk;
+    }
+    // The plane positions this thread stages: offset in the plane, and flags
+    // (1: sign of the ghost rule, 2: the lid's ghost)
+    unsigned off[PER][3], flags = 0;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int e0 = g.ext[c][0], e1 = g.ext[c][1], e2 = g.ext[c][2];
-        const long long plane = (long long)e1 * e0;
-        long long zoff[PS_Z];
-        T zsign[PS_Z];
-        bool zghost[PS_Z], znear[PS_Z];
+    for (int h = 0; h < PER; ++h) {
+        const int pq = t + h * NT;
+        const int py = pq / SX, px = pq - py * SX;
+        const int gi = i0 - PH + px, gj = j0 - PH + py;
 #pragma unroll
-        for (int z = 0; z < PS_Z; ++z) {
-            const int gk = k0 - PH + z;
-            int qk = gk;
-            T sg = T(1), ad = T(0);
-            ghost_axis(g, c, 2, qk, sg, ad);
-            zoff[z] = qk * plane;
-            zsign[z] = sg;
-            zghost[z] = gk < 0 || gk >= e2;
-            znear[z] = gk >= -PH && gk < e2 + PH;
+        for (int c = 0; c < 3; ++c) {
+            const int e0 = g.ext[c][0], e1 = g.ext[c][1];
+            int qi = gi, qj = gj;
+            T sign = T(1), add = T(0);
+            // only positions up to two beyond the stored range are ever read
+            const bool near = pq < PLANE && gi < e0 + PH && gj < e1 + PH;
+            ghost_axis(g, c, 0, qi, sign, add);
+            ghost_axis(g, c, 1, qj, sign, add);
+            off[h][c] = near ? (unsigned)qj * (unsigned)e0 + (unsigned)qi : 0u;
+            const bool lid = near && c == 0 && gj >= e1 && g.bc[1] == BC_WALL;
+            flags |= ((near && sign < T(0) ? 1u : 0u) | (lid ? 2u : 0u)) << (2 * (3 * h + c));
+        }
+    }
+    const T lid2 = T(2.0 * g.u_lid);
+    __syncthreads();
+    T val[PER][3];
+    unsigned zneg = 0;
+    // plane z (from k0 - 2) into registers; then into the ring, ghost values
+    // (the lid) + sign * mirror applied
+    auto load_plane = [&](int z) {
+        zneg = 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const int zs = zsrc[c][z];
+            if (zs < 0) zneg |= 1u << c;
+            const T* __restrict__ a =
+                vel3[c] + (long long)(zs < 0 ? ~zs : zs) * (g.ext[c][1] * g.ext[c][0]);
+#pragma unroll
+            for (int h = 0; h < PER; ++h) val[h][c] = a[off[h][c]];
+        }
+    };
+    auto put_plane = [&](int slot) {
+        if ((flags | zneg) != 0) {
+#pragma unroll
+            for (int h = 0; h < PER; ++h)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const unsigned f = flags >> (2 * (3 * h + c));
+                    if (((f ^ (zneg >> c)) & 1u) != 0) val[h][c] = -val[h][c];
+                    if (f & 2u) val[h][c] += lid2;
+                }
         }
 #pragma unroll
-        for (int h = 0; h < PER; ++h) {
-            const int pq = t + h * PT_THREADS;
-            if (pq >= PLANE) break;
-            const int x = pq % PS_X, y = pq / PS_X;
-            const int gi = i0 - PH + x, gj = j0 - PH + y;
-            int qi = gi, qj = gj;
-            T sxy = T(1), add = T(0);
-            ghost_axis(g, c, 0, qi, sxy, add);
-            ghost_axis(g, c, 1, qj, sxy, add);
-            const bool xy_ghost = gi < 0 || gj < 0 || gi >= e0 || gj >= e1;
-            // only positions up to two beyond the stored range are ever read
-            const bool xy_near = gi >= -PH && gj >= -PH && gi < e0 + PH && gj < e1 + PH;
-            const T* __restrict__ a = vel3[c] + (long long)qj * e0 + qi;
-            T* dst = sm + c * PS_N + pq;
+        for (int h = 0; h < PER; ++h)
+            if ((h + 1) * NT <= PLANE || t + h * NT < PLANE) {
 #pragma unroll
-            for (int z = 0; z < PS_Z; ++z) {
-                T val = T(0);
-                if (xy_near && znear[z]) {
-                    const T st = a[zoff[z]];
-                    // stored values as they are (wall-normal boundary faces
-                    // are stored as 0); ghosts = add + sign * mirror
-                    val = (xy_ghost || zghost[z]) ? add + (sxy * zsign[z]) * st : st;
-                }
-                dst[z * PLANE] = val;
+                for (int c = 0; c < 3; ++c) sm[c * SN + slot + t + h * NT] = val[h][c];
             }
+    };
+#pragma unroll 1
+    for (int z = 0; z < PT_RING; ++z) {
+        load_plane(z);
+        put_plane(z * PLANE);
+    }
+    __syncthreads();
+    const int y = t / PX, x = t - y * PX;
+    // this thread's column in the ring's planes z - 1 .. z + 2, and the offset
+    // of the plane being stored
+    const T* qm = sm + (y + PH) * SX + x + PH + PLANE;
+    const T* q0 = qm + PLANE;
+    const T* q1 = q0 + PLANE;
+    const T* q2 = q1 + PLANE;
+    int pn = 0;
+    // the low face this thread also computes (from the last thread on, the
+    // first ones stage more): component, position, transport
+    constexpr int NE = 3 * (PX + PY), EPER = (NE + NT - 1) / NT;
+    int eb[EPER], et[EPER], el[EPER];
+    T* eo[EPER];
+    bool ey[EPER];
+#pragma unroll
+    for (int h = 0; h < EPER; ++h) {
+        const int q = min(NT - 1 - t + h * NT, NE - 1);
+        const bool yf = q < 3 * PX;
+        const int r = yf ? q : q - 3 * PX, len = yf ? PX : PY;
+        const int c = r >= 2 * len ? 2 : (r >= len ? 1 : 0), e = r - c * len;
+        const int at = yf ? (PH - 1) * SX + e + PH : (e + PH) * SX + PH - 1;
+        eb[h] = c * SN + at;
+        et[h] = (yf ? SN : 0) + at + (yf ? SX : 1);
+        // its transport's low neighbour: one back along c
+        el[h] = c == 0 ? 1 : (c == 1 ? SX : 0);
+        eo[h] = yf ? &ylo[0][c][e] : &xlo[0][c][e];
+        ey[h] = yf;
+    }
+    const T kc[3] = {coef[0], coef[1], coef[2]}, kd[3] = {coef[3], coef[4], coef[5]};
+    const int i = i0 + x, j = j0 + y;
+    T fz[3], zm[3], zc[3], zp[3];
+    T* dst[3];
+    // twice the flux through the low z face of the tile's first cell
+    {
+        const T w0 = q0[2 * SN];
+        const T tr[3] = {q0[2 * SN - 1] + w0, q0[2 * SN - SX] + w0, qm[2 * SN] + w0};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            zm[c] = qm[c * SN];
+            zc[c] = q0[c * SN];
+            zp[c] = q1[c * SN];
+            fz[c] = mul_rounded(tr[c], smart_phi(tr[c], qm[c * SN - PLANE], zm[c], zc[c], zp[c]));
+            dst[c] = out[c] + vindex(g, c, i, j, k0);
         }
     }
     __syncthreads();
-    const T tdt = T(dt), inv_re = g_inv_re<T>(g);
-    constexpr int strd[3] = {1, PS_X, PS_X * PS_Y};
-    // Each thread owns the column (x, y) = (lane, warp) of the tile and marches
-    // its PT_Z cells in z.  A face flux is evaluated once: the flux entering
-    // cell x across its low x face is the one lane x-1 computed for its high
-    // face (a shuffle), and the low z face flux is the high one of the cell
-    // below (carried along the march); only y fluxes are evaluated on both
-    // faces.  The operands are the same values either way, so the fluxes are
-    // identical to evaluating every face from both sides.
-    const int x = t % PT_X, y = t / PT_X;
-    const unsigned lane = t & 31u;
+    const bool in_xy = i < g.n[0] && j < g.n[1];
+    // faces on the walls: the low one, and the high one beside the last cell
+    const bool wlo[2] = {g.bc[0] != BC_PERIODIC && i == 0, g.bc[1] != BC_PERIODIC && j == 0};
+    const bool whi[2] = {g.bc[0] != BC_PERIODIC && i == g.n[0] - 1,
+                         g.bc[1] != BC_PERIODIC && j == g.n[1] - 1};
+#pragma unroll 1
+    for (int z = 0; z < zn; ++z) {
+        const int par = z & 1;
+        const bool more = z + 1 < zn;
+        if (more) load_plane(z + 5);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const T* sc = sm + c * PS_N;
-        const int sc_c = strd[c];
-        // transport velocity at the high face of direction d of the cell at o
-        auto up_at = [&](int d, int o) -> T {
-            const int sd = strd[d];
-            if (d == c) return T(0.5) * (sc[o] + sc[o + sd]);
-            const T* sdc = sm + d * PS_N;
-            return T(0.5) * (sdc[o - sc_c + sd] + sdc[o + sd]);
-        };
-        T fz_lo = T(0);
-        for (int z = 0; z < PT_Z; ++z) {
-            const int o = ((z + PH) * PS_Y + (y + PH)) * PS_X + (x + PH);
-            T conv = T(0), diff = T(0);
+        for (int h = 0; h < EPER; ++h)
+            if (NT - 1 - t + h * NT < NE) {
+                const int p0 = (int)(q0 - (sm + (y + PH) * SX + x + PH));
+                const int pm = (int)(qm - (sm + (y + PH) * SX + x + PH));
+                const T* sc = sm + eb[h] + p0;
+                const T* st = sm + et[h];
+                const int sd = ey[h] ? SX : 1;
+                const T tl = el[h] == 0 ? st[pm] : st[p0 - el[h]];
+                const T tr = tl + st[p0];
+                eo[h][par * (ey[h] ? 3 * PX : 3 * PY)] =
+                    mul_rounded(tr, smart_phi(tr, sc[-sd], sc[0], sc[sd], sc[2 * sd]));
+            }
+        T inc[3], tx[3], ty[3], px[3], py[3], fxl[3];
+        const T uh = q0[1], vh = q0[SN + SX], wh = zp[2];
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const int sd = strd[d];
-                const T a0 = sc[o - 2 * sd], a1 = sc[o - sd], a2 = sc[o], a3 = sc[o + sd],
-                        a4 = sc[o + 2 * sd];
-                const T fp = smart_flux_sel(up_at(d, o), a1, a2, a3, a4);
-                T fm;
-                if (d == 0) {
-                    fm = __shfl_up_sync(0xffffffffu, fp, 1);
-                    if (lane == 0) fm = smart_flux_sel(up_at(0, o - 1), a0, a1, a2, a3);
-                } else if (d == 1 || z == 0) {
-                    fm = smart_flux_sel(up_at(d, o - sd), a0, a1, a2, a3);
-                } else {
-                    fm = fz_lo;
-                }
-                if (d == 2) fz_lo = fp;
-                conv += (fp - fm) * g_ih<T>(g, d);
-                diff += (a3 - T(2) * a2 + a1) * g_ih2<T>(g, d);
-            }
-            const int f[3] = {i0 + x, j0 + y, k0 + z};
-            if (f[0] >= g.n[0] || f[1] >= g.n[1] || f[2] >= g.n[2]) continue;
-            const long long id = vindex(g, c, f[0], f[1], f[2]);
-            // the high wall face of the last cell along c is inactive: zero it
-            if (g.bc[c] != BC_PERIODIC && f[c] == g.n[c] - 1) {
-                int h3[3] = {f[0], f[1], f[2]};
-                h3[c] += 1;
-                out[c][vindex(g, c, h3[0], h3[1], h3[2])] = T(0);
-            }
-            if (!(g.bc[c] == BC_PERIODIC || f[c] > 0)) {
-                out[c][id] = T(0);
-                continue;
-            }
-            const T incr = tdt * (inv_re * diff - conv);
-            out[c][id] = INCR ? incr : sc[o] + incr;
+        for (int c = 0; c < 3; ++c) {
+            const T a = zc[c];
+            const T xl = q0[c * SN - 1], xh = c == 0 ? uh : q0[c * SN + 1];
+            const T yl = q0[c * SN - SX], yh = c == 1 ? vh : q0[c * SN + SX], zpp = q2[c * SN];
+            // transport sums of the high x, y, z faces, face values
+            tx[c] = uh + (c == 0 ? a : (c == 1 ? q0[1 - SX] : qm[1]));
+            ty[c] = vh + (c == 1 ? a : (c == 0 ? q0[SN + SX - 1] : qm[SN + SX]));
+            const T tw = wh + (c == 2 ? a : q1[2 * SN - (c == 0 ? 1 : SX)]);
+            px[c] = smart_phi(tx[c], xl, a, xh, q0[c * SN + 2]);
+            py[c] = smart_phi(ty[c], yl, a, yh, q0[c * SN + 2 * SX]);
+            const T pz = smart_phi(tw, zm[c], a, zp[c], zpp);
+            yex[par][c][y][x] = mul_rounded(ty[c], py[c]);
+            fxl[c] = __shfl_up_sync(0xffffffffu, mul_rounded(tx[c], px[c]), 1);
+            // (fma by fma: every tile shape rounds alike; the cell's own high
+            // flux enters unrounded)
+            inc[c] = fma((yh - a) - (a - yl), kd[1], ((xh - a) - (a - xl)) * kd[0]);
+            inc[c] = fma((zp[c] - a) - (a - zm[c]), kd[2], inc[c]);
+            inc[c] = fma(-fma(tw, pz, -fz[c]), kc[2], inc[c]);
+            fz[c] = mul_rounded(tw, pz);
+            zm[c] = a;
+            zc[c] = zp[c];
+            zp[c] = zpp;
         }
+        if (more) put_plane(pn);
+        __syncthreads();
+        const int k = k0 + z;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const T xl = x == 0 ? xlo[par][c][y] : fxl[c];
+            const T yl = y == 0 ? ylo[par][c][x] : yex[par][c][y > 0 ? y - 1 : 0][x];
+            const T incr = fma(-fma(ty[c], py[c], -yl), kc[1],
+                               fma(-fma(tx[c], px[c], -xl), kc[0], inc[c]));
+            const bool wall = g.bc[c] != BC_PERIODIC;
+            const bool lo = c < 2 ? wlo[c < 2 ? c : 0] : (wall && k == 0);
+            // the high wall face of the last cell along c is inactive: zero it
+            const bool hi = c < 2 ? whi[c < 2 ? c : 0] : (wall && k == g.n[2] - 1);
+            if (in_xy) {
+                *dst[c] = lo ? T(0) : (INCR ? incr : zm[c] + incr);
+                if (hi)
+                    dst[c][c == 0 ? 1 : (c == 1 ? g.ext[1][0] : g.ext[2][0] * g.ext[2][1])] = T(0);
+            }
+            dst[c] += g.ext[c][0] * g.ext[c][1];
+        }
+        const int qn = (int)(qm - (sm + (y + PH) * SX + x + PH));
+        qm = q0;
+        q0 = q1;
+        q1 = q2;
+        q2 = sm + (y + PH) * SX + x + PH + pn;
+        pn = qn;
     }
 }
 
