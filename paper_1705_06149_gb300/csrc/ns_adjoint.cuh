@@ -10,7 +10,7 @@
 // reading it as a mirror), each interface flux weighted by the difference of
 // mu on its two faces.  Every output is written by one thread in a fixed
 // order, so the gradient does not depend on scheduling.  SMART takes the
-// branch the forward kernel took (the same division-free comparisons); a
+// branch the forward kernel took (comparisons equal up to rounding); a
 // flux with zero transporting velocity takes the derivative of its
 // left-upwind form.  T = double (FP64 grids) or float (FP32 storage; the lid
 // derivative and J are summed in FP64).
@@ -329,6 +329,251 @@ __global__ void __launch_bounds__(NTHREADS)
     }
     double v1[1] = {acc};
     write_partials<1>(v1, part + s * 3LL * gridDim.x + (long long)c * gridDim.x + blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// the reverse step from shared memory, and the wide sum
+// ---------------------------------------------------------------------------
+
+// Tile of k_adj_tile: 32 x 4 columns, AT_Z cells along z, halo 3.
+constexpr int AT_Z = 4, AT_H = 3;
+constexpr int AT_SX = TX + 2 * AT_H, AT_SY = TY + 2 * AT_H, AT_SZ = AT_Z + 2 * AT_H;
+constexpr int AT_PLANE = AT_SX * AT_SY, AT_N = AT_PLANE * AT_SZ;
+
+// Where position i of component c along axis d is read from: the stored index,
+// ~index with the ghost rule's sign -1, AT_NONE beyond the two ghosts of a
+// wall.  lid: the ghost adds twice the lid speed.
+constexpr int AT_NONE = -(1 << 30);
+__device__ __forceinline__ int adj_src(const Geo& g, int c, int d, int i, bool& lid) {
+    const int e = g.ext[c][d], n = g.n[d];
+    if (g.bc[d] == BC_PERIODIC) return ((i % e) + e) % e;
+    if (i >= 0 && i < e) return i;
+    if (i < -2 || i > e + 1) return AT_NONE;
+    const bool hi = i >= e;
+    int q;
+    bool neg = true;
+    if (d == c) {
+        q = hi ? 2 * n - i : -i;
+    } else {
+        q = hi ? 2 * n - 1 - i : -i - 1;
+        neg = g.bc[d] == BC_WALL;
+        if (neg && c == 0 && d == 1 && hi) lid = true;
+    }
+    if (q < 0 || q >= e) return AT_NONE;
+    return neg ? ~q : q;
+}
+
+// The same for mu: AT_NONE (zero) outside the stored range and on inactive
+// faces.
+__device__ __forceinline__ int adj_mu_src(const Geo& g, int c, int d, int i) {
+    const int e = g.ext[c][d];
+    if (g.bc[d] == BC_PERIODIC) return ((i % e) + e) % e;
+    if (d == c) return i > 0 && i < g.n[d] ? i : AT_NONE;
+    return i >= 0 && i < e ? i : AT_NONE;
+}
+
+// Face value of a line bb, b, f, ff transported by uf, and its derivatives by
+// the four values: the branch the forward kernel takes (the smallest of 2 |k|,
+// |k|/8 + 3|g|/8 and |g| as in smart_phi).
+template <typename T>
+__device__ __forceinline__ T adj_face(T uf, T bb, T b, T f, T ff, T (&d4)[4]) {
+    const bool neg = uf < T(0);
+    const T U = neg ? ff : bb, C = neg ? f : b, D = neg ? b : f;
+    const T k = C - U, g = D - C;
+    const T q = fma(T(0.375), g, T(0.125) * k);
+    const T ak = fabs(k + k), aq = fabs(q), ag = fabs(g);
+    const bool flat = (k == T(0) && g == T(0)) || (k < T(0) && g > T(0)) || (k > T(0) && g < T(0));
+    const bool steep = !flat && ak <= aq && ak <= ag;
+    const bool down = !flat && !steep && ag <= aq;
+    const bool quick = !flat && !steep && !down;
+    const T dU = steep ? T(-2) : (quick ? T(-0.125) : T(0));
+    const T dC = steep ? T(3) : (quick ? T(0.75) : (down ? T(0) : T(1)));
+    const T dD = quick ? T(0.375) : (down ? T(1) : T(0));
+    d4[0] = neg ? T(0) : dU;
+    d4[1] = neg ? dD : dC;
+    d4[2] = neg ? dC : dD;
+    d4[3] = neg ? dU : T(0);
+    return flat ? C : (steep ? C + (k + k) : (down ? D : C + q));
+}
+
+// lambda = mu + dt (dR/du)^T mu on active faces (zero on wall faces) of a
+// tile, every stored value written once; per-CTA partial sums of
+// (dR/du_lid)^T mu in part_lid[state][cta].  The velocity with its ghost values
+// and mu (zero outside) are staged once, so an interior value is a fixed set
+// of 16 face evaluations without a boundary rule: interfaces that do not exist
+// have mu differences of zero.  The ghosts that mirror a value add their part
+// in the threads next to a wall.  Bound: instruction issue (each face is
+// evaluated by the values that read it).  64^3, one state, FP32: 305 us
+// gathering from global memory with the rules at every read -> 92 us.
+template <typename T>
+__global__ void __launch_bounds__(NTHREADS)
+    k_adj_tile(Geo g, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ w,
+               const T* __restrict__ mu_u, const T* __restrict__ mu_v, const T* __restrict__ mu_w,
+               T* __restrict__ lu, T* __restrict__ lv, T* __restrict__ lw, double dt, int tbx,
+               int tby, double* __restrict__ part_lid) {
+    extern __shared__ __align__(16) unsigned char asm_raw[];
+    T* sv = reinterpret_cast<T*>(asm_raw);  // [3][AT_SZ][AT_SY][AT_SX]
+    T* sm = sv + 3 * AT_N;                  // the same of mu
+    __shared__ int zv[3][AT_SZ], zu[3][AT_SZ];
+    const long long s = blockIdx.y;
+    const T* const vel3[3] = {u + s * g.cnt[0], v + s * g.cnt[1], w + s * g.cnt[2]};
+    const T* const mu3[3] = {mu_u + s * g.cnt[0], mu_v + s * g.cnt[1], mu_w + s * g.cnt[2]};
+    T* const out[3] = {lu + s * g.cnt[0], lv + s * g.cnt[1], lw + s * g.cnt[2]};
+    const int cta = blockIdx.x, r = cta / tbx, tz = r / tby;
+    const int i0 = (cta - r * tbx) * TX, j0 = (r - tz * tby) * TY, k0 = tz * AT_Z;
+    const int t = tid_flat();
+    for (int q = t; q < 3 * AT_SZ; q += NTHREADS) {
+        const int c = q / AT_SZ, z = q - c * AT_SZ;
+        bool lid = false;
+        zv[c][z] = adj_src(g, c, 2, k0 - AT_H + z, lid);
+        zu[c][z] = adj_mu_src(g, c, 2, k0 - AT_H + z);
+    }
+    __syncthreads();
+    const T lid2 = T(2.0 * g.u_lid);
+    for (int pq = t; pq < AT_PLANE; pq += NTHREADS) {
+        const int py = pq / AT_SX, px = pq - py * AT_SX;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const int e0 = g.ext[c][0];
+            const long long plane = (long long)e0 * g.ext[c][1];
+            bool lid = false;
+            const int qi = adj_src(g, c, 0, i0 - AT_H + px, lid);
+            const int qj = adj_src(g, c, 1, j0 - AT_H + py, lid);
+            const int mi = adj_mu_src(g, c, 0, i0 - AT_H + px);
+            const int mj = adj_mu_src(g, c, 1, j0 - AT_H + py);
+            const bool ok = qi != AT_NONE && qj != AT_NONE, mok = mi >= 0 && mj >= 0;
+            const bool nxy = (qi < 0) != (qj < 0);
+            const int o = ok ? (qj < 0 ? ~qj : qj) * e0 + (qi < 0 ? ~qi : qi) : 0;
+            const int m = mok ? mj * e0 + mi : 0;
+#pragma unroll
+            for (int z = 0; z < AT_SZ; ++z) {
+                const int a = zv[c][z], b = zu[c][z];
+                T x = T(0);
+                if (ok && a != AT_NONE) {
+                    x = vel3[c][(a < 0 ? ~a : a) * plane + o];
+                    if (nxy != (a < 0)) x = -x;
+                    if (lid) x += lid2;
+                }
+                sv[c * AT_N + z * AT_PLANE + pq] = x;
+                sm[c * AT_N + z * AT_PLANE + pq] =
+                    (mok && b >= 0) ? mu3[c][b * plane + m] : T(0);
+            }
+        }
+    }
+    __syncthreads();
+    constexpr int strd[3] = {1, AT_SX, AT_PLANE};
+    const T inv_re = g_inv_re<T>(g), tdt = T(dt);
+    const int x0 = (int)threadIdx.x, y0 = (int)threadIdx.y;
+    double dl = 0.0;
+    if (i0 + x0 < g.n[0] && j0 + y0 < g.n[1]) {
+        const int zn = min(AT_Z, g.n[2] - k0);
+        for (int z = 0; z < zn; ++z) {
+            const int f[3] = {i0 + x0, j0 + y0, k0 + z};
+            const int o = ((z + AT_H) * AT_SY + y0 + AT_H) * AT_SX + x0 + AT_H;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const T* a = sv + c * AT_N + o;
+                const T* mc = sm + c * AT_N + o;
+                T acc = T(0);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const int sd = strd[d];
+                    const T ih = g_ih<T>(g, d), kd = inv_re * g_ih2<T>(g, d);
+                    acc += kd * (mc[sd] - T(2) * mc[0] + mc[-sd]);
+                    // the ghosts that mirror this value, as offsets from it
+                    // (0: none): beyond the low and the high wall
+                    int lo = 0, hi = 0;
+                    T sg = T(-1);
+                    const int n = g.n[d], x = f[d];
+                    if (g.bc[d] != BC_PERIODIC) {
+                        if (d == c) {
+                            if (x == 1) lo = -2;
+                            if (x == n - 1) hi = 2;
+                        } else {
+                            if (g.bc[d] == BC_SLIP) sg = T(1);
+                            if (x <= 1) lo = -2 * x - 1;
+                            if (x >= n - 2) hi = 2 * (n - x) - 1;
+                        }
+                    }
+                    const bool lid = c == 0 && d == 1 && g.bc[1] == BC_WALL;
+                    T top = T(0);  // the high ghost's part, before its sign
+                    if (d != c) {
+                        if (lo == -1) acc += sg * kd * mc[0];
+                        if (hi == 1) top += kd * mc[0];
+                    }
+#pragma unroll
+                    for (int q = -2; q <= 1; ++q) {
+                        // interface between the values at q and q + 1
+                        const T nu = (mc[(q + 1) * sd] - mc[q * sd]) * ih;
+                        const T b = a[q * sd], fw = a[(q + 1) * sd];
+                        const T* tr = sv + d * AT_N + o + (q + 1) * sd;
+                        const T uf = d == c ? T(0.5) * (b + fw) : T(0.5) * (tr[-strd[c]] + tr[0]);
+                        T d4[4];
+                        const T phi = adj_face(uf, a[(q - 1) * sd], b, fw, a[(q + 2) * sd], d4);
+                        T wt = uf * d4[1 - q];
+                        if (d == c && (q == 0 || q == -1)) wt += T(0.5) * phi;
+                        acc += nu * wt;
+                        if (lo != 0) {
+                            const int role = lo - q + 1;
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (role == e) acc += sg * (nu * (uf * d4[e]));
+                        }
+                        if (hi != 0) {
+                            const int role = hi - q + 1;
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (role == e) top += nu * (uf * d4[e]);
+                        }
+                    }
+                    acc += sg * top;
+                    if (lid && hi != 0) dl += 2.0 * double(top);
+                }
+                // as the transport of the other components along c
+                const int sc = strd[c];
+                const T ih = g_ih<T>(g, c);
+#pragma unroll
+                for (int c2 = 0; c2 < 3; ++c2) {
+                    if (c2 == c) continue;
+                    const int s2 = strd[c2];
+#pragma unroll
+                    for (int cand = 0; cand < 2; ++cand) {
+                        const int at = o - sc + (cand ? s2 : 0);  // the interface's low value
+                        const T* l = sv + c2 * AT_N + at;
+                        const T* m2 = sm + c2 * AT_N + at;
+                        const T nu = (m2[sc] - m2[0]) * ih;
+                        const T* tr = sv + c * AT_N + at + sc;
+                        const T uf = T(0.5) * (tr[-s2] + tr[0]);
+                        T d4[4];
+                        acc += T(0.5) * nu * adj_face(uf, l[-sc], l[0], l[sc], l[2 * sc], d4);
+                    }
+                }
+                const long long id = vindex(g, c, f[0], f[1], f[2]);
+                const bool wall = g.bc[c] != BC_PERIODIC;
+                out[c][id] = (wall && f[c] == 0) ? T(0) : mc[0] + tdt * acc;
+                if (wall && f[c] == g.n[c] - 1) {
+                    int h[3] = {f[0], f[1], f[2]};
+                    h[c] += 1;
+                    out[c][vindex(g, c, h[0], h[1], h[2])] = T(0);
+                }
+            }
+        }
+    }
+    double v1[1] = {dl};
+    write_partials<1>(v1, part_lid + s * (long long)gridDim.x + blockIdx.x);
+}
+
+// out[s] (+)= sum of part[s][0..n-1], one CTA per state, in a fixed order.
+// One thread per state (k_adj_sum) reads its partials one after another, 279
+// us for 5000; up to ADJ_SERIAL_SUM of them it is as fast.
+constexpr int ADJ_SERIAL_SUM = 32;
+__global__ void __launch_bounds__(NTHREADS)
+    k_adj_sum_block(const double* __restrict__ part, int n, double* __restrict__ out, int add) {
+    const int s = blockIdx.x;
+    double v[1] = {0.0};
+    for (int q = tid_flat(); q < n; q += NTHREADS) v[0] += part[(long long)s * n + q];
+    block_sum<1>(v);
+    if (tid_flat() == 0) out[s] = add ? out[s] + v[0] : v[0];
 }
 
 }  // namespace nsk

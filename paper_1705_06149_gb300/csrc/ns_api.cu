@@ -2470,6 +2470,16 @@ ns_status parareal_impl(ns_grid* g, ns_state u0, ns_state slices, int N, int S, 
     return sync_stream(g);
 }
 
+// out[s] (+)= the sum of state s's n partials.
+void adj_sum(ns_grid* g, const double* part, int n, int batch, double* out, int add) {
+    if (n > ADJ_SERIAL_SUM)
+        NS_LAUNCH(g, NS_K_ADJOINT, 0,
+                  k_adj_sum_block<<<batch, block_dim(), 0, g->stream>>>(part, n, out, add));
+    else
+        NS_LAUNCH(g, NS_K_ADJOINT, 0,
+                  k_adj_sum<<<ceil_div(batch, 32), 32, 0, g->stream>>>(part, n, batch, out, add));
+}
+
 // Reverse mode through nsteps fine steps with checkpoints of (u, p) every
 // ckpt_every steps: forward once storing checkpoints, then per segment (last
 // first) recompute its states from the checkpoint and run the adjoint steps
@@ -2515,10 +2525,22 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
     double* pmu = (double*)alloc(sizeof(double) * np);  // phi of the adjoint projections
     double* dJ = (double*)alloc(sizeof(double) * 2 * B);
     double* part_J = (double*)alloc(sizeof(double) * 3 * tblocks * B);
-    // (dR/du)^T mu: 32 x 4 column tiles over the face extents, ADJ_TZ
-    // positions along z per thread, one grid z-slice per component
+    // the reverse step: tiles of 32 x 4 x AT_Z cells; FP64 calls whose tiles
+    // would leave half the SMs idle, the gather (32 x 4 column tiles over the
+    // face extents, ADJ_TZ positions along z per thread, one grid z-slice per
+    // component).  A gradient over 10 steps, gather -> tiles: 16^3 FP64 (16
+    // tiles) 5.4 -> 6.0 ms, FP32 4.9 -> 4.3; 48 x 40 x 36 FP64 11.4 -> 10.1;
+    // 64^3 FP32 9.1 -> 6.5, FP64 22.5 -> 16.8.
+    const int atx = ceil_div(G.n[0], TX), aty = ceil_div(G.n[1], TY);
+    const int tile_ctas = atx * aty * ceil_div(G.n[2], AT_Z);
+    const size_t tile_smem = 6 * (size_t)AT_N * sizeof(T);
+    const bool tiled = sizeof(T) == 4 || (long long)tile_ctas * B >= 76;
+    if (tiled && cudaFuncSetAttribute(k_adj_tile<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)tile_smem) != cudaSuccess)
+        return fail(NS_ERR_CUDA, "ns_adjoint: shared memory attribute");
     const int adj_ctas = G.fbx * G.fby * ceil_div(G.n[2] + 1, ADJ_TZ);
-    double* part_lid = (double*)alloc(sizeof(double) * 3 * adj_ctas * B);
+    const int lid_parts = tiled ? tile_ctas : 3 * adj_ctas;
+    double* part_lid = (double*)alloc(sizeof(double) * lid_parts * B);
     if (mine.size() != 12) {
         release();
         return fail(NS_ERR_OOM, "ns_adjoint: workspace allocation failed");
@@ -2556,8 +2578,7 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
                       k_adj_terminal<T><<<dim3(tblocks, B), block_dim(), 0, g->stream>>>(
                           G, c, cur + off, lam + off, part_J, vol));
         }
-        NS_LAUNCH(g, NS_K_ADJOINT, 0,
-                  k_adj_sum<<<(B + 31) / 32, 32, 0, g->stream>>>(part_J, 3 * tblocks, B, dJ, 0));
+        adj_sum(g, part_J, 3 * tblocks, B, dJ, 0);
         if (cudaGetLastError() != cudaSuccess) st = fail(NS_ERR_CUDA, "ns_adjoint: launch failed");
     }
     // reverse, segment by segment
@@ -2576,23 +2597,32 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
             // each adjoint projection starts from the previous one's phi
             st = project_impl<T>(g, vel_state(mu, pmu), pmu);
             if (st != NS_OK) break;
-            // acc = (dR/du)^T mu at u^n, dJ/du_lid += dt (dR/du_lid)^T mu
+            // lambda = mu + dt (dR/du)^T mu at u^n (active faces), dJ/du_lid +=
+            // dt (dR/du_lid)^T mu (dt at the end)
             T* un = seg + (size_t)(n - n0) * vel_elems;
-            NS_LAUNCH(g, NS_K_ADJOINT, 0,
-                      k_adj_rhs<T><<<dim3(adj_ctas, B, 3), block_dim(), 0, g->stream>>>(
-                          G, un, un + nv[0], un + nv[0] + nv[1], mu, mu + nv[0],
-                          mu + nv[0] + nv[1], acc, acc + nv[0], acc + nv[0] + nv[1], part_lid));
-            NS_LAUNCH(g, NS_K_ADJOINT, 0,
-                      k_adj_sum<<<(B + 31) / 32, 32, 0, g->stream>>>(part_lid, 3 * adj_ctas, B,
-                                                                    dJ + B, 1));
-            // lambda = mu + dt acc (active faces); acc <- 0
-            for (int c = 0; c < 3; ++c) {
-                const size_t off = c == 0 ? 0 : (c == 1 ? nv[0] : nv[0] + nv[1]);
-                const int blocks = (int)std::min<long long>(((long long)nv[c] + 255) / 256, 4096);
+            if (tiled) {
                 NS_LAUNCH(g, NS_K_ADJOINT, 0,
-                          k_adj_finish<T><<<blocks, 256, 0, g->stream>>>(
-                              G, c, (long long)nv[c], mu + off, acc + off, lam + off, dt));
+                          k_adj_tile<T><<<dim3(tile_ctas, B), block_dim(), tile_smem, g->stream>>>(
+                              G, un, un + nv[0], un + nv[0] + nv[1], mu, mu + nv[0],
+                              mu + nv[0] + nv[1], lam, lam + nv[0], lam + nv[0] + nv[1], dt, atx,
+                              aty, part_lid));
+            } else {
+                NS_LAUNCH(g, NS_K_ADJOINT, 0,
+                          k_adj_rhs<T><<<dim3(adj_ctas, B, 3), block_dim(), 0, g->stream>>>(
+                              G, un, un + nv[0], un + nv[0] + nv[1], mu, mu + nv[0],
+                              mu + nv[0] + nv[1], acc, acc + nv[0], acc + nv[0] + nv[1],
+                              part_lid));
+                // (acc <- 0)
+                for (int c = 0; c < 3; ++c) {
+                    const size_t off = c == 0 ? 0 : (c == 1 ? nv[0] : nv[0] + nv[1]);
+                    const int blocks =
+                        (int)std::min<long long>(((long long)nv[c] + 255) / 256, 4096);
+                    NS_LAUNCH(g, NS_K_ADJOINT, 0,
+                              k_adj_finish<T><<<blocks, 256, 0, g->stream>>>(
+                                  G, c, (long long)nv[c], mu + off, acc + off, lam + off, dt));
+                }
             }
+            adj_sum(g, part_lid, lid_parts, B, dJ + B, 1);
             if (cudaGetLastError() != cudaSuccess)
                 st = fail(NS_ERR_CUDA, "ns_adjoint: launch failed");
         }
@@ -3047,8 +3077,7 @@ ns_status ns_kinetic_energy(ns_grid* grid, ns_state state, double* J) {
                 G, c, (const double*)vel[c], nullptr, part, vol);
         grid->stats.launches += 1;
     }
-    k_adj_sum<<<(B + 31) / 32, 32, 0, grid->stream>>>(part, 3 * tblocks, B, dJ, 0);
-    grid->stats.launches += 1;
+    adj_sum(grid, part, 3 * tblocks, B, dJ, 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(J, dJ, sizeof(double) * B, cudaMemcpyDeviceToHost, grid->stream);
