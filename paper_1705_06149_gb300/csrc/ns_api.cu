@@ -473,6 +473,24 @@ bool cluster_ready(ns_grid* g) {
     return cudaOccupancyMaxActiveClusters(&n, k_mg_cluster<T>, &cfg) == cudaSuccess && n >= 1;
 }
 
+// Calls f with the rows and columns per thread of k_dir_xy as constants.
+template <typename F>
+void with_dir_shape(int rb, int ncol, F&& f) {
+    using std::integral_constant;
+    using One = integral_constant<int, 1>;
+    using Two = integral_constant<int, 2>;
+    if (rb == 16)
+        f(integral_constant<int, 16>{}, Two{});
+    else if (rb == 8 && ncol == 2)
+        f(integral_constant<int, 8>{}, Two{});
+    else if (rb == 8)
+        f(integral_constant<int, 8>{}, One{});
+    else if (ncol == 2)
+        f(integral_constant<int, 4>{}, Two{});
+    else
+        f(integral_constant<int, 4>{}, One{});
+}
+
 template <typename T>
 ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
     const Geo& G = g->geo;
@@ -489,12 +507,27 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
     P.ly[0] = t + off[2];
     P.ly[1] = t + off[3];
     P.col = t + off[4];
-    g->dir_smem = dir_smem_elems(P) * sizeof(T);
-    if (cudaFuncSetAttribute(k_dir_xy<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)DIR_MAX_SMEM) != cudaSuccess ||
-        cudaFuncSetAttribute(k_dir_xy<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)DIR_MAX_SMEM) != cudaSuccess)
-        return fail(NS_ERR_CUDA, "ns_create_grid: direct solve shared memory attribute");
+    bool ok = true;
+    auto most = [&](auto kernel, size_t elems) {
+        ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)(elems * sizeof(T))) == cudaSuccess;
+    };
+    // the whole of an SM's, whatever this grid needs: the attribute belongs to
+    // the kernel, not to the grid
+    constexpr size_t all = DIR_MAX_SMEM / sizeof(T);
+    if (P.lines) {
+        most(k_dir_x<T, false>, all);
+        most(k_dir_x<T, true>, all);
+        most(k_dir_y<T, false>, all);
+        most(k_dir_y<T, true>, all);
+    } else {
+        g->dir_smem = dir_smem_elems(P) * sizeof(T);
+        with_dir_shape(P.rb, P.ncol, [&](auto rb, auto nc) {
+            most(k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value>, all);
+            most(k_dir_xy<T, true, decltype(rb)::value, decltype(nc)::value>, all);
+        });
+    }
+    if (!ok) return fail(NS_ERR_CUDA, "ns_create_grid: direct solve shared memory attribute");
     g->dir = true;
     g->mg = true;
     if (sizeof(T) == 4) {
@@ -829,6 +862,16 @@ template <> const DirPlan<double>& dirplan<double>(const ns_grid* g) { return g-
 
 long long dir_stride(const ns_grid* g) { return (long long)g->geo.cnt[3] * g->cap; }
 
+template <typename T>
+void direct_z(ns_grid* g, const DirPlan<T>& P, T* spec, dim3 zg, dim3 zb, long long units) {
+    if (P.zm == DIR_ZC)
+        NS_LAUNCH(g, NS_K_DIRECT_Z, units,
+                  (k_dir_z<T, DIR_ZC><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
+    else
+        NS_LAUNCH(g, NS_K_DIRECT_Z, units,
+                  (k_dir_z<T, DIR_ZC_LONG><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
+}
+
 // e = L^-1 r for every active state: FP32+refine from the residual's high
 // part into the application's slot of the ring, FP64 from kv[1] into kv[4];
 // the spectral planes in kv[3].
@@ -843,16 +886,35 @@ void direct_apply(ns_grid* g, int batch) {
     const dim3 pg(P.nz * P.xb, batch), zg(ceil_div(P.nx * P.ny, DIR_ZX), batch);
     const dim3 zb(DIR_ZX, P.zc);
     const long long units = P.cells * batch;
-    NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-              (k_dir_xy<T, false><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, r, spec, 0)));
-    if (P.zm == DIR_ZC)
-        NS_LAUNCH(g, NS_K_DIRECT_Z, units,
-                  (k_dir_z<T, DIR_ZC><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
-    else
-        NS_LAUNCH(g, NS_K_DIRECT_Z, units,
-                  (k_dir_z<T, DIR_ZC_LONG><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
-    NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-              (k_dir_xy<T, true><<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, spec, e, ring)));
+    if (P.lines) {
+        const unsigned gx = (unsigned)std::min<long long>(
+            152, (long long)ceil_div(P.ny * P.nz, P.lines) * batch);
+        const unsigned gy =
+            (unsigned)std::min<long long>(152, (long long)ceil_div(P.nx, P.lines) * P.nz * batch);
+        const size_t sx = dir_x_elems(P) * sizeof(T), sy = dir_y_elems(P) * sizeof(T);
+        NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+                  (k_dir_x<T, false><<<gx, P.ntx, sx, g->stream>>>(P, g->ctl, r, spec, 0, batch)));
+        NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+                  (k_dir_y<T, false><<<gy, P.nty, sy, g->stream>>>(P, g->ctl, spec, batch)));
+        direct_z<T>(g, P, spec, zg, zb, units);
+        NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+                  (k_dir_y<T, true><<<gy, P.nty, sy, g->stream>>>(P, g->ctl, spec, batch)));
+        NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+                  (k_dir_x<T, true><<<gx, P.ntx, sx, g->stream>>>(P, g->ctl, spec, e, ring,
+                                                                 batch)));
+        return;
+    }
+    with_dir_shape(P.rb, P.ncol, [&](auto rb, auto nc) {
+        NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+                  (k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value>
+                   <<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, r, spec, 0)));
+    });
+    direct_z<T>(g, P, spec, zg, zb, units);
+    with_dir_shape(P.rb, P.ncol, [&](auto rb, auto nc) {
+        NS_LAUNCH(g, NS_K_DIRECT_XY, units,
+                  (k_dir_xy<T, true, decltype(rb)::value, decltype(nc)::value>
+                   <<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, spec, e, ring)));
+    });
 }
 
 // One application of the direct solve and the correction with it, on every
@@ -1792,7 +1854,10 @@ ns_status parareal_update(ns_grid* g, const void* const fy[4], const void* const
 
 // Kernels one preconditioned iteration launches (mg_apply twice + 3).
 long long mg_iteration_launches(const ns_grid* g) {
-    if (g->dir) return g->fp32 ? 3 : 4;  // the correction counts with FP32+refine's
+    if (g->dir) {  // the correction counts with FP32+refine's
+        const bool lines = g->fp32 ? g->dirf.lines > 0 : g->dird.lines > 0;
+        return (lines ? 5 : 3) + (g->fp32 ? 0 : 1);
+    }
     const int lc = g->plan.lc;
     const long long apply = 1 + lc + std::max(lc - 1, 0) + 1 + lc;
     return 2 * apply + 3;

@@ -39,10 +39,14 @@ template <typename T>
 struct DirPlan {
     int nx, ny, nz, per_z;
     int hx, hy;    // even modes (= length of the folded line) along x, y
-    int hxp, hyp;  // the same rounded up to 4
-    int ldx, ldy;  // shared-memory row strides of the folded plane / the y matrix
+    int hxp;       // hx rounded up to 4
+    int rb, ncol;  // rows and columns per thread of k_dir_xy
+    int hyp;       // hy rounded up to rb
+    int ldf;       // column stride of the folded plane in shared memory
     int cb, xb;    // columns per CTA (of a half), CTAs per plane
     int nt;        // threads of k_dir_xy
+    int lines;     // > 0: one axis at a time, lines per block of k_dir_x / k_dir_y
+    int ntx, nty;  // their threads
     int zm, zc;    // k_dir_z: cells per chunk, chunks per column
     long long cells;
     const T* rx[2];  // x matrices, forward and inverse: [parity][hxp][hxp]
@@ -86,40 +90,55 @@ template <> __device__ __forceinline__ int dir_slot<float>(const SliceCtl* c) {
 }
 template <> __device__ __forceinline__ int dir_slot<double>(const SliceCtl*) { return 0; }
 
-// acc[i][j] += sum_k L[i rs][k] R[k][j], i, j < 4, k ascending (K a multiple
-// of 4; rows of L are rs apart so that neighbouring threads read
-// neighbouring rows).
-template <typename T>
-__device__ __forceinline__ void dir_tile(const T* L, int rs, const T* R, int ldr, int K,
-                                         T (&acc)[4][4]) {
-    for (int k = 0; k < K; k += 4) {
-        Q4<T> l[4];
+// acc[n][i] += sum_k L[k][i] R[k][n dc], i < RB, n < NC, k ascending; rows of L
+// (16-byte aligned) are ldl apart, of R ldr.  Neighbouring threads hold
+// neighbouring columns of R, so the reads of L are broadcasts and those of R
+// without conflict: RB / 4 + NC shared-memory cycles per RB NC products of a
+// warp (four per cycle and SM).
+template <typename T, int RB, int NC>
+__device__ __forceinline__ void dir_cols(const T* L, int ldl, const T* R, int ldr, int dc, int K,
+                                         T (&acc)[NC][RB]) {
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        T r[NC];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) l[i] = q4_ld<T>(L + i * rs + k);
+        for (int n = 0; n < NC; ++n) r[n] = R[n * dc];
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            const Q4<T> r = q4_ld<T>(R + (k + kk) * ldr);
+        for (int b = 0; b < RB / 4; ++b) {
+            const Q4<T> l = q4_ld<T>(L + 4 * b);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(l[i].v[kk], r.v[j], acc[i][j]);
+                for (int n = 0; n < NC; ++n)
+                    acc[n][4 * b + q] = fma(l.v[q], r[n], acc[n][4 * b + q]);
         }
+        L += ldl;
+        R += ldr;
     }
 }
 
+// Copies n elements (a multiple of 4, both sides 16-byte aligned) to shared
+// memory.
+template <typename T>
+__device__ __forceinline__ void dir_copy(T* d, const T* __restrict__ g, int n, int t, int nt) {
+    for (int q = 4 * t; q < n; q += 4 * nt) q4_st<T>(d + q, q4_ld<T>(g + q));
+}
+
 // Shared memory of k_dir_xy in elements: x matrices of the column block, y
-// matrices, the folded plane, the product of the first stage.
+// matrices, the folded plane (columns of rows), the product of the first stage.
 template <typename T>
 inline size_t dir_smem_elems(const DirPlan<T>& P) {
-    return 2 * (size_t)P.hxp * P.cb + 2 * (size_t)P.hyp * P.ldy + 4 * (size_t)P.hyp * P.ldx +
+    return 2 * (size_t)P.hxp * P.cb + 2 * (size_t)P.hyp * P.hyp + 4 * (size_t)P.hxp * P.ldf +
            4 * (size_t)P.hyp * P.cb;
 }
 
 // Forward (INV false): src [nz][ny][nx] cells -> dst [nz][ky][kx].  Inverse:
 // src [nz][ky][kx] -> dst cells (FP32: the application's slot of the ring,
 // slots `ring` elements apart).  blockIdx.x = plane and column block,
-// blockIdx.y = state.
-template <typename T, bool INV>
+// blockIdx.y = state.  Bound by instruction issue (FP64: by the FP64 pipe).
+// 64^3 x 32 states, FP32: 57 us with 4 x 4 tiles of operands both read per
+// thread -> 46 us.
+template <typename T, bool INV, int RB, int NC>
 __global__ void __launch_bounds__(DIR_MAX_THREADS)
     k_dir_xy(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const T* __restrict__ src,
              T* __restrict__ dst, long long ring) {
@@ -129,111 +148,112 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const T scale = dir_scale<T>(ctl + s, INV);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, ny = P.ny, hx = P.hx, hy = P.hy, hxp = P.hxp, hyp = P.hyp;
-    const int ldx = P.ldx, ldy = P.ldy, cb = P.cb;
+    const int ldf = P.ldf, cb = P.cb;
     T* R = reinterpret_cast<T*>(smem_raw);
     T* Lm = R + 2 * hxp * cb;
-    T* F = Lm + 2 * hyp * ldy;
-    T* T1 = F + 4 * hyp * ldx;
+    T* F = Lm + 2 * hyp * hyp;
+    T* T1 = F + 4 * hxp * ldf;
     const int z = (int)blockIdx.x / P.xb;
     const int c0 = ((int)blockIdx.x - z * P.xb) * cb;
     const int t = (int)threadIdx.x, nt = (int)blockDim.x;
     const T* __restrict__ a = src + s * P.cells + (long long)z * nx * ny;
     T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s) * ring : 0) + s * P.cells +
                         (long long)z * nx * ny;
-    {
-        // the plane: thread (row, column j) of a pass; rows and columns beyond
-        // the halves are zero
-        const int rpp = nt / hxp, y0 = t / hxp, j = t - y0 * hxp;
-        if (y0 < rpp) {
-#pragma unroll 4
-            for (int y = y0; y < hyp; y += rpp) {
-                T q[4] = {T(0), T(0), T(0), T(0)};  // (y, x) parity: ee, eo, oe, oo
-                if (!INV) {
-                    if (y < hy && j < hx) {
-                        const int ym = ny - 1 - y, xm = nx - 1 - j;
-                        const T a00 = a[y * nx + j];
-                        const T a01 = xm != j ? a[y * nx + xm] : T(0);
-                        const T a10 = ym != y ? a[ym * nx + j] : T(0);
-                        const T a11 = (xm != j && ym != y) ? a[ym * nx + xm] : T(0);
-                        // the middle of an odd extent: itself in the sum, zero
-                        // in the difference
-                        const T e0 = a00 + a01, o0 = xm != j ? a00 - a01 : T(0);
-                        const T e1 = a10 + a11, o1 = xm != j ? a10 - a11 : T(0);
-                        q[0] = e0 + e1;
-                        q[1] = o0 + o1;
-                        q[2] = ym != y ? e0 - e1 : T(0);
-                        q[3] = ym != y ? o0 - o1 : T(0);
-                    }
-                } else {
-                    const bool ye = y < hy, yo = y < ny - hy, xe = j < hx, xo = j < nx - hx;
-                    if (ye && xe) q[0] = a[y * nx + j];
-                    if (ye && xo) q[1] = a[y * nx + hx + j];
-                    if (yo && xe) q[2] = a[(hy + y) * nx + j];
-                    if (yo && xo) q[3] = a[(hy + y) * nx + hx + j];
-                }
+    // the plane: four rows of one column at a time (F[quadrant][column][row]);
+    // rows and columns beyond the halves are zero
+    for (int w = t; w < hxp * (hyp / 4); w += nt) {
+        const int y0 = 4 * (w / hxp), j = w - (y0 / 4) * hxp;
+        // (loads without conditions, so that they are issued together)
+        const int jj = min(j, hx - 1), xm = INV ? hx + min(jj, nx - hx - 1) : nx - 1 - jj;
+        Q4<T> q[4];  // (y, x) parity: ee, eo, oe, oo
 #pragma unroll
-                for (int h = 0; h < 4; ++h)
-                    F[(h * hyp + y) * ldx + j] = INV ? q[h] : q[h] * scale;
+        for (int r = 0; r < 4; ++r) {
+            const int y = min(y0 + r, hy - 1), ym = INV ? hy + min(y, ny - hy - 1) : ny - 1 - y;
+            q[0].v[r] = a[y * nx + jj];
+            q[1].v[r] = a[y * nx + xm];
+            q[2].v[r] = a[ym * nx + jj];
+            q[3].v[r] = a[ym * nx + xm];
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int y = y0 + r;
+            const bool ye = y < hy, xe = j < hx;
+            if (!INV) {
+                // the middle of an odd extent: itself in the sum, zero in the
+                // difference
+                const bool xp = xm != jj, yp = ny - 1 - y != y;
+                const T a00 = q[0].v[r], a01 = q[1].v[r], a10 = q[2].v[r], a11 = q[3].v[r];
+                const T e0 = xp ? a00 + a01 : a00, o0 = xp ? a00 - a01 : T(0);
+                const T e1 = xp ? a10 + a11 : a10, o1 = xp ? a10 - a11 : T(0);
+                const bool in = ye && xe;
+                q[0].v[r] = in ? scale * (yp ? e0 + e1 : e0) : T(0);
+                q[1].v[r] = in ? scale * (yp ? o0 + o1 : o0) : T(0);
+                q[2].v[r] = in && yp ? scale * (e0 - e1) : T(0);
+                q[3].v[r] = in && yp ? scale * (o0 - o1) : T(0);
+            } else {
+                const bool yo = y < ny - hy, xo = j < nx - hx;
+                if (!(ye && xe)) q[0].v[r] = T(0);
+                if (!(ye && xo)) q[1].v[r] = T(0);
+                if (!(yo && xe)) q[2].v[r] = T(0);
+                if (!(yo && xo)) q[3].v[r] = T(0);
             }
         }
-        // the matrices
-        const T* __restrict__ rx = P.rx[INV ? 1 : 0];
-        const T* __restrict__ ly = P.ly[INV ? 1 : 0];
-        const int cq = cb / 4, yq = hyp / 4;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) q4_st<T>(F + (h * hxp + j) * ldf + y0, q[h]);
+    }
+    // the matrices (the broadcast one by columns: the other direction's rows)
+    const T* __restrict__ rx = P.rx[INV ? 1 : 0];
+    dir_copy<T>(Lm, P.ly[INV ? 0 : 1], 2 * hyp * hyp, t, nt);
+    if (cb == hxp) {
+        dir_copy<T>(R, rx, 2 * hxp * hxp, t, nt);
+    } else {
+        const int cq = cb / 4;
         for (int q = t; q < 2 * hxp * cq; q += nt) {
             const int row = q / cq, c = 4 * (q - row * cq);
             Q4<T> v{{T(0), T(0), T(0), T(0)}};
             if (c0 + c < hxp) v = q4_ld<T>(rx + row * hxp + c0 + c);
             q4_st<T>(R + row * cb + c, v);
         }
-        for (int q = t; q < 2 * hyp * yq; q += nt) {
-            const int row = q / yq, c = 4 * (q - row * yq);
-            q4_st<T>(Lm + row * ldy + c, q4_ld<T>(ly + row * hyp + c));
-        }
     }
     __syncthreads();
-    const int nty = hyp / 4, ntx = cb / 4, tiles = 4 * nty * ntx;
-    // along x: T1[q][row][c] = sum_j F[q][row][j] R[px][j][c]
-    for (int w = t; w < tiles; w += nt) {
-        const int r = w / nty, mr = w - r * nty, q = r / ntx, nc = r - q * ntx;
-        T acc[4][4] = {};
-        dir_tile<T>(F + (q * hyp + mr) * ldx, nty * ldx, R + (q & 1) * hxp * cb + 4 * nc, cb, hxp,
-                    acc);
+    // A thread holds RB rows of NC columns (dc apart) of a quadrant: w = (row
+    // block, quadrant, column).
+    const int dc = cb / NC, cols = 4 * dc, items = cols * (hyp / RB);
+    // along x: T1[q][row][c] = sum_j F[q][j][row] R[px][j][c]
+    for (int w = t; w < items; w += nt) {
+        const int rb = w / cols, fc = w - rb * cols, q = fc / dc, c = fc - q * dc;
+        T acc[NC][RB] = {};
+        dir_cols<T, RB, NC>(F + q * hxp * ldf + rb * RB, ldf, R + (q & 1) * hxp * cb + c, cb, dc,
+                            hx, acc);
+        T* d = T1 + (q * hyp + rb * RB) * cb + c;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            q4_st<T>(T1 + (q * hyp + mr + i * nty) * cb + 4 * nc,
-                     Q4<T>{{acc[i][0], acc[i][1], acc[i][2], acc[i][3]}});
+        for (int i = 0; i < RB; ++i)
+#pragma unroll
+            for (int n = 0; n < NC; ++n) d[i * cb + n * dc] = acc[n][i];
     }
     __syncthreads();
-    // along y: out[q][row][c] = sum_y Lm[py][row][y] T1[q][y][c]
-    for (int w = t; w < tiles; w += nt) {
-        const int r = w / nty, mr = w - r * nty, q = r / ntx, nc = r - q * ntx;
-        T acc[4][4] = {};
-        dir_tile<T>(Lm + ((q >> 1) * hyp + mr) * ldy, nty * ldy, T1 + q * hyp * cb + 4 * nc, cb,
-                    hyp, acc);
+    // along y: out[q][row][c] = sum_y Lm[py][y][row] T1[q][y][c]
+    for (int w = t; w < items; w += nt) {
+        const int rb = w / cols, fc = w - rb * cols, q = fc / dc, c = fc - q * dc;
+        T acc[NC][RB] = {};
+        dir_cols<T, RB, NC>(Lm + (q >> 1) * hyp * hyp + rb * RB, hyp, T1 + q * hyp * cb + c, cb,
+                            dc, hy, acc);
         if (INV) {
             // (the folded plane is no longer read)
+            T* d = F + (q * hyp + rb * RB) * cb + c;
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                q4_st<T>(F + (q * hyp + mr + i * nty) * cb + 4 * nc,
-                         Q4<T>{{acc[i][0], acc[i][1], acc[i][2], acc[i][3]}});
+            for (int i = 0; i < RB; ++i)
+#pragma unroll
+                for (int n = 0; n < NC; ++n) d[i * cb + n * dc] = acc[n][i];
         } else {
             const int cy = (q >> 1) ? ny - hy : hy, cx = (q & 1) ? nx - hx : hx;
             const int oy = (q >> 1) ? hy : 0, ox = (q & 1) ? hx : 0;
-            const int c = c0 + 4 * nc;
+            T* d = o + (oy + rb * RB) * nx + ox + c0 + c;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int ky = mr + i * nty;
-                if (ky >= cy) continue;
-                T* row = o + (oy + ky) * nx + ox + c;
-                if (c + 4 <= cx && ((nx | hx) & 3) == 0) {
-                    q4_st<T>(row, Q4<T>{{acc[i][0], acc[i][1], acc[i][2], acc[i][3]}});
-                } else {
+            for (int i = 0; i < RB; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (c + j < cx) row[j] = acc[i][j];
-                }
-            }
+                for (int n = 0; n < NC; ++n)
+                    if (rb * RB + i < cy && c0 + c + n * dc < cx) d[i * nx + n * dc] = acc[n][i];
         }
     }
     if (INV) {
@@ -253,6 +273,172 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
                 if (ym != y) {
                     o[ym * nx + x] = me + mo;
                     if (xm != x) o[ym * nx + xm] = me - mo;
+                }
+            }
+        }
+    }
+}
+
+// Planes too large for one CTA's shared memory: the same transforms one axis at
+// a time, in persistent CTAs that keep the axis's matrices (both parities) in
+// shared memory and run over blocks of P.lines lines.  A thread holds DIR_LRB
+// rows of DIR_LNC columns in both parities, so folding and unfolding need no
+// exchange.  256 x 256 planes, FP32: 128 products per value and axis, bound by
+// the FP32 pipe and the shared-memory reads that feed it (4 of each per 16
+// products): 485 us per axis for 67e6 cells, floor of the pipe alone 221 us
+// (16 rows per thread, half the warps: 545 to 919 us).
+constexpr int DIR_LRB = 8, DIR_LNC = 2;
+
+template <typename T>
+inline size_t dir_x_elems(const DirPlan<T>& P) {
+    return 2 * (size_t)P.hxp * P.hxp + 2 * (size_t)P.hxp * (P.lines + 4);
+}
+template <typename T>
+inline size_t dir_y_elems(const DirPlan<T>& P) {
+    return 2 * (size_t)P.hyp * P.hyp + 2 * (size_t)P.hyp * P.lines;
+}
+
+template <typename T>
+__device__ __forceinline__ bool dir_any_active(const SliceCtl* ctl, int batch) {
+    for (int s = 0; s < batch; ++s)
+        if (dir_active<T>(ctl + s)) return true;
+    return false;
+}
+
+// Along x: rows of src to rows of dst (INV: the application's slot of the
+// ring), P.lines rows at a time.
+template <typename T, bool INV>
+__global__ void __launch_bounds__(DIR_MAX_THREADS)
+    k_dir_x(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const T* __restrict__ src,
+            T* __restrict__ dst, long long ring, int batch) {
+    pdl_wait();
+    if (!dir_any_active<T>(ctl, batch)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int nx = P.nx, hx = P.hx, hxp = P.hxp, L = P.lines, ldf = L + 4;
+    T* R = reinterpret_cast<T*>(smem_raw);
+    T* F = R + 2 * hxp * hxp;  // [parity][column][row]
+    const int t = (int)threadIdx.x, nt = (int)blockDim.x;
+    dir_copy<T>(R, P.rx[INV ? 1 : 0], 2 * hxp * hxp, t, nt);
+    const int rows = P.ny * P.nz, blocks = (rows + L - 1) / L, dc = hxp / DIR_LNC;
+    for (long long it = blockIdx.x; it < (long long)blocks * batch; it += gridDim.x) {
+        const int s = (int)(it / blocks), r0 = (int)(it - (long long)s * blocks) * L;
+        if (!dir_active<T>(ctl + s)) continue;
+        const T scale = dir_scale<T>(ctl + s, INV);
+        const T* __restrict__ a = src + s * P.cells + (long long)r0 * nx;
+        T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s) * ring : 0) + s * P.cells +
+                            (long long)r0 * nx;
+        const int nr = min(L, rows - r0);
+        __syncthreads();  // the previous block's lines are read
+#pragma unroll 2
+        for (int w = t; w < hxp * (L / 4); w += nt) {
+            const int y0 = 4 * (w / hxp), j = w - (y0 / 4) * hxp;
+            // (loads without conditions, so that they are issued together)
+            const int jj = min(j, hx - 1), xm = INV ? hx + min(jj, nx - hx - 1) : nx - 1 - jj;
+            Q4<T> e, d;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const T* __restrict__ line = a + min(y0 + r, nr - 1) * nx;
+                e.v[r] = line[jj];
+                d.v[r] = line[xm];
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const bool in = y0 + r < nr && j < hx;
+                const T a0 = in ? e.v[r] : T(0);
+                T a1 = in ? d.v[r] : T(0);
+                if (!INV) {
+                    // the middle of an odd extent: itself in the sum, zero in
+                    // the difference
+                    e.v[r] = scale * (xm != jj ? a0 + a1 : a0);
+                    d.v[r] = xm != jj ? scale * (a0 - a1) : T(0);
+                } else {
+                    e.v[r] = a0;
+                    d.v[r] = j < nx - hx ? a1 : T(0);
+                }
+            }
+            q4_st<T>(F + j * ldf + y0, e);
+            q4_st<T>(F + (hxp + j) * ldf + y0, d);
+        }
+        __syncthreads();
+        for (int w = t; w < dc * (L / DIR_LRB); w += nt) {
+            const int rb = w / dc, c = w - rb * dc;
+            T e[DIR_LNC][DIR_LRB] = {}, d[DIR_LNC][DIR_LRB] = {};
+            dir_cols<T, DIR_LRB, DIR_LNC>(F + rb * DIR_LRB, ldf, R + c, hxp, dc, hx, e);
+            dir_cols<T, DIR_LRB, DIR_LNC>(F + hxp * ldf + rb * DIR_LRB, ldf, R + hxp * hxp + c,
+                                          hxp, dc, hx, d);
+#pragma unroll
+            for (int i = 0; i < DIR_LRB; ++i) {
+                const int row = rb * DIR_LRB + i;
+                if (row >= nr) break;
+                T* line = o + row * nx;
+#pragma unroll
+                for (int n = 0; n < DIR_LNC; ++n) {
+                    const int x = c + n * dc, xm = nx - 1 - x;
+                    if (x >= hx) continue;
+                    if (!INV) {
+                        line[x] = e[n][i];
+                        if (x < nx - hx) line[hx + x] = d[n][i];
+                    } else {
+                        line[x] = scale * (e[n][i] + d[n][i]);
+                        if (xm != x) line[xm] = scale * (e[n][i] - d[n][i]);
+                    }
+                }
+            }
+        }
+    }
+}
+
+// Along y, in place: P.lines columns of a plane at a time.
+template <typename T, bool INV>
+__global__ void __launch_bounds__(DIR_MAX_THREADS)
+    k_dir_y(DirPlan<T> P, const SliceCtl* __restrict__ ctl, T* __restrict__ spec, int batch) {
+    pdl_wait();
+    if (!dir_any_active<T>(ctl, batch)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int nx = P.nx, ny = P.ny, hy = P.hy, hyp = P.hyp, L = P.lines;
+    T* Lm = reinterpret_cast<T*>(smem_raw);
+    T* F = Lm + 2 * hyp * hyp;  // [parity][row][column]
+    const int t = (int)threadIdx.x, nt = (int)blockDim.x;
+    dir_copy<T>(Lm, P.ly[INV ? 0 : 1], 2 * hyp * hyp, t, nt);
+    const int xb = (nx + L - 1) / L, blocks = xb * P.nz, dc = L / DIR_LNC;
+    for (long long it = blockIdx.x; it < (long long)blocks * batch; it += gridDim.x) {
+        const int s = (int)(it / blocks), r = (int)(it - (long long)s * blocks);
+        if (!dir_active<T>(ctl + s)) continue;
+        const int z = r / xb, x0 = (r - z * xb) * L, nc = min(L, nx - x0);
+        T* __restrict__ a = spec + s * P.cells + (long long)z * nx * ny + x0;
+        __syncthreads();
+#pragma unroll 8
+        for (int q = t; q < hy * L; q += nt) {
+            const int y = q / L, c = q - y * L;
+            const int ym = INV ? hy + min(y, ny - hy - 1) : ny - 1 - y, cc = min(c, nc - 1);
+            const T a0 = a[y * nx + cc], a1 = a[ym * nx + cc];
+            const T e = INV ? a0 : (ym != y ? a0 + a1 : a0);
+            const T d = INV ? (y < ny - hy ? a1 : T(0)) : (ym != y ? a0 - a1 : T(0));
+            F[q] = e;
+            F[hyp * L + q] = d;
+        }
+        __syncthreads();
+        for (int w = t; w < dc * (hyp / DIR_LRB); w += nt) {
+            const int rb = w / dc, c = w - rb * dc;
+            T e[DIR_LNC][DIR_LRB] = {}, d[DIR_LNC][DIR_LRB] = {};
+            dir_cols<T, DIR_LRB, DIR_LNC>(Lm + rb * DIR_LRB, hyp, F + c, L, dc, hy, e);
+            dir_cols<T, DIR_LRB, DIR_LNC>(Lm + hyp * hyp + rb * DIR_LRB, hyp, F + hyp * L + c, L,
+                                          dc, hy, d);
+#pragma unroll
+            for (int i = 0; i < DIR_LRB; ++i) {
+                const int ky = rb * DIR_LRB + i, ym = ny - 1 - ky;
+                if (ky >= hy) break;
+#pragma unroll
+                for (int n = 0; n < DIR_LNC; ++n) {
+                    const int x = c + n * dc;
+                    if (x >= nc) continue;
+                    if (!INV) {
+                        a[ky * nx + x] = e[n][i];
+                        if (ky < ny - hy) a[(hy + ky) * nx + x] = d[n][i];
+                    } else {
+                        a[ky * nx + x] = e[n][i] + d[n][i];
+                        if (ym != ky) a[ym * nx + x] = e[n][i] - d[n][i];
+                    }
                 }
             }
         }
@@ -845,8 +1031,32 @@ inline void dir_basis(int n, bool periodic, std::vector<double>& q, std::vector<
     }
 }
 
-// Fills P's sizes for n cells; false where the plane does not fit shared
-// memory or a column the chunks of one CTA.
+// Stride of rows of w elements (a multiple of 4): an odd number of 16-byte
+// units, so that eight threads' 16-byte stores hit different banks.
+inline int dir_odd(int w) { return (w / 4) % 2 ? w : w + 4; }
+
+// Sizes of the transforms one axis at a time; false where an axis's matrices
+// do not fit.
+template <typename T>
+inline bool dir_line_sizes(DirPlan<T>& P) {
+    P.rb = DIR_LRB;
+    P.hyp = (P.hy + DIR_LRB - 1) / DIR_LRB * DIR_LRB;
+    for (P.lines = 64; P.lines >= 32; P.lines /= 2)
+        if (dir_x_elems(P) * sizeof(T) <= DIR_MAX_SMEM &&
+            dir_y_elems(P) * sizeof(T) <= DIR_MAX_SMEM) {
+            auto threads = [](int items) {
+                const int nt = (items + 31) / 32 * 32;
+                return nt > DIR_MAX_THREADS ? DIR_MAX_THREADS : nt;
+            };
+            P.ntx = threads(P.hxp / DIR_LNC * (P.lines / DIR_LRB));
+            P.nty = threads(P.lines / DIR_LNC * (P.hyp / DIR_LRB));
+            return true;
+        }
+    return false;
+}
+
+// Fills P's sizes for n cells; false where neither the plane nor an axis's
+// matrices fit shared memory, or a column does not fit the chunks of one CTA.
 template <typename T>
 inline bool dir_sizes(const int n[3], bool per_z, int planes, DirPlan<T>& P) {
     P = DirPlan<T>{};
@@ -858,12 +1068,17 @@ inline bool dir_sizes(const int n[3], bool per_z, int planes, DirPlan<T>& P) {
     P.hx = (n[0] + 1) / 2;
     P.hy = (n[1] + 1) / 2;
     P.hxp = (P.hx + 3) / 4 * 4;
-    P.hyp = (P.hy + 3) / 4 * 4;
-    // rows an odd number of 16-byte units apart: eight rows' reads then hit
-    // different banks
-    auto odd = [](int w) { return (w / 4) % 2 ? w : w + 4; };
-    P.ldx = odd(P.hxp);
-    P.ldy = odd(P.hyp);
+    // rows and columns per thread: shared-memory cycles of a block of 16 rows
+    // (with the padded rows), (rows / 4 + columns) / columns; a call that
+    // leaves SMs idle prefers more threads
+    P.ncol = planes < 152 ? 1 : 2;
+    P.rb = 4;
+    for (int rb = 8; rb <= (planes < 152 ? 8 : 16); rb *= 2) {
+        auto cost = [&](int r) { return (P.hy + r - 1) / r * (r / 4 + P.ncol); };
+        if (cost(rb) <= cost(P.rb)) P.rb = rb;
+    }
+    P.hyp = (P.hy + P.rb - 1) / P.rb * P.rb;
+    P.ldf = dir_odd(P.hyp);
     P.zm = n[2] <= 16 * DIR_ZC ? DIR_ZC : DIR_ZC_LONG;
     P.zc = (n[2] + P.zm - 1) / P.zm;
     if (P.zc * DIR_ZX > dir_z_threads<T>(P.zm)) return false;
@@ -873,15 +1088,15 @@ inline bool dir_sizes(const int n[3], bool per_z, int planes, DirPlan<T>& P) {
         P.cb = (P.hxp / 4 + xb - 1) / xb * 4;
         P.xb = (P.hxp + P.cb - 1) / P.cb;
         if (dir_smem_elems(P) * sizeof(T) <= DIR_MAX_SMEM) {
-            const int tiles = P.hyp * P.cb / 4;
-            P.nt = (tiles + 31) / 32 * 32;
+            const int items = 4 * (P.cb / P.ncol) * (P.hyp / P.rb);
+            P.nt = (items + 31) / 32 * 32;
             P.nt = P.nt < 64 ? 64 : P.nt;
-            P.nt = P.nt < P.hxp ? (P.hxp + 31) / 32 * 32 : P.nt;
+            P.nt = P.nt < P.cb ? (P.cb + 31) / 32 * 32 : P.nt;
             P.nt = P.nt > DIR_MAX_THREADS ? DIR_MAX_THREADS : P.nt;
-            return P.nt >= P.hxp;
+            if (P.nt >= P.cb) return true;
         }
     }
-    return false;
+    return dir_line_sizes<T>(P);
 }
 
 // The tables of a plan: x matrices (forward, inverse), y matrices (forward,

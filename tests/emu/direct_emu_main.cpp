@@ -4,15 +4,18 @@
 // inactive), every CTA as host threads, and writes e.
 //
 // usage: direct_emu T nx ny nz bcx bcy bcz lx ly lz planes in.bin out.bin
-//   T: f or d; in.bin: r, two states; out.bin: e, two states (the inactive
+//   planes: of a call, 0: the transforms one axis at a time; T: f or d; in.bin: r, two states; out.bin: e, two states (the inactive
 //   one's untouched zeros).
 
 #include <functional>
+#include <type_traits>
 
-static void launch(int gx, int bx, int by, size_t smem, const std::function<void()>& body) {
+static void launch(int gx, int bx, int by, size_t smem, const std::function<void()>& body,
+                   int states = 2) {
     const int n = bx * by;
     blockDim = EmuDim3{(unsigned)bx, (unsigned)by, 1};
-    for (int st = 0; st < 2; ++st)
+    gridDim = EmuDim3{(unsigned)gx, (unsigned)states, 1};
+    for (int st = 0; st < states; ++st)
         for (int c = 0; c < gx; ++c) {
             std::barrier<> bar(n);
             emu_cta_barrier = &bar;
@@ -42,7 +45,9 @@ static int run(char** argv) {
         ih2[a] = 1.0 / (h * h);
     }
     DirPlan<T> P;
-    if (!dir_sizes<T>(n, bc[2] == BC_PERIODIC, atoi(argv[11]), P)) return 2;
+    const int planes = atoi(argv[11]);
+    if (!dir_sizes<T>(n, bc[2] == BC_PERIODIC, planes ? planes : 500, P)) return 2;
+    if (!planes && !dir_line_sizes<T>(P)) return 2;
     size_t off[5];
     std::vector<T> tab = dir_tables<T>(P, bc, ih2, off);
     P.rx[0] = tab.data() + off[0];
@@ -63,8 +68,36 @@ static int run(char** argv) {
     ctl[1].status = ST_CONV;
     ctl[1].o_status = OS_DONE;
     const size_t smem = dir_smem_elems(P) * sizeof(T);
-    launch(P.nz * P.xb, P.nt, 1, smem,
-           [&] { k_dir_xy<T, false>(P, ctl, r.data(), spec.data(), 0); });
+    auto xy = [&](auto inv, const T* src, T* dst) {
+        constexpr bool INV = decltype(inv)::value;
+        auto go = [&](auto rb, auto nc) {
+            launch(P.nz * P.xb, P.nt, 1, smem,
+                   [&] { k_dir_xy<T, INV, decltype(rb)::value, decltype(nc)::value>(P, ctl, src, dst, 0); });
+        };
+        // one axis at a time: CTAs of each kernel take several blocks of lines
+        auto x = [&] {
+            launch(3, P.ntx, 1, dir_x_elems(P) * sizeof(T),
+                   [&] { k_dir_x<T, INV>(P, ctl, src, dst, 0, 2); }, 1);
+        };
+        auto y = [&] {
+            launch(2, P.nty, 1, dir_y_elems(P) * sizeof(T),
+                   [&] { k_dir_y<T, INV>(P, ctl, spec.data(), 2); }, 1);
+        };
+        if (P.lines) {
+            if (INV) y();
+            x();
+            if (!INV) y();
+        } else {
+            using One = std::integral_constant<int, 1>;
+            using Two = std::integral_constant<int, 2>;
+            using R4 = std::integral_constant<int, 4>;
+            using R8 = std::integral_constant<int, 8>;
+            if (P.rb == 16) go(std::integral_constant<int, 16>{}, Two{});
+            else if (P.rb == 8) P.ncol == 2 ? go(R8{}, Two{}) : go(R8{}, One{});
+            else P.ncol == 2 ? go(R4{}, Two{}) : go(R4{}, One{});
+        }
+    };
+    xy(std::false_type{}, r.data(), spec.data());
     const int zg = (P.nx * P.ny + DIR_ZX - 1) / DIR_ZX;
     launch(zg, DIR_ZX, P.zc, 0, [&] {
         if (P.zm == DIR_ZC)
@@ -72,8 +105,7 @@ static int run(char** argv) {
         else
             k_dir_z<T, DIR_ZC_LONG>(P, ctl, spec.data());
     });
-    launch(P.nz * P.xb, P.nt, 1, smem,
-           [&] { k_dir_xy<T, true>(P, ctl, spec.data(), e.data(), 0); });
+    xy(std::true_type{}, spec.data(), e.data());
     f = fopen(argv[13], "wb");
     fwrite(e.data(), sizeof(T), 2 * N, f);
     fclose(f);

@@ -77,7 +77,8 @@ def _lap(p, h, bc):
     return out
 
 
-# (cells, boundaries, box, planes of a call: below 152 two column blocks)
+# (cells, boundaries, box, planes of a call: below 152 two column blocks, 0: the
+# transforms one axis at a time)
 CASES = [
     ((16, 16, 16), ("wall",) * 3, (1.0, 1.0, 1.0), 16),
     ((2, 2, 2), ("wall",) * 3, (1.0, 1.0, 1.0), 2),
@@ -90,6 +91,9 @@ CASES = [
     ((6, 5, 130), ("wall", "periodic", "wall"), (1.0, 1.0, 20.0), 500),   # long chunks
     ((5, 6, 133), ("wall", "wall", "periodic"), (1.0, 1.0, 20.0), 500),
     ((72, 128, 2), ("slip", "wall", "wall"), (1.0, 2.0, 0.1), 500),       # FP64: column blocks
+    ((19, 33, 9), ("wall", "slip", "wall"), (1.0, 1.5, 0.5), 0),
+    ((70, 10, 5), ("periodic", "wall", "wall"), (3.0, 0.5, 0.3), 0),      # ragged line blocks
+    ((4, 2, 6), ("wall", "periodic", "periodic"), (1.0, 1.0, 1.0), 0),
 ]
 
 
