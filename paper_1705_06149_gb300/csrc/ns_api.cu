@@ -101,11 +101,17 @@ struct ns_grid {
     // mg stays set (the solves share the multigrid path's start, correction
     // and graphs), hier tells whether the grid has the hierarchy's levels
     bool dir = false;
+    // with solid cells (FP32+refine): conjugate gradients it preconditions
+    bool cg = false;
     bool hier = false;
     DirPlan<float> dirf{};
     DirPlan<double> dird{};
     size_t dir_smem = 0;
     int dir_hint = 2;  // applications the last solves took
+    // with solid cells: the faces whose stencil meets one (null: all faces are
+    // evaluated as if theirs did)
+    long long* near_faces = nullptr;
+    long long near_count = 0;
     DirTile dir_tile{};                         // FP32+refine: tiling of the step kernels
     float* dir_ring = nullptr;                  // FP32+refine: the last applications
     double* dir_part = nullptr;                 // [cap][dir_tile.ctas][7]
@@ -1630,6 +1636,29 @@ ns_status solve_pressure(ns_grid* g, int batch, const double* p_in) {
     return NS_OK;
 }
 
+// The faces near solid cells, where they are at most a quarter of all (one
+// costs about 16 times a tile's face): the predictor then runs the tiles and
+// those faces, above that every face by the solid cells' rules.
+ns_status list_near_faces(ns_grid* g) {
+    const Geo& G = g->geo;
+    const long long total = G.cnt[0] + G.cnt[1] + G.cnt[2];
+    const unsigned ctas = (unsigned)((total + 255) / 256);
+    unsigned long long *count = nullptr, n = 0;
+    NS_TRY(dalloc(g, (void**)&count, sizeof(*count)));
+    for (int fill = 0; fill < 2; ++fill) {
+        NS_CUDA(cudaMemsetAsync(count, 0, sizeof(*count), g->stream));
+        k_list_faces<<<ctas, 256, 0, g->stream>>>(G, g->near_faces, count);
+        NS_CUDA(cudaGetLastError());
+        NS_CUDA(cudaMemcpyAsync(&n, count, sizeof(n), cudaMemcpyDeviceToHost, g->stream));
+        NS_CUDA(cudaStreamSynchronize(g->stream));
+        if (fill) break;
+        if (4 * (long long)n > total) return NS_OK;
+        NS_TRY(dalloc(g, (void**)&g->near_faces, sizeof(long long) * std::max(n, 1ull)));
+    }
+    g->near_count = (long long)n;
+    return NS_OK;
+}
+
 // Calls f with the predictor tile (px, py, pz) as constants.
 template <typename F>
 auto with_predict_tile(int px, int py, int pz, F&& f) {
@@ -1660,7 +1689,7 @@ template <typename T, bool INCR>
 void launch_predict(ns_grid* g, int batch, const T* u, const T* v, const T* w, T* fu, T* fv, T* fw,
                     double dt) {
     const Geo& G = g->geo;
-    if (G.solid) {
+    if (G.solid && !g->near_faces) {
         k_predict_masked<T, INCR><<<dim3(G.fctas, batch), block_dim(), 0, g->stream>>>(
             G, u, v, w, fu, fv, fw, dt);
         return;
@@ -1674,6 +1703,10 @@ void launch_predict(ns_grid* g, int batch, const T* u, const T* v, const T* w, T
         k_predict_tile<T, INCR, PY, PZ, PX><<<dim3(tbx * tby * tbz, batch), PX * PY, smem,
                                               g->stream>>>(G, u, v, w, fu, fv, fw, dt, tbx, tby);
     });
+    if (g->near_count)
+        k_predict_faces<T, INCR>
+            <<<dim3((unsigned)((g->near_count + NTHREADS - 1) / NTHREADS), batch), block_dim(), 0,
+               g->stream>>>(G, u, v, w, fu, fv, fw, dt, g->near_faces, g->near_count);
 }
 
 // Shared memory limit of the predictor instantiation the grid uses (a value
@@ -2805,6 +2838,7 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             st = fail(NS_ERR_CUDA, "ns_create_grid: mask copy failed");
         g->geo.solid = (const uint8_t*)m;
         g->geo.n_fluid = (int)(ncell - n_solid);
+        if (st == NS_OK) st = list_near_faces(g);
     }
     if (d.preconditioner == NS_PC_MULTIGRID && st == NS_OK) {
         // levels at or below this size run in one CTA per state (FP32: up to
