@@ -500,6 +500,7 @@ void with_dir_shape(int rb, int ncol, F&& f) {
 template <typename T>
 ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
     const Geo& G = g->geo;
+    const bool solid = G.solid != nullptr;
     if (!dir_sizes<T>(G.n, G.bc[2] == BC_PERIODIC, G.n[2] * g->cap, P)) return NS_OK;
     size_t off[5];
     const std::vector<T> tab = dir_tables<T>(P, G.bc, G.ih2, off);
@@ -534,6 +535,11 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
         });
     }
     if (!ok) return fail(NS_ERR_CUDA, "ns_create_grid: direct solve shared memory attribute");
+    if (solid) {
+        P.precond = 1;
+        g->cg = true;
+        return NS_OK;
+    }
     g->dir = true;
     g->mg = true;
     if (sizeof(T) == 4) {
@@ -554,12 +560,14 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
 // precision can mean (below it the Krylov recursion decides, as it always
 // did).  The environment variables that select a form of the multigrid solve
 // (NS_MG_CLUSTER, NS_MG_BLOCK_CELLS, NS_PERSISTENT), when set, select it;
-// NS_DIRECT=0 turns the direct solve off.
+// NS_DIRECT=0 turns the direct solve off.  With solid cells, FP32+refine, the
+// same conditions make it the preconditioner of the inner solves.
 ns_status setup_direct(ns_grid* g) {
     for (const char* v : {"NS_MG_CLUSTER", "NS_MG_BLOCK_CELLS", "NS_PERSISTENT"})
         if (std::getenv(v)) return NS_OK;
     const char* env = std::getenv("NS_DIRECT");
-    if ((env && std::atoi(env) == 0) || g->geo.solid) return NS_OK;
+    if (env && std::atoi(env) == 0) return NS_OK;
+    if (g->geo.solid && !(g->mg && g->fp32)) return NS_OK;
     const double rtol = g->fp32 ? g->d.refine_rtol : g->d.poisson_rtol;
     const double cond = dir_condition(g->geo.n, g->geo.bc, g->geo.ih2);
     if (!(rtol >= 1e-14) || !(cond <= (g->fp32 ? 1e7 : 1e12))) return NS_OK;
@@ -885,10 +893,11 @@ template <typename T>
 void direct_apply(ns_grid* g, int batch) {
     const DirPlan<T>& P = dirplan<T>(g);
     const bool f32 = sizeof(T) == 4;
-    const T* r = f32 ? (const T*)g->ffb[2] : (const T*)g->kv[1];
-    T* spec = (T*)g->kv[3];
-    T* e = f32 ? (T*)g->dir_ring : (T*)g->kv[4];
-    const long long ring = f32 ? dir_stride(g) : 0;
+    // (as a preconditioner: from kv[1] into kv[6], the spectral planes in kv[7])
+    const T* r = f32 && !g->cg ? (const T*)g->ffb[2] : (const T*)g->kv[1];
+    T* spec = (T*)g->kv[g->cg ? 7 : 3];
+    T* e = g->cg ? (T*)g->kv[6] : (f32 ? (T*)g->dir_ring : (T*)g->kv[4]);
+    const long long ring = f32 && !g->cg ? dir_stride(g) : 0;
     const dim3 pg(P.nz * P.xb, batch), zg(ceil_div(P.nx * P.ny, DIR_ZX), batch);
     const dim3 zb(DIR_ZX, P.zc);
     const long long units = P.cells * batch;
@@ -955,6 +964,19 @@ ns_status mg_iteration(ns_grid* g, int batch, double tol2, int zero_start) {
     MgBuf<T> mb = mgbuf<T>(g);
     const dim3 grid(L0.ctas, batch), blk = block_dim();
     // x pairs per thread where the level has no solid cells and an even nx
+    if (g->cg) {
+        const T* z = (const T*)g->kv[6];
+        direct_apply<T>(g, batch);
+        NS_LAUNCH(g, NS_K_MG_LAP_T, 0,
+                  k_cg_dot<T><<<grid, blk, 0, g->stream>>>(L0, mb, z, g->ctl, g->part_mg));
+        NS_LAUNCH(g, NS_K_MG_LAP_V, 0,
+                  k_cg_lap<T><<<grid, blk, 0, g->stream>>>(L0, mb, z, g->ctl, g->part_mg));
+        NS_LAUNCH(g, NS_K_KRYLOV_C, 0,
+                  k_cg_update<T><<<grid, blk, 0, g->stream>>>(L0, mb, g->ctl, g->part_mg, tol2,
+                                                              g->maxit));
+        NS_CUDA(cudaGetLastError());
+        return NS_OK;
+    }
     const bool pair = L0.fcode == nullptr && L0.n[0] % 2 == 0;
     const int pbx = ceil_div(L0.n[0], 64);
     const int pctas = pbx * L0.by * L0.bz;
@@ -1891,6 +1913,7 @@ long long mg_iteration_launches(const ns_grid* g) {
         const bool lines = g->fp32 ? g->dirf.lines > 0 : g->dird.lines > 0;
         return (lines ? 5 : 3) + (g->fp32 ? 0 : 1);
     }
+    if (g->cg) return (g->dirf.lines > 0 ? 5 : 3) + 3;
     const int lc = g->plan.lc;
     const long long apply = 1 + lc + std::max(lc - 1, 0) + 1 + lc;
     return 2 * apply + 3;
@@ -2865,8 +2888,8 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
     for (int q = 0; q < 8; ++q)
         if (!g->dir || q == 3 || (!g->fp32 && q < 5)) A(&g->kv[q], ncell * ev * B);
     if (g->mg) {
-        for (int q = 0; q < 3 && !g->dir; ++q) A(&g->mg_vec[q], ncell * ev * B);
-        for (int l = 1; l <= g->plan.lc && !g->dir; ++l) {
+        for (int q = 0; q < 3 && !(g->dir || g->cg); ++q) A(&g->mg_vec[q], ncell * ev * B);
+        for (int l = 1; l <= g->plan.lc && !(g->dir || g->cg); ++l) {
             A(&g->mg_B[l], (size_t)g->plan.lev[l].cells * ev * B);
             A(&g->mg_Y[l], (size_t)g->plan.lev[l].cells * ev * B);
         }
@@ -2877,7 +2900,7 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             for (int q = 0; q < 8; ++q) A((void**)&g->ffb[q], ncell * sizeof(float) * B);
         A((void**)&g->part_mg, nparts * 6 * sizeof(double));
     }
-    if (g->mg && !g->dir && st == NS_OK) {
+    if (g->mg && !g->dir && !g->cg && st == NS_OK) {
         // the coarse levels on a thread-block cluster per state, where they
         // split into slabs (NS_MG_CLUSTER=0 turns it off)
         const char* ce = std::getenv("NS_MG_CLUSTER");
@@ -2957,7 +2980,7 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
             if (cudaMemsetAsync(g->counter, 0, sizeof(unsigned int) * B, g->stream) !=
                 cudaSuccess)
                 st = fail(NS_ERR_CUDA, "ns_create_grid: memset failed");
-            for (int q = 0; q < 3 && !g->dir && st == NS_OK; ++q)
+            for (int q = 0; q < 3 && !(g->dir || g->cg) && st == NS_OK; ++q)
                 if (cudaMemsetAsync(g->mg_vec[q], 0, ncell * ev * B, g->stream) != cudaSuccess)
                     st = fail(NS_ERR_CUDA, "ns_create_grid: memset failed");
             // k_mg_block's shared memory stays within the default 48 KB

@@ -38,6 +38,7 @@ constexpr int DIR_ZX = 32;       // columns per CTA of k_dir_z
 template <typename T>
 struct DirPlan {
     int nx, ny, nz, per_z;
+    int precond;   // 1: the transforms precondition the conjugate gradients below
     int hx, hy;    // even modes (= length of the folded line) along x, y
     int hxp;       // hx rounded up to 4
     int rb, ncol;  // rows and columns per thread of k_dir_xy
@@ -62,12 +63,14 @@ constexpr int dir_z_threads(int zm) {
 }
 
 // Whether the state takes part in the current application: FP32+refine while
-// its outer residual is above the target, FP64 while it iterates.
-template <typename T> __device__ __forceinline__ bool dir_active(const SliceCtl* c);
-template <> __device__ __forceinline__ bool dir_active<float>(const SliceCtl* c) {
+// its outer residual is above the target; FP64, or as a preconditioner, while
+// it iterates.
+template <typename T> __device__ __forceinline__ bool dir_active(const SliceCtl* c, int precond);
+template <> __device__ __forceinline__ bool dir_active<float>(const SliceCtl* c, int precond) {
+    if (precond) return c->status == ST_ITER;
     return c->o_status == OS_REFINE && c->status != ST_NONFINITE;
 }
-template <> __device__ __forceinline__ bool dir_active<double>(const SliceCtl* c) {
+template <> __device__ __forceinline__ bool dir_active<double>(const SliceCtl* c, int) {
     return c->status == ST_ITER;
 }
 
@@ -75,20 +78,25 @@ template <> __device__ __forceinline__ bool dir_active<double>(const SliceCtl* c
 // the pressure is the warm start plus the applications not yet folded into it
 // (the last three at most).  The residual is scaled by a power of two on its
 // way into the transforms and e unscaled on its way out, so that neither
-// underflows however far the refinement has come.
+// underflows however far the refinement has come (a preconditioned residual
+// carries its scale already and has one buffer).
 constexpr int DIR_RING = 4;
-template <typename T> __device__ __forceinline__ T dir_scale(const SliceCtl* c, bool inv);
-template <> __device__ __forceinline__ float dir_scale<float>(const SliceCtl* c, bool inv) {
+template <typename T>
+__device__ __forceinline__ T dir_scale(const SliceCtl* c, bool inv, int precond);
+template <>
+__device__ __forceinline__ float dir_scale<float>(const SliceCtl* c, bool inv, int precond) {
+    if (precond) return 1.0f;
     return inv ? 1.0f / c->o_fsc : c->o_fsc;
 }
-template <> __device__ __forceinline__ double dir_scale<double>(const SliceCtl*, bool) {
+template <>
+__device__ __forceinline__ double dir_scale<double>(const SliceCtl*, bool, int) {
     return 1.0;
 }
-template <typename T> __device__ __forceinline__ int dir_slot(const SliceCtl* c);
-template <> __device__ __forceinline__ int dir_slot<float>(const SliceCtl* c) {
-    return c->o_steps & (DIR_RING - 1);
+template <typename T> __device__ __forceinline__ int dir_slot(const SliceCtl* c, int precond);
+template <> __device__ __forceinline__ int dir_slot<float>(const SliceCtl* c, int precond) {
+    return precond ? 0 : c->o_steps & (DIR_RING - 1);
 }
-template <> __device__ __forceinline__ int dir_slot<double>(const SliceCtl*) { return 0; }
+template <> __device__ __forceinline__ int dir_slot<double>(const SliceCtl*, int) { return 0; }
 
 // acc[n][i] += sum_k L[k][i] R[k][n dc], i < RB, n < NC, k ascending; rows of L
 // (16-byte aligned) are ldl apart, of R ldr.  Neighbouring threads hold
@@ -144,8 +152,8 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
              T* __restrict__ dst, long long ring) {
     pdl_wait();
     const long long s = blockIdx.y;
-    if (!dir_active<T>(ctl + s)) return;
-    const T scale = dir_scale<T>(ctl + s, INV);
+    if (!dir_active<T>(ctl + s, P.precond)) return;
+    const T scale = dir_scale<T>(ctl + s, INV, P.precond);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, ny = P.ny, hx = P.hx, hy = P.hy, hxp = P.hxp, hyp = P.hyp;
     const int ldf = P.ldf, cb = P.cb;
@@ -157,7 +165,7 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const int c0 = ((int)blockIdx.x - z * P.xb) * cb;
     const int t = (int)threadIdx.x, nt = (int)blockDim.x;
     const T* __restrict__ a = src + s * P.cells + (long long)z * nx * ny;
-    T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s) * ring : 0) + s * P.cells +
+    T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s, P.precond) * ring : 0) + s * P.cells +
                         (long long)z * nx * ny;
     // the plane: four rows of one column at a time (F[quadrant][column][row]);
     // rows and columns beyond the halves are zero
@@ -299,9 +307,9 @@ inline size_t dir_y_elems(const DirPlan<T>& P) {
 }
 
 template <typename T>
-__device__ __forceinline__ bool dir_any_active(const SliceCtl* ctl, int batch) {
+__device__ __forceinline__ bool dir_any_active(const SliceCtl* ctl, int batch, int precond) {
     for (int s = 0; s < batch; ++s)
-        if (dir_active<T>(ctl + s)) return true;
+        if (dir_active<T>(ctl + s, precond)) return true;
     return false;
 }
 
@@ -312,7 +320,7 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     k_dir_x(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const T* __restrict__ src,
             T* __restrict__ dst, long long ring, int batch) {
     pdl_wait();
-    if (!dir_any_active<T>(ctl, batch)) return;
+    if (!dir_any_active<T>(ctl, batch, P.precond)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, hx = P.hx, hxp = P.hxp, L = P.lines, ldf = L + 4;
     T* R = reinterpret_cast<T*>(smem_raw);
@@ -322,10 +330,10 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const int rows = P.ny * P.nz, blocks = (rows + L - 1) / L, dc = hxp / DIR_LNC;
     for (long long it = blockIdx.x; it < (long long)blocks * batch; it += gridDim.x) {
         const int s = (int)(it / blocks), r0 = (int)(it - (long long)s * blocks) * L;
-        if (!dir_active<T>(ctl + s)) continue;
-        const T scale = dir_scale<T>(ctl + s, INV);
+        if (!dir_active<T>(ctl + s, P.precond)) continue;
+        const T scale = dir_scale<T>(ctl + s, INV, P.precond);
         const T* __restrict__ a = src + s * P.cells + (long long)r0 * nx;
-        T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s) * ring : 0) + s * P.cells +
+        T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s, P.precond) * ring : 0) + s * P.cells +
                             (long long)r0 * nx;
         const int nr = min(L, rows - r0);
         __syncthreads();  // the previous block's lines are read
@@ -393,7 +401,7 @@ template <typename T, bool INV>
 __global__ void __launch_bounds__(DIR_MAX_THREADS)
     k_dir_y(DirPlan<T> P, const SliceCtl* __restrict__ ctl, T* __restrict__ spec, int batch) {
     pdl_wait();
-    if (!dir_any_active<T>(ctl, batch)) return;
+    if (!dir_any_active<T>(ctl, batch, P.precond)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, ny = P.ny, hy = P.hy, hyp = P.hyp, L = P.lines;
     T* Lm = reinterpret_cast<T*>(smem_raw);
@@ -403,7 +411,7 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const int xb = (nx + L - 1) / L, blocks = xb * P.nz, dc = L / DIR_LNC;
     for (long long it = blockIdx.x; it < (long long)blocks * batch; it += gridDim.x) {
         const int s = (int)(it / blocks), r = (int)(it - (long long)s * blocks);
-        if (!dir_active<T>(ctl + s)) continue;
+        if (!dir_active<T>(ctl + s, P.precond)) continue;
         const int z = r / xb, x0 = (r - z * xb) * L, nc = min(L, nx - x0);
         T* __restrict__ a = spec + s * P.cells + (long long)z * nx * ny + x0;
         __syncthreads();
@@ -454,7 +462,7 @@ __global__ void __launch_bounds__(dir_z_threads<T>(ZM))
     k_dir_z(DirPlan<T> P, SliceCtl* __restrict__ ctl, T* __restrict__ a) {
     pdl_wait();
     const long long s = blockIdx.y;
-    if (!dir_active<T>(ctl + s)) return;
+    if (!dir_active<T>(ctl + s, P.precond)) return;
     __shared__ T sY[32][DIR_ZX], sL[32][DIR_ZX], sP[32][DIR_ZX], sX[32][DIR_ZX], sE[DIR_ZX];
     const int lane = (int)threadIdx.x, ch = (int)threadIdx.y, C = (int)blockDim.y;
     const int cols = P.nx * P.ny, nz = P.nz;
@@ -543,7 +551,7 @@ __global__ void __launch_bounds__(dir_z_threads<T>(ZM))
         }
     if (blockIdx.x == 0 && lane == 0 && ch == 0) {
         // an application counts as an iteration (no other CTA reads these)
-        if (sizeof(T) == 4) {
+        if (sizeof(T) == 4 && !P.precond) {
             ctl[s].it_cur = 1;
             ctl[s].total_iters += 1;
         }
@@ -777,7 +785,7 @@ __global__ void __launch_bounds__(NTHREADS)
     pdl_wait();
     const long long s = blockIdx.y;
     SliceCtl* c = ctl + s;
-    if (!dir_active<float>(c)) return;
+    if (!dir_active<float>(c, 0)) return;
     const long long off = s * L.cells;
     const int step = c->o_steps;
     const float* __restrict__ e = ring + (step & (DIR_RING - 1)) * stride + off;
@@ -993,6 +1001,184 @@ __global__ void __launch_bounds__(NTHREADS)
         c->total_iters += 1;
         bicg_decide(c, tot[0], tot[0], tot[1], tol2, maxit);
         c->rmean = c->status == ST_ITER ? tot[2] / nfluid : 0.0;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// solid cells: conjugate gradients preconditioned by the direct solve
+// ---------------------------------------------------------------------------
+
+// With solid cells L (minus it is symmetric and semidefinite) is the Neumann
+// operator of the fluid cells; z = the fluid part of the box solution of r (zero
+// in solid cells) preconditions it with a condition number that depends on the
+// obstacles' shapes and not on the grid (an extension of a fluid field into a
+// solid has at most a fixed multiple of its energy).  An iteration is one
+// application and three passes, 56 B/cell next to the transforms.  128^3 x 8
+// states, 8 boxes: 21 iterations of 392 us per step, where BiCGStab, whose
+// V-cycles know the solids on the finest level only, took 23 of 770 us.
+//
+// The direction survives the outer corrections, which replace r by the true
+// residual: beta = -(z, q) / (p, q) makes the next one conjugate to the last and
+// alpha = (r, p) / (p, q) whatever r is (a restart after each correction took 23
+// iterations per solve).
+//
+// beta from the last iteration's q = L p.
+template <typename T>
+__global__ void __launch_bounds__(NTHREADS)
+    k_cg_dot(Lev L, MgBuf<T> mb, const T* __restrict__ zvec, SliceCtl* __restrict__ ctl,
+             double* __restrict__ part) {
+    pdl_wait();
+    const long long s = blockIdx.y;
+    SliceCtl* c = ctl + s;
+    if (c->status != ST_ITER) return;
+    const bool first = c->it_cur == 0 && c->o_steps == 0;
+    const T* __restrict__ q = mb.V[0] + s * L.cells;
+    const T* __restrict__ z = zvec + s * L.cells;
+    T acc[1] = {T(0)};
+    int i, j, k0;
+    lev_origin(L, blockIdx.x, i, j, k0);
+    if (!first && i < L.n[0] && j < L.n[1]) {
+        const int k1 = min(k0 + L.tz, L.n[2]), plane = L.n[0] * L.n[1];
+        const int base = lindex(L, i, j, 0);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) acc[0] += q[base + k * plane] * z[base + k * plane];
+    }
+    double tot[1];
+    if (partials_arrive<T, 1>(acc, part + s * L.ctas, mb.counter + s, L.ctas, tot) &&
+        tid_flat() == 0)
+        c->beta = first ? 0.0 : -tot[0] / c->rho[1];
+}
+
+// p = z + beta p (zero in solid cells; into the other parity's buffer, the
+// neighbours still read this one's), q = L p, alpha.
+template <typename T>
+__global__ void __launch_bounds__(NTHREADS)
+    k_cg_lap(Lev L, MgBuf<T> mb, const T* __restrict__ zvec, SliceCtl* __restrict__ ctl,
+             double* __restrict__ part) {
+    pdl_wait();
+    const long long s = blockIdx.y;
+    SliceCtl* c = ctl + s;
+    if (c->status != ST_ITER) return;
+    const long long off = s * L.cells;
+    const int par = (int)(c->total_iters & 1);
+    const bool first = c->it_cur == 0 && c->o_steps == 0;
+    const T beta = T(c->beta);
+    const T* __restrict__ r = mb.r + off;
+    const T* __restrict__ z = zvec + off;
+    const T* __restrict__ po = mb.P[par ^ 1] + off;
+    T* __restrict__ p = mb.P[par] + off;
+    T* __restrict__ q = mb.V[0] + off;
+    T acc[2] = {T(0), T(0)};
+    int i, j, k0;
+    lev_origin(L, blockIdx.x, i, j, k0);
+    if (i < L.n[0] && j < L.n[1]) {
+        const int k1 = min(k0 + L.tz, L.n[2]);
+        const NbrXY xy = make_nbr_xy(L, i, j);
+        constexpr int ZB = 2;
+        for (int kb = k0; kb < k1; kb += ZB) {
+            Vals7<T> zv[ZB], pv[ZB];
+            T rv[ZB];
+            int id[ZB];
+            bool fl[ZB];
+#pragma unroll
+            for (int u = 0; u < ZB; ++u) {
+                const Nbr nb = nbr_at(L, xy, min(kb + u, k1 - 1));
+                id[u] = nb.c;
+                fl[u] = lev_fluid(L, nb.c);
+                zv[u] = load7<T>(nb, z);
+                rv[u] = r[nb.c];
+                // (the first iteration's buffer holds anything)
+                pv[u] = first ? Vals7<T>{} : load7<T>(nb, po);
+            }
+#pragma unroll
+            for (int u = 0; u < ZB; ++u) {
+                if (kb + u >= k1) break;
+                Vals7<T> v;
+                v.c = fma(beta, pv[u].c, zv[u].c);
+                v.xh = fma(beta, pv[u].xh, zv[u].xh);
+                v.xl = fma(beta, pv[u].xl, zv[u].xl);
+                v.yh = fma(beta, pv[u].yh, zv[u].yh);
+                v.yl = fma(beta, pv[u].yl, zv[u].yl);
+                v.zh = fma(beta, pv[u].zh, zv[u].zh);
+                v.zl = fma(beta, pv[u].zl, zv[u].zl);
+                // (a solid cell's neighbours are clamped to itself: q = 0)
+                const T lq = lap_vals<T>(L, v);
+                const T pc = fl[u] ? v.c : T(0);
+                p[id[u]] = pc;
+                q[id[u]] = lq;
+                acc[0] += pc * lq;
+                acc[1] += pc * rv[u];
+            }
+        }
+    }
+    double tot[2];
+    if (partials_arrive<T, 2>(acc, part + s * L.ctas * 2, mb.counter + s, L.ctas, tot) &&
+        tid_flat() == 0) {
+        c->rho[1] = tot[0];
+        c->alpha = tot[1] / tot[0];
+    }
+}
+
+// x += alpha p (from zero in a solve's first iteration), r -= alpha q, (r, r),
+// sum x, the decision.
+template <typename T>
+__global__ void __launch_bounds__(NTHREADS)
+    k_cg_update(Lev L, MgBuf<T> mb, SliceCtl* __restrict__ ctl, double* __restrict__ part,
+                double tol2, int maxit) {
+    pdl_wait();
+    const long long s = blockIdx.y;
+    SliceCtl* c = ctl + s;
+    if (c->status != ST_ITER) return;
+    const long long off = s * L.cells;
+    const bool first = c->it_cur == 0;
+    const T alpha = T(c->alpha);
+    const T* __restrict__ p = mb.P[c->total_iters & 1] + off;
+    const T* __restrict__ q = mb.V[0] + off;
+    T* __restrict__ x = mb.x + off;
+    T* __restrict__ r = mb.r + off;
+    T acc[2] = {T(0), T(0)};
+    int i, j, k0;
+    lev_origin(L, blockIdx.x, i, j, k0);
+    if (i < L.n[0] && j < L.n[1]) {
+        const int k1 = min(k0 + L.tz, L.n[2]), plane = L.n[0] * L.n[1];
+        const int base = lindex(L, i, j, 0);
+        for (int kb = k0; kb < k1; kb += MG_ZB) {
+            T xo[MG_ZB], ro[MG_ZB], pv[MG_ZB], qv[MG_ZB];
+#pragma unroll
+            for (int u = 0; u < MG_ZB; ++u) {
+                const int id = base + min(kb + u, k1 - 1) * plane;
+                xo[u] = first ? T(0) : x[id];
+                ro[u] = r[id];
+                pv[u] = p[id];
+                qv[u] = q[id];
+            }
+#pragma unroll
+            for (int u = 0; u < MG_ZB; ++u) {
+                if (kb + u >= k1) break;
+                const int id = base + (kb + u) * plane;
+                const T xv = fma(alpha, pv[u], xo[u]);
+                const T rv = fma(-alpha, qv[u], ro[u]);
+                x[id] = xv;
+                r[id] = rv;
+                acc[0] += rv * rv;
+                acc[1] += xv;
+            }
+        }
+    }
+    double tot[2];
+    if (partials_arrive<T, 2>(acc, part + s * L.ctas * 2, mb.counter + s, L.ctas, tot) &&
+        tid_flat() == 0) {
+        c->it_cur += 1;
+        c->total_iters += 1;
+        c->rr = tot[0];
+        c->sx = tot[1];
+        // (a breakdown, (p, q) = 0 with r != 0, ends as non-finite too)
+        if (!isfinite(tot[0]) || !isfinite(c->alpha))
+            c->status = ST_NONFINITE;
+        else if (tot[0] <= fmax(tol2, c->tol2_in) * c->bb)
+            c->status = ST_CONV;
+        else if (c->it_cur >= maxit)
+            c->status = ST_MAXIT;
     }
 }
 

@@ -87,3 +87,33 @@ def test_direct_solve_off_gives_the_multigrid_result(prec, monkeypatch):
         g.close()
     for c in range(4):
         assert rel(out[0][c], out[1][c]) <= TOL[prec]
+
+
+# conjugate gradients around the direct solve: remainders of its tiles, one and
+# several chunks of a column, every boundary type, a dense mask (whose predictor
+# takes every face by the solid cells' rules)
+@pytest.mark.parametrize("dims,bc,count,edge",
+                         [((16, 12, 8), ("wall",) * 3, 3, (0.15, 0.3)),
+                          ((36, 20, 24), ("periodic", "wall", "slip"), 3, (0.1, 0.2)),
+                          ((8, 12, 144), ("wall", "slip", "periodic"), 3, (0.1, 0.3)),
+                          ((20, 16, 12), ("wall",) * 3, 1, (0.6, 0.6))])
+def test_obstacle_steps_match_the_oracle(dims, bc, count, edge, monkeypatch):
+    box = [d / max(dims) for d in dims]
+    _, solid = inputs.obstacle_boxes(dims, seed=5, count=count, edge=edge)
+    og = oracle.Grid(*dims, *box, re=100.0, bc=bc, solid=solid, rtol=1e-13)
+    init = inputs.random_state(*dims, seed=3, sigma=0.2, bc=bc, solid=solid)
+    want = oracle.copy_state(init)
+    og.step(want, 2e-4, 3)
+    for env in ("1", "0"):
+        monkeypatch.setenv("NS_DIRECT", env)
+        g = Grid(*dims, *box, re=100.0, bc=bc, solid=solid, precision="fp32_refine")
+        st = g.state_from(init)
+        g.profile(True)
+        g.step_fine(st, 2e-4, 3)
+        assert (g.profile_read()["direct_xy"]["launches"] > 0) == (env == "1")
+        got = st.numpy()
+        vg = np.concatenate([np.ravel(got[c][0]) for c in range(3)])
+        vw = np.concatenate([np.ravel(want[c]) for c in range(3)])
+        assert rel(vg, vw) <= TOL["fp32_refine"]
+        assert rel(got[3][0], want[3]) <= TOL["fp32_refine"]
+        g.close()
