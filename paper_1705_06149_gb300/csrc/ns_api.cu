@@ -103,6 +103,7 @@ struct ns_grid {
     bool dir = false;
     // with solid cells (FP32+refine): conjugate gradients it preconditions
     bool cg = false;
+    bool mixed = false;  // FP64 grids: FP32 corrections
     bool hier = false;
     DirPlan<float> dirf{};
     DirPlan<double> dird{};
@@ -524,6 +525,7 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
     constexpr size_t all = DIR_MAX_SMEM / sizeof(T);
     if (P.lines) {
         most(k_dir_x<T, false>, all);
+        most(k_dir_x<T, false, double>, all);
         most(k_dir_x<T, true>, all);
         most(k_dir_y<T, false>, all);
         most(k_dir_y<T, true>, all);
@@ -531,18 +533,19 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
         g->dir_smem = dir_smem_elems(P) * sizeof(T);
         with_dir_shape(P.rb, P.ncol, [&](auto rb, auto nc) {
             most(k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value>, all);
+            most(k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value, double>, all);
             most(k_dir_xy<T, true, decltype(rb)::value, decltype(nc)::value>, all);
         });
     }
     if (!ok) return fail(NS_ERR_CUDA, "ns_create_grid: direct solve shared memory attribute");
     if (solid) {
-        P.precond = 1;
+        P.mode = DM_PRECOND;
         g->cg = true;
         return NS_OK;
     }
     g->dir = true;
     g->mg = true;
-    if (sizeof(T) == 4) {
+    if (g->fp32) {
         g->dir_tile = dir_tile_of(G.n, g->cap, g->d.tile_z);
         NS_TRY(dalloc(g, (void**)&g->dir_ring,
                       (size_t)G.cnt[3] * g->cap * DIR_RING * sizeof(float)));
@@ -562,6 +565,13 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
 // (NS_MG_CLUSTER, NS_MG_BLOCK_CELLS, NS_PERSISTENT), when set, select it;
 // NS_DIRECT=0 turns the direct solve off.  With solid cells, FP32+refine, the
 // same conditions make it the preconditioner of the inner solves.
+//
+// FP64 grids of DIR_MIXED_CELLS cells or more (all states) take FP32 corrections
+// (DM_MIXED) of the FP64 iterate and residual, two or three in the place of
+// one: an FP64 application is bound by its pipe (64^3 x 4 states: 125 us per
+// transform against 8).  4 steps of 64^3 x 4 FP64 3.14 -> 2.47 ms, of one state
+// equal, of smaller ones slower by their launches (32^3 0.58 -> 0.73 ms).
+constexpr long long DIR_MIXED_CELLS = 3 << 17;
 ns_status setup_direct(ns_grid* g) {
     for (const char* v : {"NS_MG_CLUSTER", "NS_MG_BLOCK_CELLS", "NS_PERSISTENT"})
         if (std::getenv(v)) return NS_OK;
@@ -569,9 +579,17 @@ ns_status setup_direct(ns_grid* g) {
     if (env && std::atoi(env) == 0) return NS_OK;
     if (g->geo.solid && !(g->mg && g->fp32)) return NS_OK;
     const double rtol = g->fp32 ? g->d.refine_rtol : g->d.poisson_rtol;
-    const double cond = dir_condition(g->geo.n, g->geo.bc, g->geo.ih2);
+    const Geo& G = g->geo;
+    const double cond = dir_condition(G.n, G.bc, G.ih2);
     if (!(rtol >= 1e-14) || !(cond <= (g->fp32 ? 1e7 : 1e12))) return NS_OK;
-    return g->fp32 ? setup_direct_of<float>(g, g->dirf) : setup_direct_of<double>(g, g->dird);
+    if (g->fp32) return setup_direct_of<float>(g, g->dirf);
+    if (cond <= 1e7 && rtol >= 1e-13 && G.cnt[3] * g->cap >= DIR_MIXED_CELLS) {
+        NS_TRY(setup_direct_of<float>(g, g->dirf));
+        g->dirf.mode = DM_MIXED;
+        g->mixed = g->dir;
+        if (g->dir) return NS_OK;
+    }
+    return setup_direct_of<double>(g, g->dird);
 }
 
 ns_status check_state(const ns_grid* g, const ns_state& s, const char* what) {
@@ -889,15 +907,17 @@ void direct_z(ns_grid* g, const DirPlan<T>& P, T* spec, dim3 zg, dim3 zb, long l
 // e = L^-1 r for every active state: FP32+refine from the residual's high
 // part into the application's slot of the ring, FP64 from kv[1] into kv[4];
 // the spectral planes in kv[3].
-template <typename T>
+template <typename T, typename S = T>
 void direct_apply(ns_grid* g, int batch) {
     const DirPlan<T>& P = dirplan<T>(g);
-    const bool f32 = sizeof(T) == 4;
-    // (as a preconditioner: from kv[1] into kv[6], the spectral planes in kv[7])
-    const T* r = f32 && !g->cg ? (const T*)g->ffb[2] : (const T*)g->kv[1];
+    // FP32+refine: from the residual's high part into the application's slot
+    // of the ring; else from kv[1] into kv[4] (as a preconditioner kv[6]; the
+    // spectral planes then in kv[7])
+    const bool refine = g->fp32 && !g->cg;
+    const S* r = refine ? (const S*)g->ffb[2] : (const S*)g->kv[1];
     T* spec = (T*)g->kv[g->cg ? 7 : 3];
-    T* e = g->cg ? (T*)g->kv[6] : (f32 ? (T*)g->dir_ring : (T*)g->kv[4]);
-    const long long ring = f32 && !g->cg ? dir_stride(g) : 0;
+    T* e = refine ? (T*)g->dir_ring : (T*)g->kv[g->cg ? 6 : 4];
+    const long long ring = refine ? dir_stride(g) : 0;
     const dim3 pg(P.nz * P.xb, batch), zg(ceil_div(P.nx * P.ny, DIR_ZX), batch);
     const dim3 zb(DIR_ZX, P.zc);
     const long long units = P.cells * batch;
@@ -908,7 +928,7 @@ void direct_apply(ns_grid* g, int batch) {
             (unsigned)std::min<long long>(152, (long long)ceil_div(P.nx, P.lines) * P.nz * batch);
         const size_t sx = dir_x_elems(P) * sizeof(T), sy = dir_y_elems(P) * sizeof(T);
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_x<T, false><<<gx, P.ntx, sx, g->stream>>>(P, g->ctl, r, spec, 0, batch)));
+                  (k_dir_x<T, false, S><<<gx, P.ntx, sx, g->stream>>>(P, g->ctl, r, spec, 0, batch)));
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
                   (k_dir_y<T, false><<<gy, P.nty, sy, g->stream>>>(P, g->ctl, spec, batch)));
         direct_z<T>(g, P, spec, zg, zb, units);
@@ -921,7 +941,7 @@ void direct_apply(ns_grid* g, int batch) {
     }
     with_dir_shape(P.rb, P.ncol, [&](auto rb, auto nc) {
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value>
+                  (k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value, S>
                    <<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, r, spec, 0)));
     });
     direct_z<T>(g, P, spec, zg, zb, units);
@@ -945,11 +965,20 @@ void direct_correct(ns_grid* g, int batch) {
                       g->dir_base[1], ffbuf(g), g->dir_part, g->counter,
                       g->d.refine_rtol * g->d.refine_rtol, g->max_outer));
     } else {
-        direct_apply<double>(g, batch);
-        NS_LAUNCH(g, NS_K_REFINE, units,
-                  k_dir_update<<<dim3(L0.ctas, batch), block_dim(), 0, g->stream>>>(
-                      L0, mgbuf<double>(g), g->ctl, (const double*)g->kv[4], g->part_mg,
-                      g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid));
+        auto update = [&](const auto* e) {
+            using E = std::remove_cv_t<std::remove_pointer_t<decltype(e)>>;
+            NS_LAUNCH(g, NS_K_REFINE, units,
+                      k_dir_update<E><<<dim3(L0.ctas, batch), block_dim(), 0, g->stream>>>(
+                          L0, mgbuf<double>(g), g->ctl, e, g->part_mg,
+                          g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid));
+        };
+        if (g->mixed) {
+            direct_apply<float, double>(g, batch);
+            update((const float*)g->kv[4]);
+        } else {
+            direct_apply<double>(g, batch);
+            update((const double*)g->kv[4]);
+        }
     }
 }
 
@@ -1910,7 +1939,7 @@ ns_status parareal_update(ns_grid* g, const void* const fy[4], const void* const
 // Kernels one preconditioned iteration launches (mg_apply twice + 3).
 long long mg_iteration_launches(const ns_grid* g) {
     if (g->dir) {  // the correction counts with FP32+refine's
-        const bool lines = g->fp32 ? g->dirf.lines > 0 : g->dird.lines > 0;
+        const bool lines = g->fp32 || g->mixed ? g->dirf.lines > 0 : g->dird.lines > 0;
         return (lines ? 5 : 3) + (g->fp32 ? 0 : 1);
     }
     if (g->cg) return (g->dirf.lines > 0 ? 5 : 3) + 3;

@@ -35,10 +35,15 @@ constexpr int DIR_ZC = 8;        // cells per chunk of a column
 constexpr int DIR_ZC_LONG = 16;  // the same where nz needs more than 16 chunks
 constexpr int DIR_ZX = 32;       // columns per CTA of k_dir_z
 
+// DM_CORRECT: corrections in the grid's precision; DM_PRECOND: the preconditioner
+// of the conjugate gradients below; DM_MIXED: FP32 corrections of an FP64
+// grid's iterate and residual.
+enum { DM_CORRECT = 0, DM_PRECOND = 1, DM_MIXED = 2 };
+
 template <typename T>
 struct DirPlan {
     int nx, ny, nz, per_z;
-    int precond;   // 1: the transforms precondition the conjugate gradients below
+    int mode;      // DM_*: what the application is part of
     int hx, hy;    // even modes (= length of the folded line) along x, y
     int hxp;       // hx rounded up to 4
     int rb, ncol;  // rows and columns per thread of k_dir_xy
@@ -63,15 +68,10 @@ constexpr int dir_z_threads(int zm) {
 }
 
 // Whether the state takes part in the current application: FP32+refine while
-// its outer residual is above the target; FP64, or as a preconditioner, while
-// it iterates.
-template <typename T> __device__ __forceinline__ bool dir_active(const SliceCtl* c, int precond);
-template <> __device__ __forceinline__ bool dir_active<float>(const SliceCtl* c, int precond) {
-    if (precond) return c->status == ST_ITER;
+// its outer residual is above the target; otherwise while it iterates.
+template <typename T> __device__ __forceinline__ bool dir_active(const SliceCtl* c, int mode) {
+    if (sizeof(T) == 8 || mode != DM_CORRECT) return c->status == ST_ITER;
     return c->o_status == OS_REFINE && c->status != ST_NONFINITE;
-}
-template <> __device__ __forceinline__ bool dir_active<double>(const SliceCtl* c, int) {
-    return c->status == ST_ITER;
 }
 
 // FP32 corrections live in a ring of DIR_RING buffers, one per application;
@@ -79,24 +79,29 @@ template <> __device__ __forceinline__ bool dir_active<double>(const SliceCtl* c
 // (the last three at most).  The residual is scaled by a power of two on its
 // way into the transforms and e unscaled on its way out, so that neither
 // underflows however far the refinement has come (a preconditioned residual
-// carries its scale already and has one buffer).
+// carries its scale already; it and an FP64 grid's corrections have one buffer).
 constexpr int DIR_RING = 4;
 template <typename T>
-__device__ __forceinline__ T dir_scale(const SliceCtl* c, bool inv, int precond);
-template <>
-__device__ __forceinline__ float dir_scale<float>(const SliceCtl* c, bool inv, int precond) {
-    if (precond) return 1.0f;
+__device__ __forceinline__ int dir_slot(const SliceCtl* c, int mode) {
+    return sizeof(T) == 4 && mode == DM_CORRECT ? c->o_steps & (DIR_RING - 1) : 0;
+}
+// log2 of the scale: FP64 grids, from the exponents of (r, r) and the cells.
+__device__ __forceinline__ int dir_shift(double rr, long long cells) {
+    if (!(rr > 0.0)) return 0;
+    const int e = (int)((__double_as_longlong(rr) >> 52) & 0x7ff) - 1023;
+    int l = 0;
+    while (cells >> (l + 1)) ++l;
+    return -((e - l) / 2);
+}
+template <typename T>
+__device__ __forceinline__ double dir_scale(const SliceCtl* c, bool inv, const DirPlan<T>& P) {
+    if (sizeof(T) == 8 || P.mode == DM_PRECOND) return 1.0;
+    if (P.mode == DM_MIXED) {
+        const int e = dir_shift(c->rr, P.cells);
+        return ldexp(1.0, inv ? -e : e);
+    }
     return inv ? 1.0f / c->o_fsc : c->o_fsc;
 }
-template <>
-__device__ __forceinline__ double dir_scale<double>(const SliceCtl*, bool, int) {
-    return 1.0;
-}
-template <typename T> __device__ __forceinline__ int dir_slot(const SliceCtl* c, int precond);
-template <> __device__ __forceinline__ int dir_slot<float>(const SliceCtl* c, int precond) {
-    return precond ? 0 : c->o_steps & (DIR_RING - 1);
-}
-template <> __device__ __forceinline__ int dir_slot<double>(const SliceCtl*, int) { return 0; }
 
 // acc[n][i] += sum_k L[k][i] R[k][n dc], i < RB, n < NC, k ascending; rows of L
 // (16-byte aligned) are ldl apart, of R ldr.  Neighbouring threads hold
@@ -125,6 +130,12 @@ __device__ __forceinline__ void dir_cols(const T* L, int ldl, const T* R, int ld
     }
 }
 
+// An element of the source: FP64 values are scaled before they become FP32.
+template <typename T, typename S>
+__device__ __forceinline__ T dir_in(S v, double scale) {
+    return sizeof(S) > sizeof(T) ? T(v * S(scale)) : T(v);
+}
+
 // Copies n elements (a multiple of 4, both sides 16-byte aligned) to shared
 // memory.
 template <typename T>
@@ -146,14 +157,15 @@ inline size_t dir_smem_elems(const DirPlan<T>& P) {
 // blockIdx.y = state.  Bound by instruction issue (FP64: by the FP64 pipe).
 // 64^3 x 32 states, FP32: 57 us with 4 x 4 tiles of operands both read per
 // thread -> 46 us.
-template <typename T, bool INV, int RB, int NC>
+template <typename T, bool INV, int RB, int NC, typename S = T>
 __global__ void __launch_bounds__(DIR_MAX_THREADS)
-    k_dir_xy(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const T* __restrict__ src,
+    k_dir_xy(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const S* __restrict__ src,
              T* __restrict__ dst, long long ring) {
     pdl_wait();
     const long long s = blockIdx.y;
-    if (!dir_active<T>(ctl + s, P.precond)) return;
-    const T scale = dir_scale<T>(ctl + s, INV, P.precond);
+    if (!dir_active<T>(ctl + s, P.mode)) return;
+    const double dscale = dir_scale<T>(ctl + s, INV, P);
+    const T scale = sizeof(S) > sizeof(T) ? T(1) : T(dscale);  // (else applied to S)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, ny = P.ny, hx = P.hx, hy = P.hy, hxp = P.hxp, hyp = P.hyp;
     const int ldf = P.ldf, cb = P.cb;
@@ -164,8 +176,8 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const int z = (int)blockIdx.x / P.xb;
     const int c0 = ((int)blockIdx.x - z * P.xb) * cb;
     const int t = (int)threadIdx.x, nt = (int)blockDim.x;
-    const T* __restrict__ a = src + s * P.cells + (long long)z * nx * ny;
-    T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s, P.precond) * ring : 0) + s * P.cells +
+    const S* __restrict__ a = src + s * P.cells + (long long)z * nx * ny;
+    T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s, P.mode) * ring : 0) + s * P.cells +
                         (long long)z * nx * ny;
     // the plane: four rows of one column at a time (F[quadrant][column][row]);
     // rows and columns beyond the halves are zero
@@ -177,10 +189,10 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int y = min(y0 + r, hy - 1), ym = INV ? hy + min(y, ny - hy - 1) : ny - 1 - y;
-            q[0].v[r] = a[y * nx + jj];
-            q[1].v[r] = a[y * nx + xm];
-            q[2].v[r] = a[ym * nx + jj];
-            q[3].v[r] = a[ym * nx + xm];
+            q[0].v[r] = dir_in<T>(a[y * nx + jj], dscale);
+            q[1].v[r] = dir_in<T>(a[y * nx + xm], dscale);
+            q[2].v[r] = dir_in<T>(a[ym * nx + jj], dscale);
+            q[3].v[r] = dir_in<T>(a[ym * nx + xm], dscale);
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -307,20 +319,20 @@ inline size_t dir_y_elems(const DirPlan<T>& P) {
 }
 
 template <typename T>
-__device__ __forceinline__ bool dir_any_active(const SliceCtl* ctl, int batch, int precond) {
+__device__ __forceinline__ bool dir_any_active(const SliceCtl* ctl, int batch, int mode) {
     for (int s = 0; s < batch; ++s)
-        if (dir_active<T>(ctl + s, precond)) return true;
+        if (dir_active<T>(ctl + s, mode)) return true;
     return false;
 }
 
 // Along x: rows of src to rows of dst (INV: the application's slot of the
 // ring), P.lines rows at a time.
-template <typename T, bool INV>
+template <typename T, bool INV, typename S = T>
 __global__ void __launch_bounds__(DIR_MAX_THREADS)
-    k_dir_x(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const T* __restrict__ src,
+    k_dir_x(DirPlan<T> P, const SliceCtl* __restrict__ ctl, const S* __restrict__ src,
             T* __restrict__ dst, long long ring, int batch) {
     pdl_wait();
-    if (!dir_any_active<T>(ctl, batch, P.precond)) return;
+    if (!dir_any_active<T>(ctl, batch, P.mode)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, hx = P.hx, hxp = P.hxp, L = P.lines, ldf = L + 4;
     T* R = reinterpret_cast<T*>(smem_raw);
@@ -330,10 +342,11 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const int rows = P.ny * P.nz, blocks = (rows + L - 1) / L, dc = hxp / DIR_LNC;
     for (long long it = blockIdx.x; it < (long long)blocks * batch; it += gridDim.x) {
         const int s = (int)(it / blocks), r0 = (int)(it - (long long)s * blocks) * L;
-        if (!dir_active<T>(ctl + s, P.precond)) continue;
-        const T scale = dir_scale<T>(ctl + s, INV, P.precond);
-        const T* __restrict__ a = src + s * P.cells + (long long)r0 * nx;
-        T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s, P.precond) * ring : 0) + s * P.cells +
+        if (!dir_active<T>(ctl + s, P.mode)) continue;
+        const double dscale = dir_scale<T>(ctl + s, INV, P);
+        const T scale = sizeof(S) > sizeof(T) ? T(1) : T(dscale);
+        const S* __restrict__ a = src + s * P.cells + (long long)r0 * nx;
+        T* __restrict__ o = dst + (INV ? dir_slot<T>(ctl + s, P.mode) * ring : 0) + s * P.cells +
                             (long long)r0 * nx;
         const int nr = min(L, rows - r0);
         __syncthreads();  // the previous block's lines are read
@@ -345,9 +358,9 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
             Q4<T> e, d;
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                const T* __restrict__ line = a + min(y0 + r, nr - 1) * nx;
-                e.v[r] = line[jj];
-                d.v[r] = line[xm];
+                const S* __restrict__ line = a + min(y0 + r, nr - 1) * nx;
+                e.v[r] = dir_in<T>(line[jj], dscale);
+                d.v[r] = dir_in<T>(line[xm], dscale);
             }
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -401,7 +414,7 @@ template <typename T, bool INV>
 __global__ void __launch_bounds__(DIR_MAX_THREADS)
     k_dir_y(DirPlan<T> P, const SliceCtl* __restrict__ ctl, T* __restrict__ spec, int batch) {
     pdl_wait();
-    if (!dir_any_active<T>(ctl, batch, P.precond)) return;
+    if (!dir_any_active<T>(ctl, batch, P.mode)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = P.nx, ny = P.ny, hy = P.hy, hyp = P.hyp, L = P.lines;
     T* Lm = reinterpret_cast<T*>(smem_raw);
@@ -411,7 +424,7 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
     const int xb = (nx + L - 1) / L, blocks = xb * P.nz, dc = L / DIR_LNC;
     for (long long it = blockIdx.x; it < (long long)blocks * batch; it += gridDim.x) {
         const int s = (int)(it / blocks), r = (int)(it - (long long)s * blocks);
-        if (!dir_active<T>(ctl + s, P.precond)) continue;
+        if (!dir_active<T>(ctl + s, P.mode)) continue;
         const int z = r / xb, x0 = (r - z * xb) * L, nc = min(L, nx - x0);
         T* __restrict__ a = spec + s * P.cells + (long long)z * nx * ny + x0;
         __syncthreads();
@@ -462,7 +475,7 @@ __global__ void __launch_bounds__(dir_z_threads<T>(ZM))
     k_dir_z(DirPlan<T> P, SliceCtl* __restrict__ ctl, T* __restrict__ a) {
     pdl_wait();
     const long long s = blockIdx.y;
-    if (!dir_active<T>(ctl + s, P.precond)) return;
+    if (!dir_active<T>(ctl + s, P.mode)) return;
     __shared__ T sY[32][DIR_ZX], sL[32][DIR_ZX], sP[32][DIR_ZX], sX[32][DIR_ZX], sE[DIR_ZX];
     const int lane = (int)threadIdx.x, ch = (int)threadIdx.y, C = (int)blockDim.y;
     const int cols = P.nx * P.ny, nz = P.nz;
@@ -551,7 +564,7 @@ __global__ void __launch_bounds__(dir_z_threads<T>(ZM))
         }
     if (blockIdx.x == 0 && lane == 0 && ch == 0) {
         // an application counts as an iteration (no other CTA reads these)
-        if (sizeof(T) == 4 && !P.precond) {
+        if (sizeof(T) == 4 && P.mode == DM_CORRECT) {
             ctl[s].it_cur = 1;
             ctl[s].total_iters += 1;
         }
@@ -785,7 +798,7 @@ __global__ void __launch_bounds__(NTHREADS)
     pdl_wait();
     const long long s = blockIdx.y;
     SliceCtl* c = ctl + s;
-    if (!dir_active<float>(c, 0)) return;
+    if (!dir_active<float>(c, DM_CORRECT)) return;
     const long long off = s * L.cells;
     const int step = c->o_steps;
     const float* __restrict__ e = ring + (step & (DIR_RING - 1)) * stride + off;
@@ -946,16 +959,29 @@ __global__ void __launch_bounds__(NTHREADS)
 // mean of the residual, made by rounding, is out of every correction's reach
 // (L has no range there): it is taken out of the next residual, or it would
 // be the floor of a solve whose right side is itself close to rounding.
+// E = float: the FP32 corrections of DM_MIXED, L e in float-float (48 bits of a
+// correction's own size; FP32 pipe).
+template <typename E>
+__device__ __forceinline__ double dir_lap64(const Lev& L, const Vals7<E>& v);
+template <>
+__device__ __forceinline__ double dir_lap64<double>(const Lev& L, const Vals7<double>& v) {
+    return lap_vals<double>(L, v);
+}
+template <>
+__device__ __forceinline__ double dir_lap64<float>(const Lev& L, const Vals7<float>& v) {
+    return ff_to_double(lap_ff_vals(L, v));
+}
+template <typename E>
 __global__ void __launch_bounds__(NTHREADS)
     k_dir_update(Lev L, MgBuf<double> mb, SliceCtl* __restrict__ ctl,
-                 const double* __restrict__ evec, double* __restrict__ part, double tol2,
+                 const E* __restrict__ evec, double* __restrict__ part, double tol2,
                  int maxit, int nfluid) {
     pdl_wait();
     const long long s = blockIdx.y;
     SliceCtl* c = ctl + s;
     if (c->status != ST_ITER) return;
     const long long off = s * L.cells;
-    const double* __restrict__ e = evec + off;
+    const E* __restrict__ e = evec + off;
     double* __restrict__ x = mb.x + off;
     double* __restrict__ r = mb.r + off;
     int i, j, k0;
@@ -967,13 +993,13 @@ __global__ void __launch_bounds__(NTHREADS)
         const NbrXY xy = make_nbr_xy(L, i, j);
         const int plane = L.n[0] * L.n[1];
         for (int kb = k0; kb < k1; kb += MG_ZB) {
-            Vals7<double> ev[MG_ZB];
+            Vals7<E> ev[MG_ZB];
             double xo[MG_ZB], ro[MG_ZB];
 #pragma unroll
             for (int q = 0; q < MG_ZB; ++q) {
                 if (kb + q < k1) {
                     const Nbr nb = nbr_at(L, xy, kb + q);
-                    ev[q] = load7<double>(nb, e);
+                    ev[q] = load7<E>(nb, e);
                     xo[q] = x[nb.c];
                     ro[q] = r[nb.c];
                 }
@@ -983,7 +1009,7 @@ __global__ void __launch_bounds__(NTHREADS)
                 if (kb + q < k1) {
                     const int id = (kb + q) * plane + xy.base;
                     const double xv = xo[q] + ev[q].c;
-                    const double rv = ro[q] - lap_vals<double>(L, ev[q]) - rmean;
+                    const double rv = ro[q] - dir_lap64<E>(L, ev[q]) - rmean;
                     x[id] = xv;
                     r[id] = rv;
                     rr += rv * rv;

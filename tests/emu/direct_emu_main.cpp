@@ -4,7 +4,8 @@
 // inactive), every CTA as host threads, and writes e.
 //
 // usage: direct_emu T nx ny nz bcx bcy bcz lx ly lz planes in.bin out.bin
-//   planes: of a call, 0: the transforms one axis at a time; T: f or d; in.bin: r, two states; out.bin: e, two states (the inactive
+//   planes: of a call, 0: the transforms one axis at a time; T: f, d, or m (an FP64
+//   residual, FP32 transforms); in.bin: r, two states; out.bin: e, two states (the inactive
 //   one's untouched zeros).
 
 #include <functional>
@@ -34,7 +35,7 @@ static void launch(int gx, int bx, int by, size_t smem, const std::function<void
         }
 }
 
-template <typename T>
+template <typename T, typename S>
 static int run(char** argv) {
     int n[3], bc[3];
     double ih2[3];
@@ -56,19 +57,25 @@ static int run(char** argv) {
     P.ly[1] = tab.data() + off[3];
     P.col = tab.data() + off[4];
     const size_t N = (size_t)P.cells;
-    std::vector<T> r(2 * N), spec(2 * N, T(0)), e(2 * N, T(0));
+    std::vector<S> r(2 * N);
+    std::vector<T> spec(2 * N, T(0)), e(2 * N, T(0));
     FILE* f = fopen(argv[12], "rb");
-    if (!f || fread(r.data(), sizeof(T), 2 * N, f) != 2 * N) return 3;
+    if (!f || fread(r.data(), sizeof(S), 2 * N, f) != 2 * N) return 3;
     fclose(f);
     SliceCtl ctl[2] = {};
     ctl[0].status = ST_ITER;
     ctl[0].o_status = OS_REFINE;
     ctl[0].o_fsc = 4.0f;  // the scale FP32 residuals carry through the transforms
     ctl[1].o_fsc = 4.0f;
+    if (sizeof(S) > sizeof(T)) {  // scaled from the residual's norm
+        P.mode = DM_MIXED;
+        ctl[0].o_status = OS_DONE;
+        for (size_t q = 0; q < N; ++q) ctl[0].rr += double(r[q]) * double(r[q]);
+    }
     ctl[1].status = ST_CONV;
     ctl[1].o_status = OS_DONE;
     const size_t smem = dir_smem_elems(P) * sizeof(T);
-    auto xy = [&](auto inv, const T* src, T* dst) {
+    auto xy = [&](auto inv, const auto* src, T* dst) {
         constexpr bool INV = decltype(inv)::value;
         auto go = [&](auto rb, auto nc) {
             launch(P.nz * P.xb, P.nt, 1, smem,
@@ -115,5 +122,6 @@ static int run(char** argv) {
 
 int main(int argc, char** argv) {
     if (argc != 14) return 1;
-    return argv[1][0] == 'f' ? run<float>(argv) : run<double>(argv);
+    return argv[1][0] == 'f' ? run<float, float>(argv)
+                             : argv[1][0] == 'd' ? run<double, double>(argv) : run<float, double>(argv);
 }

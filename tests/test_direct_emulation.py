@@ -97,17 +97,17 @@ CASES = [
 ]
 
 
-@pytest.mark.parametrize("prec", ["f", "d"])
+@pytest.mark.parametrize("prec", ["f", "d", "m"])
 @pytest.mark.parametrize("case", range(len(CASES)))
 def test_direct_solve_inverts_the_laplacian(emulator, case, prec):
     exe, d = emulator
     n, bc, box, planes = CASES[case]
-    t = np.float32 if prec == "f" else np.float64
+    t = np.float64 if prec == "d" else np.float32
     h = [box[a] / n[a] for a in range(3)]
     rng = np.random.default_rng(case)
     r = rng.normal(size=(2,) + n[::-1])
     r -= r.mean(axis=(1, 2, 3), keepdims=True)
-    r = r.astype(t)
+    r = r.astype(np.float32 if prec == "f" else np.float64)
     fin, fout = d / "r.bin", d / "e.bin"
     r.tofile(fin)
     args = [exe, prec, *map(str, n), *(str(BC[x]) for x in bc), *map(repr, box), str(planes),
