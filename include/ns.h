@@ -101,8 +101,9 @@ typedef struct {
                                 NS_MG_CLUSTER=0 at ns_create_grid turns that off. */
     int tile_z;              /* cells each thread marches along z in the stencil and
                                 solver kernels: an even number >= 2 (clamped to nz);
-                                0: 8.  Results depend on it at rounding level (it
-                                fixes the order of the per-state reductions).       */
+                                0: 8, less on small grids.  Results depend on it at
+                                rounding level (it fixes the order of the per-state
+                                reductions).                                        */
     int parareal_chunk;      /* ns_parareal_iterate: slices per chunk of the fine
                                 sweep (> 0).  With the multigrid solver the chunks'
                                 sweeps and coarse chains are graph launches

@@ -317,8 +317,14 @@ void setup_geo(ns_grid* g) {
     G.finv_re = (float)G.inv_re;
     // cells per thread along z: fixed per grid (not per batch) so that every
     // state is reduced over the same CTAs whatever the batch size; an even
-    // number so that the multigrid restriction pairs stay inside a CTA
-    const int tz_want = d.tile_z > 0 ? std::max(2, d.tile_z & ~1) : 8;
+    // number so that the multigrid restriction pairs stay inside a CTA.  By
+    // default 8, halved (to 2) while a state's tiles leave half of the SMs
+    // without one: the march is a chain of latencies (a 16^3 FP64 step 126 ->
+    // 112 us, 32^3 144 -> 125 us).
+    int tz_want = d.tile_z > 0 ? std::max(2, d.tile_z & ~1) : 8;
+    while (d.tile_z <= 0 && tz_want > 2 &&
+           ceil_div(G.n[0], TX) * ceil_div(G.n[1], TY) * ceil_div(G.n[2], tz_want) < 76)
+        tz_want /= 2;
     G.tz = std::min(tz_want, G.n[2]);
     G.bx = ceil_div(G.n[0], TX);
     G.by = ceil_div(G.n[1], TY);
