@@ -675,6 +675,24 @@ void prof_end(ns_grid* g) {
         prof_end((g));                    \
     } while (0)
 
+// Launches a kernel whose first statement is pdl_wait: on the stream it may
+// become resident while the kernel before it ends (captured, the graph's edges
+// decide).
+template <typename... P, typename... A>
+void launch_dep(ns_grid* g, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... a) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = g->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = g->capturing ? 0 : 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(a)...);
+}
+
 ns_status poll_ctl(ns_grid* g, int batch) {
     NS_CUDA(cudaMemcpyAsync(g->h_ctl, g->ctl, sizeof(SliceCtl) * batch, cudaMemcpyDeviceToHost,
                             g->stream));
@@ -793,14 +811,14 @@ void launch_refine_init_ff(ns_grid* g, int batch, const double* p_in, double oto
     if (g->dir) mb.r = mb.rhat = (float*)g->kv[3];
     if (p_in)
         NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
-                  k_mg_refine_init_ff<true><<<grid, blk, 0, g->stream>>>(
-                      L0, mb, g->ctl, g->part_div, g->geo.n_fluid, g->b, p_in, ffbuf(g),
-                      g->part_mg, otol2, itol2, g->maxit));
+                  launch_dep(g, k_mg_refine_init_ff<true>, grid, blk, 0, L0, mb, g->ctl,
+                             g->part_div, g->geo.n_fluid, g->b, p_in, ffbuf(g), g->part_mg, otol2,
+                             itol2, g->maxit));
     else
         NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
-                  k_mg_refine_init_ff<false><<<grid, blk, 0, g->stream>>>(
-                      L0, mb, g->ctl, g->part_div, g->geo.n_fluid, g->b, nullptr, ffbuf(g),
-                      g->part_mg, otol2, itol2, g->maxit));
+                  launch_dep(g, k_mg_refine_init_ff<false>, grid, blk, 0, L0, mb, g->ctl,
+                             g->part_div, g->geo.n_fluid, g->b, nullptr, ffbuf(g), g->part_mg,
+                             otol2, itol2, g->maxit));
 }
 
 // One application of the V-cycle to the level-0 vector the source kernel of
@@ -904,10 +922,10 @@ template <typename T>
 void direct_z(ns_grid* g, const DirPlan<T>& P, T* spec, dim3 zg, dim3 zb, long long units) {
     if (P.zm == DIR_ZC)
         NS_LAUNCH(g, NS_K_DIRECT_Z, units,
-                  (k_dir_z<T, DIR_ZC><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
+                  (launch_dep(g, k_dir_z<T, DIR_ZC>, zg, zb, 0, P, g->ctl, spec)));
     else
         NS_LAUNCH(g, NS_K_DIRECT_Z, units,
-                  (k_dir_z<T, DIR_ZC_LONG><<<zg, zb, 0, g->stream>>>(P, g->ctl, spec)));
+                  (launch_dep(g, k_dir_z<T, DIR_ZC_LONG>, zg, zb, 0, P, g->ctl, spec)));
 }
 
 // e = L^-1 r for every active state: FP32+refine from the residual's high
@@ -934,27 +952,28 @@ void direct_apply(ns_grid* g, int batch) {
             (unsigned)std::min<long long>(152, (long long)ceil_div(P.nx, P.lines) * P.nz * batch);
         const size_t sx = dir_x_elems(P) * sizeof(T), sy = dir_y_elems(P) * sizeof(T);
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_x<T, false, S><<<gx, P.ntx, sx, g->stream>>>(P, g->ctl, r, spec, 0, batch)));
+                  (launch_dep(g, k_dir_x<T, false, S>, gx, P.ntx, sx, P, g->ctl, r, spec, 0,
+                              batch)));
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_y<T, false><<<gy, P.nty, sy, g->stream>>>(P, g->ctl, spec, batch)));
+                  (launch_dep(g, k_dir_y<T, false>, gy, P.nty, sy, P, g->ctl, spec, batch)));
         direct_z<T>(g, P, spec, zg, zb, units);
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_y<T, true><<<gy, P.nty, sy, g->stream>>>(P, g->ctl, spec, batch)));
+                  (launch_dep(g, k_dir_y<T, true>, gy, P.nty, sy, P, g->ctl, spec, batch)));
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_x<T, true><<<gx, P.ntx, sx, g->stream>>>(P, g->ctl, spec, e, ring,
-                                                                 batch)));
+                  (launch_dep(g, k_dir_x<T, true>, gx, P.ntx, sx, P, g->ctl, spec, e, ring,
+                              batch)));
         return;
     }
     with_dir_shape(P.rb, P.ncol, [&](auto rb, auto nc) {
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value, S>
-                   <<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, r, spec, 0)));
+                  (launch_dep(g, k_dir_xy<T, false, decltype(rb)::value, decltype(nc)::value, S>,
+                              pg, P.nt, g->dir_smem, P, g->ctl, r, spec, 0)));
     });
     direct_z<T>(g, P, spec, zg, zb, units);
     with_dir_shape(P.rb, P.ncol, [&](auto rb, auto nc) {
         NS_LAUNCH(g, NS_K_DIRECT_XY, units,
-                  (k_dir_xy<T, true, decltype(rb)::value, decltype(nc)::value>
-                   <<<pg, P.nt, g->dir_smem, g->stream>>>(P, g->ctl, spec, e, ring)));
+                  (launch_dep(g, k_dir_xy<T, true, decltype(rb)::value, decltype(nc)::value>, pg,
+                              P.nt, g->dir_smem, P, g->ctl, spec, e, ring)));
     });
 }
 
@@ -966,17 +985,17 @@ void direct_correct(ns_grid* g, int batch) {
     if (g->fp32) {
         direct_apply<float>(g, batch);
         NS_LAUNCH(g, NS_K_REFINE, units,
-                  k_dir_refine<<<dim3(g->dir_tile.ctas, batch), block_dim(), 0, g->stream>>>(
-                      L0, g->dir_tile, g->ctl, g->dir_ring, dir_stride(g), g->dir_base[0],
-                      g->dir_base[1], ffbuf(g), g->dir_part, g->counter,
-                      g->d.refine_rtol * g->d.refine_rtol, g->max_outer));
+                  launch_dep(g, k_dir_refine, dim3(g->dir_tile.ctas, batch), block_dim(), 0, L0,
+                             g->dir_tile, g->ctl, g->dir_ring, dir_stride(g), g->dir_base[0],
+                             g->dir_base[1], ffbuf(g), g->dir_part, g->counter,
+                             g->d.refine_rtol * g->d.refine_rtol, g->max_outer));
     } else {
         auto update = [&](const auto* e) {
             using E = std::remove_cv_t<std::remove_pointer_t<decltype(e)>>;
             NS_LAUNCH(g, NS_K_REFINE, units,
-                      k_dir_update<E><<<dim3(L0.ctas, batch), block_dim(), 0, g->stream>>>(
-                          L0, mgbuf<double>(g), g->ctl, e, g->part_mg,
-                          g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid));
+                      launch_dep(g, k_dir_update<E>, dim3(L0.ctas, batch), block_dim(), 0, L0,
+                                 mgbuf<double>(g), g->ctl, e, g->part_mg,
+                                 g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid));
         };
         if (g->mixed) {
             direct_apply<float, double>(g, batch);
@@ -1003,12 +1022,12 @@ ns_status mg_iteration(ns_grid* g, int batch, double tol2, int zero_start) {
         const T* z = (const T*)g->kv[6];
         direct_apply<T>(g, batch);
         NS_LAUNCH(g, NS_K_MG_LAP_T, 0,
-                  k_cg_dot<T><<<grid, blk, 0, g->stream>>>(L0, mb, z, g->ctl, g->part_mg));
+                  launch_dep(g, k_cg_dot<T>, grid, blk, 0, L0, mb, z, g->ctl, g->part_mg));
         NS_LAUNCH(g, NS_K_MG_LAP_V, 0,
-                  k_cg_lap<T><<<grid, blk, 0, g->stream>>>(L0, mb, z, g->ctl, g->part_mg));
+                  launch_dep(g, k_cg_lap<T>, grid, blk, 0, L0, mb, z, g->ctl, g->part_mg));
         NS_LAUNCH(g, NS_K_KRYLOV_C, 0,
-                  k_cg_update<T><<<grid, blk, 0, g->stream>>>(L0, mb, g->ctl, g->part_mg, tol2,
-                                                              g->maxit));
+                  launch_dep(g, k_cg_update<T>, grid, blk, 0, L0, mb, g->ctl, g->part_mg, tol2,
+                             g->maxit));
         NS_CUDA(cudaGetLastError());
         return NS_OK;
     }
@@ -1386,9 +1405,9 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
         MgBuf<double> mb = mgbuf<double>(g);
         const double tol2 = g->d.poisson_rtol * g->d.poisson_rtol;
         NS_LAUNCH(g, NS_K_SOLVE_INIT, 0,
-                  k_mg_init_warm<double><<<grid, blk, 0, g->stream>>>(
-                      L0, mb, g->ctl, g->part_div, g->geo.n_fluid, g->b,
-                      p_in ? p_in : g->p_prev, g->part_mg, tol2, g->maxit));
+                  launch_dep(g, k_mg_init_warm<double>, grid, blk, 0, L0, mb, g->ctl, g->part_div,
+                             g->geo.n_fluid, g->b, p_in ? p_in : g->p_prev, g->part_mg, tol2,
+                             g->maxit));
         NS_CUDA(cudaGetLastError());
         cudaGraphConditionalHandle h;
         NS_TRY(make_handle(g->stream, &h));
@@ -1412,9 +1431,8 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
     return add_while(g, g->body_stream[0], h, [&]() -> ns_status {
         NS_TRY(mg_iteration<float>(g, batch, itol2, 1));
         NS_LAUNCH(g, NS_K_REFINE, 0,
-                  k_mg_refine_update_ff<<<grid, blk, 0, g->stream>>>(
-                      L0, mb, g->ctl, ffbuf(g), g->geo.n_fluid, g->part_mg, otol2, itol2,
-                      g->maxit, g->max_outer, 1));
+                  launch_dep(g, k_mg_refine_update_ff, grid, blk, 0, L0, mb, g->ctl, ffbuf(g),
+                             g->geo.n_fluid, g->part_mg, otol2, itol2, g->maxit, g->max_outer, 1));
         NS_CUDA(cudaGetLastError());
         return loop_cond(g, batch, h, LC_REFINE_ITER, cap_refine);
     });
@@ -1485,10 +1503,10 @@ ns_status solve_pressure_direct(ns_grid* g, int batch, const double* p_in) {
         g->dir_base[1] = g->ffb[1];
     } else {
         NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
-                  k_mg_init_warm<double><<<dim3(L0.ctas, batch), block_dim(), 0, g->stream>>>(
-                      L0, mgbuf<double>(g), g->ctl, g->part_div, g->geo.n_fluid, g->b,
-                      p_in ? p_in : g->p_prev, g->part_mg,
-                      g->d.poisson_rtol * g->d.poisson_rtol, g->maxit));
+                  launch_dep(g, k_mg_init_warm<double>, dim3(L0.ctas, batch), block_dim(), 0, L0,
+                             mgbuf<double>(g), g->ctl, g->part_div, g->geo.n_fluid, g->b,
+                             p_in ? p_in : g->p_prev, g->part_mg,
+                             g->d.poisson_rtol * g->d.poisson_rtol, g->maxit));
     }
     return direct_loop(g, batch);
 }
@@ -1501,19 +1519,19 @@ void direct_velocity(ns_grid* g, int batch, float* const fs[3], float* const vel
                      double dt, float* const w_next[2]) {
     const Geo& G = g->geo;
     NS_LAUNCH(g, NS_K_CORRECT, G.cnt[3] * batch,
-              k_dir_correct<INCR><<<dim3(g->dir_tile.ctas, batch), block_dim(), 0, g->stream>>>(
-                  g->plan.lev[0], g->dir_tile, g->ctl, fs[0], fs[1], fs[2], vel[0], vel[1],
-                  vel[2], ffbuf(g), g->dir_base[0], g->dir_base[1], g->dir_ring, dir_stride(g),
-                  w_next ? w_next[0] : nullptr, w_next ? w_next[1] : nullptr, p, dt_ih(G, dt),
-                  G.cnt[0], G.cnt[1], G.cnt[2]));
+              launch_dep(g, k_dir_correct<INCR>, dim3(g->dir_tile.ctas, batch), block_dim(), 0,
+                         g->plan.lev[0], g->dir_tile, g->ctl, fs[0], fs[1], fs[2], vel[0], vel[1],
+                         vel[2], ffbuf(g), g->dir_base[0], g->dir_base[1], g->dir_ring,
+                         dir_stride(g), w_next ? w_next[0] : nullptr, w_next ? w_next[1] : nullptr,
+                         p, dt_ih(G, dt), G.cnt[0], G.cnt[1], G.cnt[2]));
 }
 
 // The caller's FP64 pressure as warm start (ffb[4..5]) and last pressure.
 void direct_load_p(ns_grid* g, int batch, const double* p) {
     const long long cells = g->geo.cnt[3] * batch;
     NS_LAUNCH(g, NS_K_INNER_INIT, cells,
-              k_dir_load_p<<<(unsigned)((cells + NTHREADS - 1) / NTHREADS), block_dim(), 0,
-                             g->stream>>>(cells, p, ffbuf(g)));
+              launch_dep(g, k_dir_load_p, (unsigned)((cells + NTHREADS - 1) / NTHREADS),
+                         block_dim(), 0, cells, p, ffbuf(g)));
 }
 
 // Start of an FP32+refine solve: b = D fs / dt (with vel: D (vel + fs) / dt),
@@ -1527,16 +1545,16 @@ void direct_start(ns_grid* g, int batch, float* const fs[3], float* const vel[3]
     const dim3 grid(g->dir_tile.ctas, batch), blk = block_dim();
     if (vel)
         NS_LAUNCH(g, NS_K_SOLVE_INIT, G.cnt[3] * batch,
-                  k_dir_start<true><<<grid, blk, 0, g->stream>>>(
-                      g->plan.lev[0], g->dir_tile, g->ctl, fs[0], fs[1], fs[2], vel[0], vel[1],
-                      vel[2], warm[0], warm[1], ffbuf(g), idt, ihx, ihy, ihz, G.cnt[0], G.cnt[1],
-                      G.cnt[2], g->dir_part, g->counter, otol2, g->max_outer));
+                  launch_dep(g, k_dir_start<true>, grid, blk, 0, g->plan.lev[0], g->dir_tile,
+                             g->ctl, fs[0], fs[1], fs[2], vel[0], vel[1], vel[2], warm[0], warm[1],
+                             ffbuf(g), idt, ihx, ihy, ihz, G.cnt[0], G.cnt[1], G.cnt[2],
+                             g->dir_part, g->counter, otol2, g->max_outer));
     else
         NS_LAUNCH(g, NS_K_SOLVE_INIT, G.cnt[3] * batch,
-                  k_dir_start<false><<<grid, blk, 0, g->stream>>>(
-                      g->plan.lev[0], g->dir_tile, g->ctl, fs[0], fs[1], fs[2], nullptr, nullptr,
-                      nullptr, warm[0], warm[1], ffbuf(g), idt, ihx, ihy, ihz, G.cnt[0], G.cnt[1],
-                      G.cnt[2], g->dir_part, g->counter, otol2, g->max_outer));
+                  launch_dep(g, k_dir_start<false>, grid, blk, 0, g->plan.lev[0], g->dir_tile,
+                             g->ctl, fs[0], fs[1], fs[2], nullptr, nullptr, nullptr, warm[0],
+                             warm[1], ffbuf(g), idt, ihx, ihy, ihz, G.cnt[0], G.cnt[1], G.cnt[2],
+                             g->dir_part, g->counter, otol2, g->max_outer));
     g->dir_base[0] = warm[0];
     g->dir_base[1] = warm[1];
 }
@@ -1574,9 +1592,9 @@ ns_status solve_pressure_mg(ns_grid* g, int batch, const double* p_in) {
         MgBuf<double> mb = mgbuf<double>(g);
         const double tol2 = g->d.poisson_rtol * g->d.poisson_rtol;
         NS_LAUNCH(g, NS_K_SOLVE_INIT, L0.cells * batch,
-                  k_mg_init_warm<double><<<grid, blk, 0, g->stream>>>(
-                      L0, mb, g->ctl, g->part_div, g->geo.n_fluid, g->b,
-                      p_in ? p_in : g->p_prev, g->part_mg, tol2, g->maxit));
+                  launch_dep(g, k_mg_init_warm<double>, grid, blk, 0, L0, mb, g->ctl, g->part_div,
+                             g->geo.n_fluid, g->b, p_in ? p_in : g->p_prev, g->part_mg, tol2,
+                             g->maxit));
         NS_CUDA(cudaGetLastError());
         NS_TRY(run_mg<double>(g, batch, g->d.poisson_rtol, 0, &max_iters, &max_rel));
     } else {
@@ -1596,9 +1614,9 @@ ns_status solve_pressure_mg(ns_grid* g, int batch, const double* p_in) {
             if (st != NS_OK && st != NS_ERR_NOT_CONVERGED) return st;
             g_last_error.clear();
             NS_LAUNCH(g, NS_K_REFINE, L0.cells * batch,
-                      k_mg_refine_update_ff<<<grid, blk, 0, g->stream>>>(
-                          L0, mb, g->ctl, ffbuf(g), g->geo.n_fluid, g->part_mg, otol2, itol2,
-                          g->maxit, g->max_outer, 0));
+                      launch_dep(g, k_mg_refine_update_ff, grid, blk, 0, L0, mb, g->ctl, ffbuf(g),
+                                 g->geo.n_fluid, g->part_mg, otol2, itol2, g->maxit, g->max_outer,
+                                 0));
             NS_CUDA(cudaGetLastError());
         }
         for (int s = 0; s < batch; ++s) {
@@ -1757,13 +1775,13 @@ void launch_predict(ns_grid* g, int batch, const T* u, const T* v, const T* w, T
         const int tbx = ceil_div(G.n[0], PX), tby = ceil_div(G.n[1], PY),
                   tbz = ceil_div(G.n[2], PZ);
         const size_t smem = 3 * (size_t)ptile_elems<PY, PZ, PX>() * sizeof(T);
-        k_predict_tile<T, INCR, PY, PZ, PX><<<dim3(tbx * tby * tbz, batch), PX * PY, smem,
-                                              g->stream>>>(G, u, v, w, fu, fv, fw, dt, tbx, tby);
+        launch_dep(g, k_predict_tile<T, INCR, PY, PZ, PX>, dim3(tbx * tby * tbz, batch), PX * PY,
+                   smem, G, u, v, w, fu, fv, fw, dt, tbx, tby);
     });
     if (g->near_count)
-        k_predict_faces<T, INCR>
-            <<<dim3((unsigned)((g->near_count + NTHREADS - 1) / NTHREADS), batch), block_dim(), 0,
-               g->stream>>>(G, u, v, w, fu, fv, fw, dt, g->near_faces, g->near_count);
+        launch_dep(g, k_predict_faces<T, INCR>,
+                   dim3((unsigned)((g->near_count + NTHREADS - 1) / NTHREADS), batch), block_dim(),
+                   0, G, u, v, w, fu, fv, fw, dt, g->near_faces, g->near_count);
 }
 
 // Shared memory limit of the predictor instantiation the grid uses (a value
@@ -1818,9 +1836,9 @@ ns_status step_impl(ns_grid* g, const ns_state& io, double dt, int nsteps) {
         }
         const bool with_u = INCR && n == 0;
         NS_LAUNCH(g, NS_K_DIVERGENCE, cells,
-                  k_divergence<T><<<gcell, block_dim(), 0, g->stream>>>(
-                      G, fu, fv, fw, with_u ? u : nullptr, with_u ? v : nullptr,
-                      with_u ? w : nullptr, g->b, g->part_div, 1.0 / dt));
+                  launch_dep(g, k_divergence<T>, gcell, block_dim(), 0, G, fu, fv, fw,
+                             with_u ? u : nullptr, with_u ? v : nullptr, with_u ? w : nullptr, g->b,
+                             g->part_div, 1.0 / dt));
         NS_CUDA(cudaGetLastError());
         // multigrid path: from the second step of a call the solve starts from
         // 2 p^n - p^(n-1), which the previous correction wrote (null p_in)
@@ -1829,15 +1847,13 @@ ns_status step_impl(ns_grid* g, const ns_state& io, double dt, int nsteps) {
         const bool keep = g->mg && n + 1 < nsteps;
         if (INCR && g->mg)
             NS_LAUNCH(g, NS_K_CORRECT, cells,
-                      k_correct_ff<INCR><<<gface, block_dim(), 0, g->stream>>>(
-                          G, g->ctl, (const float*)fu, (const float*)fv, (const float*)fw,
-                          (float*)u, (float*)v, (float*)w, ffbuf(g), p, dt_ih(G, dt),
-                          keep ? 1 : 0));
+                      launch_dep(g, k_correct_ff<INCR>, gface, block_dim(), 0, G, g->ctl,
+                                 (const float*)fu, (const float*)fv, (const float*)fw, (float*)u,
+                                 (float*)v, (float*)w, ffbuf(g), p, dt_ih(G, dt), keep ? 1 : 0));
         else
             NS_LAUNCH(g, NS_K_CORRECT, cells,
-                      k_correct<T, INCR><<<gface, block_dim(), 0, g->stream>>>(
-                          G, g->ctl, fu, fv, fw, u, v, w, x0, x1, p, dt,
-                          keep ? g->p_prev : nullptr));
+                      launch_dep(g, k_correct<T, INCR>, gface, block_dim(), 0, G, g->ctl, fu, fv,
+                                 fw, u, v, w, x0, x1, p, dt, keep ? g->p_prev : nullptr));
         NS_CUDA(cudaGetLastError());
         if (!g->capturing) g->stats.steps += B;
     }
@@ -1882,8 +1898,8 @@ ns_status project_impl(ns_grid* g, const ns_state& io, double* phi = nullptr) {
         return NS_OK;
     }
     NS_LAUNCH(g, NS_K_DIVERGENCE, G.cnt[3] * B,
-              k_divergence<T><<<gcell, block_dim(), 0, g->stream>>>(
-                  G, u, v, w, nullptr, nullptr, nullptr, g->b, g->part_div, 1.0));
+              launch_dep(g, k_divergence<T>, gcell, block_dim(), 0, G, u, v, w, nullptr, nullptr,
+                         nullptr, g->b, g->part_div, 1.0));
     if (!phi) {
         // zero warm start: p64[1] is free scratch at this point in both precisions
         NS_CUDA(cudaMemsetAsync(g->p64[1], 0, sizeof(double) * G.cnt[3] * B, g->stream));
@@ -1894,13 +1910,13 @@ ns_status project_impl(ns_grid* g, const ns_state& io, double* phi = nullptr) {
     const double* x1 = g->fp32 ? g->p64[1] : (const double*)g->kv[0];
     if (g->fp32 && g->mg)
         NS_LAUNCH(g, NS_K_CORRECT, G.cnt[3] * B,
-                  k_correct_ff<false><<<gface, block_dim(), 0, g->stream>>>(
-                      G, g->ctl, (const float*)u, (const float*)v, (const float*)w, (float*)u,
-                      (float*)v, (float*)w, ffbuf(g), phi, dt_ih(G, 1.0), 0));
+                  launch_dep(g, k_correct_ff<false>, gface, block_dim(), 0, G, g->ctl,
+                             (const float*)u, (const float*)v, (const float*)w, (float*)u,
+                             (float*)v, (float*)w, ffbuf(g), phi, dt_ih(G, 1.0), 0));
     else
         NS_LAUNCH(g, NS_K_CORRECT, G.cnt[3] * B,
-                  k_correct<T, false><<<gface, block_dim(), 0, g->stream>>>(
-                      G, g->ctl, u, v, w, u, v, w, x0, x1, phi, 1.0));
+                  launch_dep(g, k_correct<T, false>, gface, block_dim(), 0, G, g->ctl, u, v, w, u,
+                             v, w, x0, x1, phi, 1.0, nullptr));
     NS_CUDA(cudaGetLastError());
     return persist_settle(g);
 }
@@ -3133,22 +3149,22 @@ ns_status ns_poisson_solve(ns_grid* grid, const double* b, double* p, int batch,
         direct_velocity<false>(grid, batch, fs, fs, p, 0.0, nullptr);
     } else if (grid->fp32 && grid->mg)
         NS_LAUNCH(grid, NS_K_CORRECT, G.cnt[3] * batch,
-                  k_correct_ff<false><<<gface, block_dim(), 0, grid->stream>>>(
-                      G, grid->ctl, (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2],
-                      (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2], ffbuf(grid),
-                      p, dt_ih(G, 0.0), 0));
+                  launch_dep(grid, k_correct_ff<false>, gface, block_dim(), 0, G, grid->ctl,
+                             (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2],
+                             (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2],
+                             ffbuf(grid), p, dt_ih(G, 0.0), 0));
     else if (grid->fp32)
         NS_LAUNCH(grid, NS_K_CORRECT, G.cnt[3] * batch,
-                  k_correct<float, false><<<gface, block_dim(), 0, grid->stream>>>(
-                      G, grid->ctl, (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2],
-                      (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2], x0, x1, p,
-                      0.0));
+                  launch_dep(grid, k_correct<float, false>, gface, block_dim(), 0, G, grid->ctl,
+                             (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2],
+                             (float*)grid->fs[0], (float*)grid->fs[1], (float*)grid->fs[2], x0, x1,
+                             p, 0.0, nullptr));
     else
         NS_LAUNCH(grid, NS_K_CORRECT, G.cnt[3] * batch,
-                  k_correct<double, false><<<gface, block_dim(), 0, grid->stream>>>(
-                      G, grid->ctl, (double*)grid->fs[0], (double*)grid->fs[1],
-                      (double*)grid->fs[2], (double*)grid->fs[0], (double*)grid->fs[1],
-                      (double*)grid->fs[2], x0, x1, p, 0.0));
+                  launch_dep(grid, k_correct<double, false>, gface, block_dim(), 0, G, grid->ctl,
+                             (double*)grid->fs[0], (double*)grid->fs[1], (double*)grid->fs[2],
+                             (double*)grid->fs[0], (double*)grid->fs[1], (double*)grid->fs[2], x0,
+                             x1, p, 0.0, nullptr));
     NS_CUDA(cudaGetLastError());
     NS_TRY(persist_settle(grid));
     NS_TRY(sync_stream(grid));
