@@ -343,36 +343,38 @@ __device__ __forceinline__ bool arrive_last(unsigned int* counter, int ctas) {
     return is_last;
 }
 
-// Fixed-order sum of [ctas][NV] partials, read through L2, in the last CTA.
-// Each thread sums the CTAs t, t + NTHREADS, ... in that order; it loads a
-// batch of them before adding, so the reads of the batch overlap (the last
-// CTA's reduction is on the critical path of every solver phase).
+// Fixed-order sum of [ctas][NV] partials, read through L2, in the last CTA
+// (valid in thread 0).  A warp sums a value: lane l the CTAs l, l + 32, ... in
+// that order, a batch of loads before its sums so that the reads overlap, then
+// one tree.  Every solver phase waits for this, and an FP64 operation of a warp
+// holds the SM's pipe 16 cycles: each warp taking all values, then a second
+// tree, was 40 of them after the loads for every 5 here.
 template <int NV>
 __device__ __forceinline__ void sum_partials_l2(const double* part, int ctas, double (&out)[NV]) {
-    constexpr int UB = NV <= 3 ? 4 : 2;
-    double v[NV];
+    constexpr int UB = 8;
+    __shared__ double res_all[NSUB][NV];
+    double(&res)[NV] = res_all[sub_id()];
+    const int lane = tid_flat() & 31, warp = tid_flat() >> 5;
+    for (int q = warp; q < NV; q += NWARPS) {
+        double v = 0.0;
+        for (int c0 = lane; c0 < ctas; c0 += UB * 32) {
+            double buf[UB];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) v[q] = 0.0;
-    for (int c0 = tid_flat(); c0 < ctas; c0 += UB * NTHREADS) {
-        double buf[UB][NV];
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
-            const int c = c0 + u * NTHREADS;
-#pragma unroll
-            for (int q = 0; q < NV; ++q)
-                buf[u][q] = c < ctas ? __ldcg(part + (long long)c * NV + q) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
-            if (c0 + u * NTHREADS < ctas) {
-#pragma unroll
-                for (int q = 0; q < NV; ++q) v[q] += buf[u][q];
+            for (int u = 0; u < UB; ++u) {
+                const int c = c0 + u * 32;
+                buf[u] = c < ctas ? __ldcg(part + (long long)c * NV + q) : 0.0;
             }
-        }
-    }
-    block_sum<NV>(v);
 #pragma unroll
-    for (int q = 0; q < NV; ++q) out[q] = v[q];  // valid in thread 0
+            for (int u = 0; u < UB; ++u)
+                if (c0 + u * 32 < ctas) v += buf[u];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) res[q] = v;
+    }
+    sub_sync();
+#pragma unroll
+    for (int q = 0; q < NV; ++q) out[q] = res[q];
 }
 
 // Sum over the CTA of per-thread values: a warp-shuffle tree in the values'
