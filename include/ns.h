@@ -129,9 +129,8 @@ typedef struct {
     int coarse_tile_z;       /* tile_z of the batch-1 companion grid on which
                                 ns_parareal_iterate evaluates the coarse
                                 propagator (every G of a grid, so G_new and G_old
-                                of equal inputs stay bit-identical); 0: 8.  Deep
-                                marches (few CTAs) suit the pipelined schedule,
-                                whose chain shares the GPU with the sweeps.       */
+                                of equal inputs stay bit-identical); 0: the
+                                default of tile_z for one state.                  */
 } ns_grid_desc;
 
 typedef enum { NS_PC_NONE = 0, NS_PC_MULTIGRID = 1 } ns_preconditioner;
