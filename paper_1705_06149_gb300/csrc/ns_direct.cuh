@@ -883,11 +883,16 @@ __global__ void __launch_bounds__(NTHREADS)
     const SliceCtl* c = ctl + s;
     const long long off = s * L.cells;
     const int step = c->o_steps, ne = min(step, DIR_RING - 1);
-    const float* __restrict__ e0 = ring + ((step - 1) & (DIR_RING - 1)) * stride + off;
-    const float* __restrict__ e1 = ring + ((step - 2) & (DIR_RING - 1)) * stride + off;
-    const float* __restrict__ e2 = ring + ((step - 3) & (DIR_RING - 1)) * stride + off;
     const float* bh = base_hi + off;
     const float* bl = base_lo + off;
+    // applications that do not exist are read from the base and dropped, so
+    // that no load waits behind a condition
+    auto app = [&](int n) -> const float* {
+        return ne >= n ? ring + ((step - n) & (DIR_RING - 1)) * stride + off : bh;
+    };
+    const float* e0 = app(1);
+    const float* e1 = app(2);
+    const float* e2 = app(3);
     const FF neg_mean{-c->mean_hi, -c->mean_lo};
     const bool keep = w_hi != nullptr;
     int i, j, k0;
@@ -898,29 +903,34 @@ __global__ void __launch_bounds__(NTHREADS)
     const int base = j * nx + i;
     const int xl = i > 0 ? base - 1 : (wx ? base : base + nx - 1);
     const int yl = j > 0 ? base - nx : (wy ? base : base + (ny - 1) * nx);
+    struct Raw {
+        float h, l, a, b, c;
+    };
+    auto raw = [&](int q) -> Raw { return Raw{bh[q], bl[q], e0[q], e1[q], e2[q]}; };
     // p at a cell: the newest application is the smallest, so it is added last
-    auto pat = [&](int q) -> FF {
-        FF p{bh[q], bl[q]};
-        if (ne > 2) p = ff_add_f(p, e2[q]);
-        if (ne > 1) p = ff_add_f(p, e1[q]);
-        if (ne > 0) p = ff_add_f(p, e0[q]);
+    auto sum = [&](const Raw& v) -> FF {
+        FF p{v.h, v.l};
+        if (ne > 2) p = ff_add_f(p, v.c);
+        if (ne > 1) p = ff_add_f(p, v.b);
+        if (ne > 0) p = ff_add_f(p, v.a);
         return p;
     };
-    FF pz = pat((k0 > 0 ? k0 - 1 : (wz ? 0 : nz - 1)) * plane + base);
+    FF pz = sum(raw((k0 > 0 ? k0 - 1 : (wz ? 0 : nz - 1)) * plane + base));
     const long long ru = s * cu + (long long)j * (nx + wx) + i, pu = (long long)ny * (nx + wx);
     const long long rv = s * cv + (long long)j * nx + i, pv = (long long)(ny + wy) * nx;
     const long long rw = s * cw + base;
     const bool ax = i > 0 || !wx, ay = j > 0 || !wy;
     constexpr int ZB = 2;
     for (int kb = k0; kb < k1; kb += ZB) {
+        Raw rc[ZB], rx[ZB], ry[ZB];
         FF pc[ZB], px[ZB], py[ZB], qv[ZB];
         float fa[ZB][3], oa[ZB][3];
 #pragma unroll
         for (int q = 0; q < ZB; ++q) {
             const int k = min(kb + q, k1 - 1);
-            pc[q] = pat(k * plane + base);
-            px[q] = pat(k * plane + xl);
-            py[q] = pat(k * plane + yl);
+            rc[q] = raw(k * plane + base);
+            rx[q] = raw(k * plane + xl);
+            ry[q] = raw(k * plane + yl);
             fa[q][0] = fu[ru + k * pu];
             fa[q][1] = fv[rv + k * pv];
             fa[q][2] = fw[rw + (long long)k * plane];
@@ -933,6 +943,12 @@ __global__ void __launch_bounds__(NTHREADS)
                 const long long id = off + (long long)k * plane + base;
                 qv[q] = FF{f.q_hi[id], f.q_lo[id]};
             }
+        }
+#pragma unroll
+        for (int q = 0; q < ZB; ++q) {
+            pc[q] = sum(rc[q]);
+            px[q] = sum(rx[q]);
+            py[q] = sum(ry[q]);
         }
 #pragma unroll
         for (int q = 0; q < ZB; ++q) {
@@ -1380,7 +1396,7 @@ inline std::vector<T> dir_tables(const DirPlan<T>& P, const int bc[3], const dou
 // does not give it) the longest march of 64 cells or less that leaves the SMs
 // eight CTAs deep, 4 below that.  A CTA's sums end in FP64, which a longer march
 // pays less often: 64^3 x 32 states, 8 -> 32 cells: start 137 -> 115 us,
-// correction of r 73 -> 66, of u 143 -> 136.
+// correction of r 73 -> 66, of u 143 -> 136 (then 120 by its loads' order).
 inline DirTile dir_tile_of(const int n[3], int cap, int tile_z) {
     DirTile t;
     const int xt = (n[0] + 31) / 32;
