@@ -1438,13 +1438,20 @@ ns_status solve_pressure_mg_graph(ns_grid* g, int batch, const double* p_in) {
     });
 }
 
+// Corrections a solve from an extrapolated start takes: a captured solve runs
+// them as plain nodes (states that have converged leave at once).
+int direct_usual(const ns_grid* g) { return g->fp32 || g->mixed ? 2 : 1; }
+
 // The corrections of a started solve.  On the stream path as many as the last
 // solves took are issued back to back, then the flags are polled after each;
-// captured, they are a while loop on the device.
+// captured, the usual number is followed by a while loop on the device for the
+// rest (a loop's node costs about 20 us whenever its body runs).
 ns_status direct_loop(ns_grid* g, int batch) {
     NS_CUDA(cudaGetLastError());
     if (g->capturing) {
         const int cap = (g->fp32 ? g->max_outer : g->maxit) + 2;
+        for (int q = 0; q < direct_usual(g); ++q) direct_correct(g, batch);
+        NS_CUDA(cudaGetLastError());
         cudaGraphConditionalHandle h;
         NS_TRY(make_handle(g->stream, &h));
         NS_TRY(loop_cond(g, batch, h, g->fp32 ? LC_REFINE_START : LC_FP64_START, cap));
@@ -1986,9 +1993,11 @@ ns_status account_graph(ns_grid* g, int B, long long state_steps, long long step
     g->stats.steps += state_steps;
     // per step: predict, divergence, solve start, loop condition, correction;
     // per loop body: one iteration, (FP32) the outer correction, the condition
-    g->stats.launches += step_groups * (g->dir && g->fp32 ? 4 : 5) +
-                         bodies * (mg_iteration_launches(g) + (g->fp32 ? 2 : 1)) +
-                         extra_launches;
+    // a direct solve's usual corrections are outside the loop
+    const long long body = mg_iteration_launches(g) + (g->fp32 ? 1 : 0);
+    g->stats.launches += step_groups * ((g->dir && g->fp32 ? 4 : 5) +
+                                        (g->dir ? direct_usual(g) * body : 0)) +
+                         bodies * (body + 1) + extra_launches;
     ns_status result = NS_OK;
     for (int s = 0; s < B; ++s) {
         const SliceCtl& a = ctl[s];
