@@ -81,12 +81,16 @@ typedef struct {
                                 preconditioner (NS_PC_MULTIGRID; falls back to
                                 NS_PC_NONE on grids it cannot coarsen far enough).
                                 With NS_PC_MULTIGRID, a box without solid cells
-                                whose planes fit one SM's shared memory takes its
-                                corrections from a direct solve of L e = r instead
-                                (transforms along x and y, three-point equations
-                                along z; the same stopping tolerances, one
-                                application counted as one iteration), unless its
-                                tolerance is below 1e-14; NS_DIRECT=0 in the
+                                whose planes, or the matrices of an axis, fit one
+                                SM's shared memory takes its corrections from a
+                                direct solve of L e = r instead (transforms along x
+                                and y, three-point equations along z; the same
+                                stopping tolerances, one application counted as one
+                                iteration; large FP64 calls apply it in FP32 to the
+                                FP64 residual), unless its tolerance is below 1e-14;
+                                with solid cells it preconditions conjugate
+                                gradients in FP32_REFINE's inner solves (one
+                                iteration counted as one).  NS_DIRECT=0 in the
                                 environment at ns_create_grid, or any of the
                                 multigrid's variables below, keeps the V-cycle.
                                 The levels with at most 4096 cells (FP32_REFINE;

@@ -1,5 +1,6 @@
 // Direct solve of L e = r on a box without solid cells, the correction of the
-// pressure solve (Section 2) there: L is a sum of three 1D operators whose
+// pressure solve (Section 2) there and, with solid cells, the preconditioner of
+// its conjugate gradients: L is a sum of three 1D operators whose
 // eigenvectors are known (cosines on a Neumann axis, the real Fourier basis on
 // a periodic one), so e is r transformed along x and y, a three-point equation
 // along z per (kx, ky), and transformed back.  One application in FP32 leaves
@@ -14,6 +15,7 @@
 // columns) in shared memory: fold (or read the quadrants), multiply by the x
 // matrix, multiply by the y matrix, write the quadrants (or unfold).  The
 // spectral plane keeps the even modes of an axis first, then the odd ones.
+// Planes that do not fit go one axis at a time (k_dir_x, k_dir_y).
 //
 // Along z (k_dir_z).  With rho + 1/rho = 2 + h_z^2 (lam_x + lam_y), rho <= 1,
 // the three-point operator is (1 - rho S)(1 - rho S^-1) / rho: a recursion up
