@@ -1242,30 +1242,36 @@ __global__ void __launch_bounds__(NTHREADS)
 // one axis: even ones first; q[m * n + j] = value of vector m at cell j.
 inline void dir_basis(int n, bool periodic, std::vector<double>& q, std::vector<double>& lam) {
     const double pi = 3.14159265358979323846;
-    const int h = (n + 1) / 2;
+    const int h = (n + 1) / 2, period = 4 * n;
+    // every value is a cosine of a multiple of pi / (2 n)
+    std::vector<double> cs(period);
+    for (int m = 0; m < period; ++m) cs[m] = std::cos(pi * m / (2.0 * n));
     q.assign((size_t)n * n, 0.0);
     lam.assign(n, 0.0);
     for (int m = 0; m < n; ++m) {
         const bool even = m < h;
         const int i = even ? m : m - h;  // index within its parity
-        double w, norm = std::sqrt(2.0 / n);
+        double norm = std::sqrt(2.0 / n);
         bool sine = false;
+        int w;  // of the mode, in pi / n
         if (!periodic) {
-            const int k = even ? 2 * i : 2 * i + 1;
-            w = pi * k / n;
-            if (k == 0) norm = std::sqrt(1.0 / n);
+            w = even ? 2 * i : 2 * i + 1;
+            if (w == 0) norm = std::sqrt(1.0 / n);
         } else {
-            // cosines m = 0 .. h-1, sines m = 1 .. n/2 (the highest mode of an
-            // even n is the sine pi (j + 1/2))
+            // cosines 0 .. h-1, sines 1 .. n/2 (the highest mode of an even n
+            // is the sine pi (j + 1/2))
             const int k = even ? i : i + 1;
-            w = 2.0 * pi * k / n;
+            w = 2 * k;
             sine = !even;
             if (k == 0 || 2 * k == n) norm = std::sqrt(1.0 / n);
         }
-        const double sh = std::sin(0.5 * w);
+        const double sh = std::sin(0.5 * pi * w / n);
         lam[m] = 4.0 * sh * sh;
-        for (int j = 0; j < n; ++j)
-            q[(size_t)m * n + j] = norm * (sine ? std::sin(w * (j + 0.5)) : std::cos(w * (j + 0.5)));
+        for (int j = 0; j < n; ++j) {
+            // w pi / n (j + 1/2), a sine as a cosine a quarter turn earlier
+            const long long at = (long long)w * (2 * j + 1) + (sine ? 3 * n : 0);
+            q[(size_t)m * n + j] = norm * cs[at % period];
+        }
     }
 }
 
@@ -1379,7 +1385,9 @@ inline std::vector<T> dir_tables(const DirPlan<T>& P, const int bc[3], const dou
             const size_t q = (size_t)ky * P.nx + kx;
             const double sig = (lx[kx] * ih2[0] + ly[ky] * ih2[1]) / ih2[2];
             const double rho = 1.0 / (1.0 + 0.5 * sig + std::sqrt(sig + 0.25 * sig * sig));
-            const double rn = std::pow(rho, P.nz);
+            double rn = 1.0, base = rho;
+            for (int e = P.nz; e > 0; e >>= 1, base *= base)
+                if (e & 1) rn *= base;
             double c1 = 0.0, c2 = 0.0;
             if (q != 0) {
                 c1 = 1.0 / (P.per_z ? 1.0 - rn : 1.0 - rn * rn);
