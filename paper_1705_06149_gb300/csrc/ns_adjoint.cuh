@@ -398,7 +398,7 @@ __device__ __forceinline__ T adj_face(T uf, T bb, T b, T f, T ff, T (&d4)[4]) {
 
 // lambda = mu + dt (dR/du)^T mu on active faces (zero on wall faces) of a
 // tile, every stored value written once; per-CTA partial sums of
-// (dR/du_lid)^T mu in part_lid[state][cta].  The velocity with its ghost values
+// dt (dR/du_lid)^T mu in part_lid[state][cta].  The velocity with its ghost values
 // and mu (zero outside) are staged once, so an interior value is a fixed set
 // of 16 face evaluations without a boundary rule: interfaces that do not exist
 // have mu differences of zero.  The ghosts that mirror a value add their part
@@ -415,6 +415,9 @@ __global__ void __launch_bounds__(NTHREADS)
     T* sv = reinterpret_cast<T*>(asm_raw);  // [3][AT_SZ][AT_SY][AT_SX]
     T* sm = sv + 3 * AT_N;                  // the same of mu
     __shared__ int zv[3][AT_SZ], zu[3][AT_SZ];
+    // the forward step's coefficients, dt / h and dt / (Re h^2), then what
+    // their rounding to T left
+    __shared__ T coef[12];
     const long long s = blockIdx.y;
     const T* const vel3[3] = {u + s * g.cnt[0], v + s * g.cnt[1], w + s * g.cnt[2]};
     const T* const mu3[3] = {mu_u + s * g.cnt[0], mu_v + s * g.cnt[1], mu_w + s * g.cnt[2]};
@@ -422,6 +425,12 @@ __global__ void __launch_bounds__(NTHREADS)
     const int cta = blockIdx.x, r = cta / tbx, tz = r / tby;
     const int i0 = (cta - r * tbx) * TX, j0 = (r - tz * tby) * TY, k0 = tz * AT_Z;
     const int t = tid_flat();
+    if (t < 6) {
+        const int d = t < 3 ? t : t - 3;
+        const double k = dt * (t < 3 ? g.ih[d] : g.inv_re * g.ih2[d]);
+        coef[t] = T(k);
+        coef[6 + t] = T(k - double(T(k)));
+    }
     for (int q = t; q < 3 * AT_SZ; q += NTHREADS) {
         const int c = q / AT_SZ, z = q - c * AT_SZ;
         bool lid = false;
@@ -462,7 +471,10 @@ __global__ void __launch_bounds__(NTHREADS)
     }
     __syncthreads();
     constexpr int strd[3] = {1, AT_SX, AT_PLANE};
-    const T inv_re = g_inv_re<T>(g), tdt = T(dt);
+    // coefficient d of the list times a value (FP32: with its rounding)
+    auto scaled = [&](int d, T v) -> T {
+        return sizeof(T) == 4 ? fma(coef[d], v, coef[6 + d] * v) : coef[d] * v;
+    };
     const int x0 = (int)threadIdx.x, y0 = (int)threadIdx.y;
     double dl = 0.0;
     if (i0 + x0 < g.n[0] && j0 + y0 < g.n[1]) {
@@ -478,8 +490,7 @@ __global__ void __launch_bounds__(NTHREADS)
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     const int sd = strd[d];
-                    const T ih = g_ih<T>(g, d), kd = inv_re * g_ih2<T>(g, d);
-                    acc += kd * (mc[sd] - T(2) * mc[0] + mc[-sd]);
+                    acc += scaled(3 + d, mc[sd] - T(2) * mc[0] + mc[-sd]);
                     // the ghosts that mirror this value, as offsets from it
                     // (0: none): beyond the low and the high wall
                     int lo = 0, hi = 0;
@@ -498,13 +509,13 @@ __global__ void __launch_bounds__(NTHREADS)
                     const bool lid = c == 0 && d == 1 && g.bc[1] == BC_WALL;
                     T top = T(0);  // the high ghost's part, before its sign
                     if (d != c) {
-                        if (lo == -1) acc += sg * kd * mc[0];
-                        if (hi == 1) top += kd * mc[0];
+                        if (lo == -1) acc += sg * scaled(3 + d, mc[0]);
+                        if (hi == 1) top += scaled(3 + d, mc[0]);
                     }
 #pragma unroll
                     for (int q = -2; q <= 1; ++q) {
                         // interface between the values at q and q + 1
-                        const T nu = (mc[(q + 1) * sd] - mc[q * sd]) * ih;
+                        const T nu = scaled(d, mc[(q + 1) * sd] - mc[q * sd]);
                         const T b = a[q * sd], fw = a[(q + 1) * sd];
                         const T* tr = sv + d * AT_N + o + (q + 1) * sd;
                         const T uf = d == c ? T(0.5) * (b + fw) : T(0.5) * (tr[-strd[c]] + tr[0]);
@@ -531,7 +542,6 @@ __global__ void __launch_bounds__(NTHREADS)
                 }
                 // as the transport of the other components along c
                 const int sc = strd[c];
-                const T ih = g_ih<T>(g, c);
 #pragma unroll
                 for (int c2 = 0; c2 < 3; ++c2) {
                     if (c2 == c) continue;
@@ -541,7 +551,7 @@ __global__ void __launch_bounds__(NTHREADS)
                         const int at = o - sc + (cand ? s2 : 0);  // the interface's low value
                         const T* l = sv + c2 * AT_N + at;
                         const T* m2 = sm + c2 * AT_N + at;
-                        const T nu = (m2[sc] - m2[0]) * ih;
+                        const T nu = scaled(c, m2[sc] - m2[0]);
                         const T* tr = sv + c * AT_N + at + sc;
                         const T uf = T(0.5) * (tr[-s2] + tr[0]);
                         T d4[4];
@@ -550,7 +560,7 @@ __global__ void __launch_bounds__(NTHREADS)
                 }
                 const long long id = vindex(g, c, f[0], f[1], f[2]);
                 const bool wall = g.bc[c] != BC_PERIODIC;
-                out[c][id] = (wall && f[c] == 0) ? T(0) : mc[0] + tdt * acc;
+                out[c][id] = (wall && f[c] == 0) ? T(0) : mc[0] + acc;
                 if (wall && f[c] == g.n[c] - 1) {
                     int h[3] = {f[0], f[1], f[2]};
                     h[c] += 1;

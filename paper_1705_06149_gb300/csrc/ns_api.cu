@@ -2779,7 +2779,7 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
             st = project_impl<T>(g, vel_state(mu, pmu), pmu);
             if (st != NS_OK) break;
             // lambda = mu + dt (dR/du)^T mu at u^n (active faces), dJ/du_lid +=
-            // dt (dR/du_lid)^T mu (dt at the end)
+            // dt (dR/du_lid)^T mu (the gather leaves its dt to the end)
             T* un = seg + (size_t)(n - n0) * vel_elems;
             if (tiled) {
                 NS_LAUNCH(g, NS_K_ADJOINT, 0,
@@ -2823,7 +2823,7 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
         if (st == NS_OK) {
             for (int b = 0; b < B; ++b) {
                 J[b] = h[b];
-                dlid_out[b] = dt * h[B + b];
+                dlid_out[b] = (tiled ? 1.0 : dt) * h[B + b];
             }
         }
     }

@@ -115,7 +115,9 @@ __global__ void __launch_bounds__(PX * PY NS_MIN_CTAS(512 / (PX * PY)))
     // fluxes through the tile's low x / y faces and the rows' high y faces, by
     // parity of the z step
     __shared__ T xlo[2][3][PY], ylo[2][3][PX], yex[2][3][PY][PX];
-    __shared__ T coef[6];  // dt / (2 h) (the fluxes are twice the convective ones), dt / (Re h^2)
+    // dt / (2 h) (the fluxes are twice the convective ones) and dt / (Re h^2),
+    // then what their rounding to T left
+    __shared__ T coef[12];
     __shared__ int zsrc[3][PZ + 4];  // z index a staged plane comes from, ~ of it: sign -1
     const long long s = blockIdx.y;
     const T* vel3[3] = {u + s * g.cnt[0], v + s * g.cnt[1], w + s * g.cnt[2]};
@@ -130,7 +132,9 @@ __global__ void __launch_bounds__(PX * PY NS_MIN_CTAS(512 / (PX * PY)))
     // (one warp: a warp's FP64 operation holds the pipe whatever its lanes)
     if (t < 6) {
         const int d = t < 3 ? t : t - 3;
-        coef[t] = T(dt * (t < 3 ? 0.5 * g.ih[d] : g.inv_re * g.ih2[d]));
+        const double k = dt * (t < 3 ? 0.5 * g.ih[d] : g.inv_re * g.ih2[d]);
+        coef[t] = T(k);
+        coef[6 + t] = T(k - double(T(k)));
     }
     for (int q = t; q < 3 * (PZ + 4); q += NT) {
         const int c = q / (PZ + 4), gk = k0 - PH + q - c * (PZ + 4);
@@ -234,6 +238,10 @@ __global__ void __launch_bounds__(PX * PY NS_MIN_CTAS(512 / (PX * PY)))
         ey[h] = yf;
     }
     const T kc[3] = {coef[0], coef[1], coef[2]}, kd[3] = {coef[3], coef[4], coef[5]};
+    // FP32: the coefficients carry their rounding (up to 6e-8 of every increment
+    // of a run, which a functional of the state would show undamped).
+    constexpr bool LOW = sizeof(T) == 4;
+    const T lc[3] = {coef[6], coef[7], coef[8]}, ld[3] = {coef[9], coef[10], coef[11]};
     const int i = i0 + x, j = j0 + y;
     T fz[3], zm[3], zc[3], zp[3];
     T* dst[3];
@@ -292,9 +300,16 @@ __global__ void __launch_bounds__(PX * PY NS_MIN_CTAS(512 / (PX * PY)))
             fxl[c] = __shfl_up_sync(0xffffffffu, mul_rounded(tx[c], px[c]), 1);
             // (fma by fma: every tile shape rounds alike; the cell's own high
             // flux enters unrounded)
-            inc[c] = fma((yh - a) - (a - yl), kd[1], ((xh - a) - (a - xl)) * kd[0]);
-            inc[c] = fma((zp[c] - a) - (a - zm[c]), kd[2], inc[c]);
-            inc[c] = fma(-fma(tw, pz, -fz[c]), kc[2], inc[c]);
+            const T d2[3] = {(xh - a) - (a - xl), (yh - a) - (a - yl),
+                             (zp[c] - a) - (a - zm[c])};
+            const T dz = -fma(tw, pz, -fz[c]);
+            if (LOW) {
+                const T low = fma(d2[2], ld[2], fma(d2[1], ld[1], d2[0] * ld[0]));
+                inc[c] = fma(d2[1], kd[1], fma(d2[0], kd[0], fma(dz, lc[2], low)));
+            } else {
+                inc[c] = fma(d2[1], kd[1], d2[0] * kd[0]);
+            }
+            inc[c] = fma(dz, kc[2], fma(d2[2], kd[2], inc[c]));
             fz[c] = mul_rounded(tw, pz);
             zm[c] = a;
             zc[c] = zp[c];
@@ -307,8 +322,9 @@ __global__ void __launch_bounds__(PX * PY NS_MIN_CTAS(512 / (PX * PY)))
         for (int c = 0; c < 3; ++c) {
             const T xl = x == 0 ? xlo[par][c][y] : fxl[c];
             const T yl = y == 0 ? ylo[par][c][x] : yex[par][c][y > 0 ? y - 1 : 0][x];
-            const T incr = fma(-fma(ty[c], py[c], -yl), kc[1],
-                               fma(-fma(tx[c], px[c], -xl), kc[0], inc[c]));
+            const T dx = -fma(tx[c], px[c], -xl), dy = -fma(ty[c], py[c], -yl);
+            const T low = LOW ? fma(dy, lc[1], fma(dx, lc[0], inc[c])) : inc[c];
+            const T incr = fma(dy, kc[1], fma(dx, kc[0], low));
             const bool wall = g.bc[c] != BC_PERIODIC;
             const bool lo = c < 2 ? wlo[c < 2 ? c : 0] : (wall && k == 0);
             // the high wall face of the last cell along c is inactive: zero it

@@ -108,3 +108,24 @@ def test_adjoint_tile_matches_oracle(emulator, dims, bc, prec):
         err = np.max(np.abs(got - lam)) / np.max(np.abs(want[c]))
         assert err <= tol, (c, err)
     assert abs(out[-1] - want_dl) <= tol * max(abs(want_dl), np.max(np.abs(want[0])))
+
+
+def test_lid_derivative_carries_no_coefficient_rounding(emulator):
+    """FP32, u = 0, mu near one: the lid's part is 2 / (Re h^2) sum mu over the
+    faces under it.  A face's sum rounds at random (2^-24 of it at most, 2e-9 of
+    the total of 600 faces at one standard deviation); the coefficient's own
+    rounding would be in every face alike (6.6e-8 here as FP32 factors)."""
+    exe, d = emulator
+    dims, bc, re = (40, 6, 15), ("periodic", "wall", "periodic"), 44.0
+    shapes = [a.shape for a in inputs.random_state(*dims, seed=1, sigma=1.0, bc=bc)]
+    rng = np.random.default_rng(3)
+    mu = [np.zeros(s) for s in shapes[:3]]
+    mu[0] = (1.0 + 0.1 * rng.random(shapes[0])).astype(np.float32).astype(np.float64)
+    zero = [np.zeros(s) for s in shapes[:3]]
+    fin, fout = d / "in_lid.bin", d / "out_lid.bin"
+    np.concatenate([np.ravel(a) for a in zero + mu]).tofile(fin)
+    r = subprocess.run([exe, "f", *map(str, dims), *(str(BC[x]) for x in bc), repr(re), "1.0",
+                        str(fin), str(fout)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stderr[-3000:])
+    want = oracle.Grid(*dims, re=re, u_lid=1.0, bc=bc).rhs_adjoint(*zero, mu)[1]
+    assert abs(np.fromfile(fout, dtype=np.float64)[-1] / want - 1.0) <= 1e-8
