@@ -24,6 +24,7 @@
 #include "ns_mg_cluster.cuh"
 #include "ns_persist.h"
 #include "ns_pipeline.h"
+#include "ns_workspace.h"
 
 using namespace nsk;
 
@@ -2680,32 +2681,6 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
     const int seg_len = std::min(C, std::max(N, 1));
     const int tblocks = (int)std::min<long long>((std::max(G.cnt[0], std::max(G.cnt[1], G.cnt[2])) +
                                                   NTHREADS - 1) / NTHREADS, 512);
-    std::vector<void*> mine;
-    auto alloc = [&](size_t bytes) -> void* {
-        void* p = nullptr;
-        if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        mine.push_back(p);
-        return p;
-    };
-    auto release = [&]() {
-        cudaStreamSynchronize(g->stream);
-        for (void* p : mine) cudaFree(p);
-        mine.clear();
-    };
-    T* cur = (T*)alloc(sizeof(T) * vel_elems);
-    double* cur_p = (double*)alloc(sizeof(double) * np);
-    T* ck = (T*)alloc(sizeof(T) * vel_elems * std::max(nck, 1));
-    double* ck_p = (double*)alloc(sizeof(double) * np * std::max(nck, 1));
-    T* seg = (T*)alloc(sizeof(T) * vel_elems * seg_len);
-    T* lam = (T*)alloc(sizeof(T) * vel_elems);
-    T* mu = (T*)alloc(sizeof(T) * vel_elems);
-    T* acc = (T*)alloc(sizeof(T) * vel_elems);
-    double* pmu = (double*)alloc(sizeof(double) * np);  // phi of the adjoint projections
-    double* dJ = (double*)alloc(sizeof(double) * 2 * B);
-    double* part_J = (double*)alloc(sizeof(double) * 3 * tblocks * B);
     // the reverse step: tiles of 32 x 4 x AT_Z cells; FP64 calls whose tiles
     // would leave half the SMs idle, the gather (32 x 4 column tiles over the
     // face extents, ADJ_TZ positions along z per thread, one grid z-slice per
@@ -2716,16 +2691,25 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
     const int tile_ctas = atx * aty * ceil_div(G.n[2], AT_Z);
     const size_t tile_smem = 6 * (size_t)AT_N * sizeof(T);
     const bool tiled = sizeof(T) == 4 || (long long)tile_ctas * B >= 76;
-    if (tiled && cudaFuncSetAttribute(k_adj_tile<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)tile_smem) != cudaSuccess)
-        return fail(NS_ERR_CUDA, "ns_adjoint: shared memory attribute");
+    if (tiled)
+        NS_CUDA(cudaFuncSetAttribute(k_adj_tile<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)tile_smem));
     const int adj_ctas = G.fbx * G.fby * ceil_div(G.n[2] + 1, ADJ_TZ);
     const int lid_parts = tiled ? tile_ctas : 3 * adj_ctas;
-    double* part_lid = (double*)alloc(sizeof(double) * lid_parts * B);
-    if (mine.size() != 12) {
-        release();
-        return fail(NS_ERR_OOM, "ns_adjoint: workspace allocation failed");
-    }
+    Workspace ws(g->stream);
+    T* cur = ws.get<T>(vel_elems);
+    double* cur_p = ws.get<double>(np);
+    T* ck = ws.get<T>(vel_elems * std::max(nck, 1));
+    double* ck_p = ws.get<double>(np * std::max(nck, 1));
+    T* seg = ws.get<T>(vel_elems * seg_len);
+    T* lam = ws.get<T>(vel_elems);
+    T* mu = ws.get<T>(vel_elems);
+    T* acc = tiled ? nullptr : ws.get<T>(vel_elems);  // the gather's (dR/du)^T mu
+    double* pmu = ws.get<double>(np);  // phi of the adjoint projections
+    double* dJ = ws.get<double>(2 * B);
+    double* part_J = ws.get<double>(3 * (size_t)tblocks * B);
+    double* part_lid = ws.get<double>((size_t)lid_parts * B);
+    if (!ws.ok()) return fail(NS_ERR_OOM, "ns_adjoint: workspace allocation failed");
     auto vel_state = [&](T* base, double* p) {
         ns_state st{base, base + nv[0], base + nv[0] + nv[1], p, B};
         return st;
@@ -2734,7 +2718,7 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
     ns_state cs = vel_state(cur, cur_p);
     void* dst0[4] = {cs.u, cs.v, cs.w, cs.p};
     ns_status st = copy_states<T>(g, dst0, src0, 0, 0, B);
-    NS_CUDA(cudaMemsetAsync(acc, 0, sizeof(T) * vel_elems, g->stream));
+    if (acc) NS_CUDA(cudaMemsetAsync(acc, 0, sizeof(T) * vel_elems, g->stream));
     NS_CUDA(cudaMemsetAsync(dJ, 0, sizeof(double) * 2 * B, g->stream));
     NS_CUDA(cudaMemsetAsync(pmu, 0, sizeof(double) * np, g->stream));
     auto copy = [&](void* dst, const void* src, size_t bytes, const char* what) {
@@ -2787,7 +2771,7 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
                               G, un, un + nv[0], un + nv[0] + nv[1], mu, mu + nv[0],
                               mu + nv[0] + nv[1], lam, lam + nv[0], lam + nv[0] + nv[1], dt, atx,
                               aty, part_lid));
-            } else {
+            } else if constexpr (sizeof(T) == 8) {
                 NS_LAUNCH(g, NS_K_ADJOINT, 0,
                           k_adj_rhs<T><<<dim3(adj_ctas, B, 3), block_dim(), 0, g->stream>>>(
                               G, un, un + nv[0], un + nv[0] + nv[1], mu, mu + nv[0],
@@ -2827,7 +2811,6 @@ ns_status adjoint_impl(ns_grid* g, const ns_state& u0, double dt, int N, int C, 
             }
         }
     }
-    release();
     return st;
 }
 
