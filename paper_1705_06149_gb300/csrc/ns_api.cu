@@ -590,7 +590,10 @@ ns_status setup_direct(ns_grid* g) {
     const double cond = dir_condition(G.n, G.bc, G.ih2);
     if (!(rtol >= 1e-14) || !(cond <= (g->fp32 ? 1e7 : 1e12))) return NS_OK;
     if (g->fp32) return setup_direct_of<float>(g, g->dirf);
-    if (cond <= 1e7 && rtol >= 1e-13 && G.cnt[3] * g->cap >= DIR_MIXED_CELLS) {
+    // (L in FP32: its coefficients within FP32's range with room for e and L e)
+    bool fp32_range = true;
+    for (double w : G.ih2) fp32_range = fp32_range && w >= 0x1p-80 && w <= 0x1p80;
+    if (cond <= 1e7 && rtol >= 1e-13 && fp32_range && G.cnt[3] * g->cap >= DIR_MIXED_CELLS) {
         NS_TRY(setup_direct_of<float>(g, g->dirf));
         g->dirf.mode = DM_MIXED;
         g->mixed = g->dir;
@@ -996,7 +999,8 @@ void direct_correct(ns_grid* g, int batch) {
             NS_LAUNCH(g, NS_K_REFINE, units,
                       launch_dep(g, k_dir_update<E>, dim3(L0.ctas, batch), block_dim(), 0, L0,
                                  mgbuf<double>(g), g->ctl, e, g->part_mg,
-                                 g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid));
+                                 g->d.poisson_rtol * g->d.poisson_rtol, g->maxit, g->geo.n_fluid,
+                                 g->dirf.log2n));
         };
         if (g->mixed) {
             direct_apply<float, double>(g, batch);

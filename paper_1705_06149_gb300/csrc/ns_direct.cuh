@@ -90,11 +90,14 @@ __device__ __forceinline__ int dir_slot(const SliceCtl* c, int mode) {
 }
 // log2 of the scale that brings a residual of squared norm rr to an RMS of order
 // one, from the exponents of rr and of the cells (no FP64 root or quotient: one
-// thread computes it at the end of a kernel that everything waits for).
-__device__ __forceinline__ int dir_shift(double rr, int log2n) {
+// thread computes it at the end of a kernel that everything waits for).  `top`
+// keeps the scale itself in range: 100 where it is an FP32 value, DIR_SHIFT64
+// where it is an FP64 one.
+constexpr int DIR_SHIFT64 = 500;
+__device__ __forceinline__ int dir_shift(double rr, int log2n, int top) {
     if (!(rr > 0.0) || !isfinite(rr)) return 0;
     const int e = (int)((__double_as_longlong(rr) >> 52) & 0x7ff) - 1023;
-    return -max(-100, min(100, (e - log2n) / 2));
+    return -max(-top, min(top, (e - log2n) / 2));
 }
 inline int dir_log2(long long n) {
     int l = 0;
@@ -104,10 +107,8 @@ inline int dir_log2(long long n) {
 template <typename T>
 __device__ __forceinline__ double dir_scale(const SliceCtl* c, bool inv, const DirPlan<T>& P) {
     if (sizeof(T) == 8 || P.mode == DM_PRECOND) return 1.0;
-    if (P.mode == DM_MIXED) {
-        const int e = dir_shift(c->rr, P.log2n);
-        return ldexp(1.0, inv ? -e : e);
-    }
+    // (an FP64 grid's e stays scaled: unscaled it may be out of FP32's range)
+    if (P.mode == DM_MIXED) return inv ? 1.0 : ldexp(1.0, dir_shift(c->rr, P.log2n, DIR_SHIFT64));
     return inv ? 1.0f / c->o_fsc : c->o_fsc;
 }
 
@@ -660,7 +661,7 @@ __device__ __forceinline__ void dir_decide(SliceCtl* c, double rr, double otol2,
                                            int max_outer) {
     c->o_rr = rr;
     c->p_final = 0;
-    c->o_fsc = ldexpf(1.0f, dir_shift(rr, log2n));
+    c->o_fsc = ldexpf(1.0f, dir_shift(rr, log2n, 100));
     c->status = ST_IDLE;
     if (!isfinite(rr)) {
         c->o_status = OS_NONFINITE;
@@ -986,7 +987,8 @@ __global__ void __launch_bounds__(NTHREADS)
 // (L has no range there): it is taken out of the next residual, or it would
 // be the floor of a solve whose right side is itself close to rounding.
 // E = float: the FP32 corrections of DM_MIXED, L e in float-float (48 bits of a
-// correction's own size; FP32 pipe).
+// correction's own size; FP32 pipe), both still in the scale that the transforms
+// gave the residual (a power of two: exact).
 template <typename E>
 __device__ __forceinline__ double dir_lap64(const Lev& L, const Vals7<E>& v);
 template <>
@@ -1001,7 +1003,7 @@ template <typename E>
 __global__ void __launch_bounds__(NTHREADS)
     k_dir_update(Lev L, MgBuf<double> mb, SliceCtl* __restrict__ ctl,
                  const E* __restrict__ evec, double* __restrict__ part, double tol2,
-                 int maxit, int nfluid) {
+                 int maxit, int nfluid, int log2n) {
     pdl_wait();
     const long long s = blockIdx.y;
     SliceCtl* c = ctl + s;
@@ -1013,6 +1015,8 @@ __global__ void __launch_bounds__(NTHREADS)
     int i, j, k0;
     lev_origin(L, blockIdx.x, i, j, k0);
     const double rmean = c->rmean;
+    const double unscale =
+        sizeof(E) == 4 ? ldexp(1.0, -dir_shift(c->rr, log2n, DIR_SHIFT64)) : 1.0;
     double rr = 0.0, sx = 0.0, sr = 0.0;
     if (i < L.n[0] && j < L.n[1]) {
         const int k1 = min(k0 + L.tz, L.n[2]);
@@ -1034,8 +1038,9 @@ __global__ void __launch_bounds__(NTHREADS)
             for (int q = 0; q < MG_ZB; ++q) {
                 if (kb + q < k1) {
                     const int id = (kb + q) * plane + xy.base;
-                    const double xv = xo[q] + ev[q].c;
-                    const double rv = ro[q] - dir_lap64<E>(L, ev[q]) - rmean;
+                    const double le = dir_lap64<E>(L, ev[q]);
+                    const double xv = fma(double(ev[q].c), unscale, xo[q]);
+                    const double rv = fma(-le, unscale, ro[q]) - rmean;
                     x[id] = xv;
                     r[id] = rv;
                     rr += rv * rv;

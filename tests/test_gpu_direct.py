@@ -117,3 +117,33 @@ def test_obstacle_steps_match_the_oracle(dims, bc, count, edge, monkeypatch):
         assert rel(vg, vw) <= TOL["fp32_refine"]
         assert rel(got[3][0], want[3]) <= TOL["fp32_refine"]
         g.close()
+
+
+# FP64 solves whose corrections are FP32 (393216 cells and more per grid): right
+# sides and boxes far outside FP32's range solve as their scaled copies do
+MIXED = (64, 64, 48)
+
+
+def _solve(b, box=(1.0, 1.0, 1.0), batch=2):
+    g = Grid(*MIXED, *box, batch=batch, poisson_rtol=1e-12)
+    p = torch.zeros_like(b)
+    its = g.poisson_solve(b, p)
+    g.close()
+    return p, its
+
+
+@pytest.mark.parametrize("power", [-400, 300])
+def test_fp64_solves_do_not_depend_on_the_size_of_the_right_side(power):
+    b = torch.tensor(np.random.default_rng(1).normal(size=(2,) + MIXED[::-1]), device="cuda")
+    p, its = _solve(b)
+    q, its_q = _solve(b * 2.0 ** power)
+    # powers of two: every operation rounds alike
+    assert its_q == its and torch.equal(q * 2.0 ** -power, p)
+
+
+def test_fp64_solves_of_a_box_beyond_fp32():
+    b = torch.tensor(np.random.default_rng(2).normal(size=(2,) + MIXED[::-1]), device="cuda")
+    p, _ = _solve(b)
+    q, _ = _solve(b, box=(2.0 ** -70,) * 3)  # h^-2 about 2^152
+    # both stop at a relative residual of 1e-12, seen through L (a few 1e3)
+    assert rel((q * 2.0 ** 140).cpu().numpy(), p.cpu().numpy()) <= 1e-8
