@@ -20,6 +20,7 @@
 #include "ns.h"
 #include "ns_adjoint.cuh"
 #include "ns_direct.cuh"
+#include "ns_mask.h"
 #include "ns_mg.cuh"
 #include "ns_mg_cluster.cuh"
 #include "ns_persist.h"
@@ -571,7 +572,7 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
 // did).  The environment variables that select a form of the multigrid solve
 // (NS_MG_CLUSTER, NS_MG_BLOCK_CELLS, NS_PERSISTENT), when set, select it;
 // NS_DIRECT=0 turns the direct solve off.  With solid cells, FP32+refine, the
-// same conditions make it the preconditioner of the inner solves.
+// same conditions and cg_suits make it the preconditioner of the inner solves.
 //
 // FP64 grids of DIR_MIXED_CELLS cells or more (all states) take FP32 corrections
 // (DM_MIXED) of the FP64 iterate and residual, two or three in the place of
@@ -579,6 +580,29 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
 // transform against 8).  4 steps of 64^3 x 4 FP64 3.14 -> 2.47 ms, of one state
 // equal, of smaller ones slower by their launches (32^3 0.58 -> 0.73 ms).
 constexpr long long DIR_MIXED_CELLS = 3 << 17;
+
+// Whether conjugate gradients preconditioned by the box solve suit the solid
+// cells.  Not with a second region of fluid: L then has a constant per region in
+// its null space, of which the box solution knows one; in FP32 the directions
+// gather them and the rounding of r in them spoils alpha (a sealed room of 10^3
+// cells in 32 x 24 x 16: no convergence where BiCGStab takes 24 iterations).
+// (Single closed cells have no equation.)  And not on planes of more than 8192
+// cells with scattered solid cells, whose iterations then outweigh their price
+// (an iteration 562 us against 770, 128^3 x 8): 1 % single cells 11.7 iterations
+// a step against 6.3, 9.7 ms against 9.2; 3 % 12.3 against 9.8; 10 % 22.2 against
+// 16.6.  There, 0.3 % 8.8 against 8.9, 8 boxes 10.3 against 12.1, pillars of 3 x 3
+// cells 8 apart 11.2 against 13.4, a plate 39 against 51; on 64^2 planes 10 %
+// single cells 2.7 against 2.9.
+bool cg_suits(const ns_grid* g) {
+    const Geo& G = g->geo;
+    const bool periodic[3] = {G.bc[0] == BC_PERIODIC, G.bc[1] == BC_PERIODIC,
+                              G.bc[2] == BC_PERIODIC};
+    const MaskShape m = mask_shape(G.n, periodic, g->mask_host.data());
+    if (m.rooms > 1) return false;
+    const bool scattered = m.faces > 4 * m.solid && 32 * m.faces > G.cnt[3];
+    return !(scattered && (long long)G.n[0] * G.n[1] > 8192);
+}
+
 ns_status setup_direct(ns_grid* g) {
     for (const char* v : {"NS_MG_CLUSTER", "NS_MG_BLOCK_CELLS", "NS_PERSISTENT"})
         if (std::getenv(v)) return NS_OK;
@@ -589,6 +613,7 @@ ns_status setup_direct(ns_grid* g) {
     const Geo& G = g->geo;
     const double cond = dir_condition(G.n, G.bc, G.ih2);
     if (!(rtol >= 1e-14) || !(cond <= (g->fp32 ? 1e7 : 1e12))) return NS_OK;
+    if (G.solid && !cg_suits(g)) return NS_OK;
     if (g->fp32) return setup_direct_of<float>(g, g->dirf);
     // (L in FP32: its coefficients within FP32's range with room for e and L e)
     bool fp32_range = true;

@@ -147,3 +147,46 @@ def test_fp64_solves_of_a_box_beyond_fp32():
     q, _ = _solve(b, box=(2.0 ** -70,) * 3)  # h^-2 about 2^152
     # both stop at a relative residual of 1e-12, seen through L (a few 1e3)
     assert rel((q * 2.0 ** 140).cpu().numpy(), p.cpu().numpy()) <= 1e-8
+
+
+def _room(dims, door):
+    solid = np.zeros(dims[::-1], np.uint8)
+    solid[2:14, 2:14, 2:14] = 1
+    solid[3:13, 3:13, 3:13] = 0
+    if door:
+        solid[7:9, 7:9, 13] = 0
+    return solid
+
+
+def _specks(dims):
+    return (np.random.default_rng(1).random(dims[::-1]) < 0.05).astype(np.uint8)
+
+
+# which solid cells keep the V-cycle: a sealed room (a second region of fluid,
+# which conjugate gradients around the box solve do not converge on) and, on large
+# planes, scattered single cells
+@pytest.mark.parametrize("dims,mask,direct",
+                         [((32, 24, 16), lambda d: _room(d, False), False),
+                          ((32, 24, 16), lambda d: _room(d, True), True),
+                          ((32, 32, 16), _specks, True),
+                          ((128, 72, 8), _specks, False)])
+def test_masks_that_keep_the_multigrid_solve(dims, mask, direct):
+    solid = mask(dims)
+    init = inputs.random_state(*dims, seed=3, sigma=0.2, solid=solid)
+    box = [d / max(dims) for d in dims] if dims[0] > 32 else (1.0, 1.0, 1.0)
+    g = Grid(*dims, *box, precision="fp32_refine", solid=solid)
+    st = g.state_from(init)
+    g.profile(True)
+    g.project(st)
+    prof = g.profile_read()
+    assert (prof["direct_xy"]["launches"] > 0) == direct
+    assert (prof["krylov_A"]["launches"] > 0) != direct
+    want = oracle.Grid(*dims, *box, solid=solid, rtol=1e-13).project(*init[:3])
+    got = st.numpy()
+    vg = np.concatenate([np.ravel(got[c][0]) for c in range(3)])
+    vw = np.concatenate([np.ravel(want[c]) for c in range(3)])
+    assert rel(vg, vw) <= 1e-6
+    # tens of iterations, where a solve that stalls takes its corrections' limit
+    # of 40 solves times 20 max(n) iterations
+    assert g.stats()["krylov_iters"] <= 100
+    g.close()
