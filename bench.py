@@ -831,7 +831,7 @@ def run_mixed(args):
         for d, re, b in specs:
             kw = {}
             if tuned:
-                r = autotune(*d, batch=b, precision=args.precision, top=2, steps=1,
+                r = autotune(*d, batch=b, precision=args.precision, top=3, steps=1,
                              grid_kwargs={"re": re, "inner_rtol": args.inner_rtol})
                 kw = {"tile_z": r["tile_z"], "predict_tile": r["predict_tile"]}
                 tiles.append({"tile_z": r["tile_z"], "predict_tile": list(r["predict_tile"]),

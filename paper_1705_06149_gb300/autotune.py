@@ -5,10 +5,11 @@ surface (Eq. 2), because the halo a subdomain exchanges grows with it.  On the
 GPU the analogue is the CTA tile, and two of them are tunable per grid:
 
 - the predictor's tile, 32 x py x pz cells (one thread per (x, y) column
-  marching z, the tile plus a two-cell halo staged in shared memory), with
-  (py, pz) among the instantiated shapes;
-- the solver kernels' tile, 32 x 4 threads each marching `tile_z` cells along
-  z (the multigrid solver's finest level; its x-pair kernels cover 64 x 4).
+  marching z with a ring of five planes and a two-cell halo in shared memory),
+  with (py, pz) among the shapes the option offers;
+- the solver kernels' tile, 32 x 4 threads (FP32 direct solves: 128 columns)
+  each marching `tile_z` cells along z (the multigrid solver's finest level;
+  its x-pair kernels cover 64 x 4).
 
 A taller or deeper tile re-reads fewer halo cells per cell (Eq. 2's surface
 per volume falls) but gives each thread more cells and leaves fewer CTAs per
@@ -16,9 +17,13 @@ launch, and once a launch has too few CTAs to fill the SMs (the device's SM
 count times the CTAs that fit on an SM) its time is the per-CTA latency and
 the tile stops paying.  The seed ranks the candidates by that model with
 the SM count and residency queried from the device; the tuner then times the
-best seeded candidates through the C ABI and keeps the fastest.  Timed choices
+library's own choice (0, or (0, 0): by the sizes, and among more shapes than
+the option offers) and the best seeded candidates through the C ABI and keeps
+the fastest, so a tuned grid is not slower than an untuned one.  Timed choices
 are cached per (grid, boundary conditions, precision, batch, device) in a JSON
-file (NS_AUTOTUNE_CACHE, else ~/.cache/paper_1705_06149_gb300/autotune.json).
+file (NS_AUTOTUNE_CACHE, else ~/.cache/paper_1705_06149_gb300/autotune.json),
+each with the version of the kernels it was timed with (a digest of their
+source); another version is timed anew.
 
 Neither choice changes the method's arithmetic: every face of the predictor
 is evaluated from the same operands whatever its tile, and `tile_z` fixes the
@@ -27,6 +32,8 @@ level only.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import math
 import os
@@ -41,7 +48,8 @@ SMEM_PER_SM = 228 * 1024             # bytes of shared memory an SM offers CTAs
 THREADS_PER_SM = 2048
 REGS_PER_SM = 65536
 SOLVER_REGS = 64                     # registers per thread of the solver kernels
-PREDICT_REGS = 32                    # registers per thread of the predictor
+PREDICT_REGS = 128                   # registers per thread of the predictor
+PREDICT_RING = 5                     # planes it keeps in shared memory
 
 
 def device_sms(default: int = 152) -> int:
@@ -98,9 +106,9 @@ def seed_cost(nx: int, ny: int, nz: int, batch: int, tz: int, sms: int = 152) ->
 def predict_seed_cost(nx: int, ny: int, nz: int, batch: int, py: int, pz: int,
                       elem_bytes: int = 4, sms: int = 152) -> float:
     """Model time per cell of the predictor tile 32 x py x pz (two-cell halo,
-    three staged components)."""
+    three components staged plane by plane)."""
     threads = PT_X * py
-    smem = 3 * (PT_X + 4) * (py + 4) * (pz + 4) * elem_bytes
+    smem = 3 * (PT_X + 4) * (py + 4) * PREDICT_RING * elem_bytes
     cells = (math.ceil(nx / PT_X) * PT_X) * (math.ceil(ny / py) * py) * (math.ceil(nz / pz) * pz)
     slots = sms * resident_ctas(threads, PREDICT_REGS, smem)
     return tile_time_per_cell(cells * batch, PT_X * py * pz, threads,
@@ -123,6 +131,12 @@ def predict_seed_order(nx: int, ny: int, nz: int, batch: int, elem_bytes: int = 
     sms = device_sms() if sms is None else sms
     return sorted(((t, predict_seed_cost(nx, ny, nz, batch, t[0], t[1], elem_bytes, sms))
                    for t in PREDICT_TILES), key=lambda x: x[1])
+
+
+def with_default(order: List, default) -> List:
+    """A ranking with the library's own choice, which the model does not rate,
+    before it."""
+    return [(default, None)] + [c for c in order if c[0] != default]
 
 
 # ---------------------------------------------------------------------------
@@ -150,6 +164,24 @@ def _load_cache() -> Dict:
         return {}
 
 
+@functools.lru_cache(maxsize=None)
+def kernels_version() -> str:
+    """A digest of the library's source: what a timed choice is true of."""
+    here = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
+    h = hashlib.sha256()
+    for name in sorted(os.listdir(here)) if os.path.isdir(here) else ():
+        if name.endswith((".cu", ".cuh", ".h")):
+            with open(os.path.join(here, name), "rb") as f:
+                h.update(f.read())
+    return h.hexdigest()[:16]
+
+
+def _cached(key: str) -> Optional[Dict]:
+    """The choice stored for key, if it was timed with these kernels."""
+    hit = _load_cache().get(key)
+    return hit if hit and hit.get("version") == kernels_version() else None
+
+
 def _store_cache(key: str, value: Dict) -> None:
     path = cache_path()
     data = _load_cache()
@@ -172,10 +204,10 @@ def _stack(a, batch: int):
 def autotune(nx: int, ny: int, nz: int, batch: int = 1, precision: str = "fp32_refine",
              top: int = 3, steps: int = 2, dt: float = 5e-4, grid_kwargs: Optional[dict] = None,
              seed: int = 0, use_cache: bool = True) -> Dict:
-    """Chooses the predictor tile and tile_z for a grid by timing the best
-    seeded candidates: `top` predictor tiles (their predictor launches alone)
-    and `top` tile_z values (`steps` fine steps
-    after a warm one).  Returns {"predict_tile": (py, pz), "tile_z": tz,
+    """Chooses the predictor tile and tile_z for a grid by timing `top`
+    candidates of each, the library's own choice ((0, 0), 0) and the best
+    seeded ones: the predictor launches alone, then `steps` fine steps after a
+    warm one.  Returns {"predict_tile": (py, pz), "tile_z": tz,
     "seed": {...}, "ms": {...}, "cached": bool}; timed results are cached."""
     import torch
 
@@ -186,14 +218,14 @@ def autotune(nx: int, ny: int, nz: int, batch: int = 1, precision: str = "fp32_r
     dev = torch.cuda.get_device_name(torch.cuda.current_device())
     key = cache_key(nx, ny, nz, batch, precision, bc, dev)
     if use_cache and kw.get("solid") is None:
-        hit = _load_cache().get(key)
+        hit = _cached(key)
         if hit:
             return {"predict_tile": tuple(hit["predict_tile"]), "tile_z": hit["tile_z"],
                     "seed": hit.get("seed"), "ms": hit.get("ms"), "cached": True}
     sms = device_sms()
     esz = 4 if precision == "fp32_refine" else 8
-    porder = predict_seed_order(nx, ny, nz, batch, esz, sms)
-    zorder = seed_order(nx, ny, nz, batch, sms=sms)
+    porder = with_default(predict_seed_order(nx, ny, nz, batch, esz, sms), (0, 0))
+    zorder = with_default(seed_order(nx, ny, nz, batch, sms=sms), 0)
     init = inputs.random_state(nx, ny, nz, seed=seed, sigma=0.1, bc=bc, solid=kw.get("solid"))
     ms_pred: Dict[str, float] = {}
     ms_step: Dict[str, float] = {}
@@ -232,7 +264,8 @@ def autotune(nx: int, ny: int, nz: int, batch: int = 1, precision: str = "fp32_r
                     "tile_z": [[t, c] for t, c in zorder], "sms": sms},
            "ms": {"predict": ms_pred, "step": ms_step}, "cached": False}
     if use_cache and kw.get("solid") is None:
-        _store_cache(key, {k: v for k, v in out.items() if k != "cached"})
+        _store_cache(key, {**{k: v for k, v in out.items() if k != "cached"},
+                           "version": kernels_version()})
     return out
 
 
@@ -240,8 +273,8 @@ def autotune_tile_z(nx: int, ny: int, nz: int, batch: int = 1, top: int = 3, ste
                     dt: float = 5e-4, candidates: Iterable[int] = TILE_Z,
                     grid_kwargs: Optional[dict] = None, seed: int = 0) -> Dict:
     """tile_z alone (the predictor tile left at its default): times `steps`
-    fine steps (after one warm step) of a seeded state for the `top`
-    seed-ranked candidates; returns {"tile_z": best, "seed": [...],
+    fine steps (after one warm step) of a seeded state for `top` candidates,
+    the library's own choice (0) and the best ranked ones; returns {"tile_z": best, "seed": [...],
     "ms_per_step": {tz: ms}}.  grid_kwargs go to Grid (re, precision, bc...)."""
     import torch
 
@@ -249,7 +282,7 @@ def autotune_tile_z(nx: int, ny: int, nz: int, batch: int = 1, top: int = 3, ste
     from .api import Grid
     kw = dict(grid_kwargs or {})
     bc = kw.get("bc", ("wall", "wall", "wall"))
-    order = seed_order(nx, ny, nz, batch, candidates)
+    order = with_default(seed_order(nx, ny, nz, batch, candidates), 0)
     init = inputs.random_state(nx, ny, nz, seed=seed, sigma=0.1, bc=bc,
                                solid=kw.get("solid"))
     times: Dict[int, float] = {}
@@ -268,14 +301,14 @@ def autotune_tile_z(nx: int, ny: int, nz: int, batch: int = 1, top: int = 3, ste
     return {"tile_z": best, "seed": order, "ms_per_step": times}
 
 
-COARSE_TILE_Z = (4, 8)
+COARSE_TILE_Z = (0, 4, 8)
 
 
 def parareal_candidates(nx: int, ny: int, nz: int, slices: int, top: int = 2,
                         coarse_candidates: Iterable[int] = COARSE_TILE_Z,
                         sms: Optional[int] = None) -> List[Tuple[int, int]]:
-    """The (tile_z, coarse_tile_z) pairs autotune_parareal times: the `top`
-    seeded tile_z values for a batch of half the slices (the pipelined
+    """The seeded (tile_z, coarse_tile_z) pairs autotune_parareal times: the
+    `top` seeded tile_z values for a batch of half the slices (the pipelined
     schedule's chunks), each with every coarse candidate."""
     order = seed_order(nx, ny, nz, (slices + 1) // 2, sms=sms)
     return [(tz, ctz) for tz, _ in order[:max(1, top)] for ctz in coarse_candidates]
@@ -290,8 +323,9 @@ def autotune_parareal(nx: int, ny: int, nz: int, slices: int, fine_steps: int,
     coarse_tile_z for ns_parareal_iterate by timing Parareal iterations.
 
     A call of two or more iterations sweeps the slices in two chunks pipelined
-    with the coarse chain, so the sweep's candidates are the `top` seeded
-    tile_z values for a batch of half the slices; the chain shares the GPU
+    with the coarse chain, so the sweep's `top` candidates are the library's own
+    choice (0) and the best seeded tile_z values for a batch of half the slices;
+    the chain shares the GPU
     with the sweeps, and which march suits it then is measured rather than
     modelled (the seed model assumes a launch has the SMs to itself), over
     `coarse_candidates`.  Each pair is timed over `iterations` iterations of
@@ -309,17 +343,21 @@ def autotune_parareal(nx: int, ny: int, nz: int, slices: int, fine_steps: int,
     key = (cache_key(nx, ny, nz, slices, precision, bc, dev) +
            f"|parareal|S{fine_steps}|M{coarse_steps}|dt{dt:g}")
     if use_cache and kw.get("solid") is None:
-        hit = _load_cache().get(key)
+        hit = _cached(key)
         if hit:
             return {"tile_z": hit["tile_z"], "coarse_tile_z": hit["coarse_tile_z"],
                     "ms_per_iteration": hit.get("ms_per_iteration"), "seed": hit.get("seed"),
                     "cached": True}
-    order = seed_order(nx, ny, nz, (slices + 1) // 2)
+    order = with_default(seed_order(nx, ny, nz, (slices + 1) // 2), 0)
+    coarse_candidates = tuple(coarse_candidates)
+    pairs = [(0, ctz) for ctz in coarse_candidates]
+    if top > 1:
+        pairs += parareal_candidates(nx, ny, nz, slices, top - 1, coarse_candidates)
     if init is None:
         init = inputs.random_state(nx, ny, nz, seed=seed, sigma=0.1, bc=bc,
                                    solid=kw.get("solid"))
     times: Dict[str, float] = {}
-    for tz, ctz in parareal_candidates(nx, ny, nz, slices, top, coarse_candidates):
+    for tz, ctz in pairs:
         g = Grid(nx, ny, nz, batch=slices, precision=precision, tile_z=tz, coarse_tile_z=ctz,
                  **kw)
         u0 = g.state_from(init)
@@ -338,5 +376,6 @@ def autotune_parareal(nx: int, ny: int, nz: int, slices: int, fine_steps: int,
     out = {"tile_z": tz, "coarse_tile_z": ctz, "ms_per_iteration": times,
            "seed": [[t, c] for t, c in order], "cached": False}
     if use_cache and kw.get("solid") is None:
-        _store_cache(key, {k: v for k, v in out.items() if k != "cached"})
+        _store_cache(key, {**{k: v for k, v in out.items() if k != "cached"},
+                           "version": kernels_version()})
     return out

@@ -37,10 +37,10 @@ def test_seed_candidates_are_even_and_fit_the_grid():
 def test_predictor_seed_ranks_every_instantiated_tile():
     big = at.predict_seed_order(64, 64, 64, 32, 4, sms=152)
     assert {t for t, _ in big} == set(at.PREDICT_TILES)
-    # a full batch fills the GPU with most tiles: a small surface per cell
-    # with every SM's slots filled wins (32 x 8 x 8 fits 3 CTAs an SM by
-    # shared memory, and its waves leave slots idle)
-    assert big[0][0] == (16, 4)
+    # a full batch fills the GPU with every tile (registers hold two CTAs of 256
+    # threads an SM whatever the march: the ring of planes does not grow with
+    # it), so the smallest surface per cell wins
+    assert big[0][0] == (8, 8)
     one = at.predict_seed_order(32, 32, 32, 1, 4, sms=152)
     # one small state leaves SMs idle with any tile: the shortest march per
     # thread (the fewest staged elements per thread) wins
@@ -69,3 +69,19 @@ def test_parareal_candidates_pair_seeded_sweep_marches_with_the_chain_candidates
     # an odd slice count rounds the chunk up
     assert at.parareal_candidates(32, 32, 32, 7, top=1, coarse_candidates=(8,), sms=152) == \
         [(at.seed_order(32, 32, 32, 4, sms=152)[0][0], 8)]
+
+
+def test_choices_timed_with_other_kernels_are_not_reused(tmp_path, monkeypatch):
+    monkeypatch.setenv("NS_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    assert at._cached("a") is None
+    at._store_cache("a", {"tile_z": 8})  # as stored before choices had a version
+    at._store_cache("b", {"tile_z": 8, "version": "another"})
+    at._store_cache("c", {"tile_z": 8, "version": at.kernels_version()})
+    assert at._cached("a") is None and at._cached("b") is None
+    assert at._cached("c")["tile_z"] == 8
+
+
+def test_the_library_choice_comes_before_the_ranking():
+    order = at.with_default([(8, 0.1), (0, 0.2), (4, 0.3)], 0)
+    assert order == [(0, None), (8, 0.1), (4, 0.3)]
+    assert 0 in at.COARSE_TILE_Z
