@@ -47,10 +47,13 @@ WORKLOAD = ("64^3 lid-driven cavity, Re=1000, u_lid=1, walls on all faces; initi
             "(seed 0), projected; 32 Parareal slices x 50 fine steps (dt=5e-4); coarse "
             "propagator 5 steps of 5e-3 per slice; one step = one Parareal iteration")
 
-# Algorithmic traffic of the finest-level solver kernels, in words (FP32 or
-# FP64 values) per cell per launch: each array is read or written once per
-# launch, neighbour reads come from cache.  Multigrid path (finest-level
-# smoothing on):
+# Algorithmic traffic of the sweep's kernels, in bytes per cell per launch: each
+# array is read or written once per launch, neighbour reads come from cache.  A
+# grid of the multigrid preconditioner takes its pressure corrections from the
+# direct solve where it can (its launches are then in the profile), else from
+# preconditioned BiCGStab; the same profile kind is another kernel on each.
+#
+# Multigrid path, in words (FP32 or FP64 values; finest-level smoothing on):
 #   krylov_A   p = r + beta (p - omega v) and 2 Jacobi sweeps: r, p, v -> p, y
 #   mg_restrict0  residual of the sweeps, restricted: p|s, y -> coarse (1/8)
 #   mg_prolong0   y += P e: y, coarse e (1/8) -> y
@@ -58,37 +61,115 @@ WORKLOAD = ("64^3 lid-driven cavity, Re=1000, u_lid=1, walls on all faces; initi
 #   krylov_B   s = r - alpha v and 2 Jacobi sweeps: r, v -> s, z
 #   mg_lap_t   t = L z, (t, s), (t, t): z, s -> t
 #   krylov_C   x += alpha y + omega z, r = s - omega t: x, y, z, s, t, r_hat -> x, r
+#   mg_coarse, mg_block, mg_cluster: their units are words moved
 WORDS_MG = {"krylov_A": 5, "mg_restrict0": 2.125, "mg_prolong0": 2.125, "mg_lap_v": 3,
-            "krylov_B": 4, "mg_lap_t": 3, "krylov_C": 8,
-            # direct solve (boxes without solid cells): a plane's transforms and
-            # the equations along z read and write the field once each
-            "direct_xy": 2, "direct_z": 2}
+            "krylov_B": 4, "mg_lap_t": 3, "krylov_C": 8, "mg_coarse": 1, "mg_block": 1,
+            "mg_cluster": 1}
 # plain BiCGStab: A reads r, p, v, r_hat, writes p, v; B reads r, v, writes t;
 # C reads x, p, r, v, t, r_hat, writes x, r
 WORDS_PLAIN = {"krylov_A": 6, "krylov_B": 3, "krylov_C": 8}
-
-# Bytes per cell per launch of the step and refinement kernels, FP32+refine
-# multigrid path (velocities and increments FP32; b and the caller's p FP64;
-# the iterate p, residual r, warm start w and last pressure q float-float,
-# 8 bytes each):
+# Step kernels of the FP32+refine multigrid path (velocities and increments FP32;
+# b and the caller's p FP64; the iterate p, residual r, warm start w and last
+# pressure q float-float, 8 bytes each):
 #   predict     u, v, w -> dt*RHS increments:             3*4 + 3*4
 #   divergence  increments -> b (FP64):                    3*4 + 8
 #   correct     u, increments, p, q -> u, p (FP64), w, q:  3*4 + 3*4 + 8 + 8 + 3*4 + 8 + 8 + 8
 #   solve_init  b, w -> p, r, r32, r_hat:                   8 + 8 + 8 + 8 + 2*4
 #   refine      p, r, e -> p, r, r32, r_hat:                8 + 8 + 4 + 8 + 8 + 2*4
-BYTES_STEP_FP32 = {"predict": 24, "divergence": 20, "correct": 76, "solve_init": 40,
-                   "refine": 44}
-
+BYTES_MG_FP32 = {"predict": 24, "divergence": 20, "correct": 76, "solve_init": 40, "refine": 44}
+# Direct path, FP32+refine (r, w, q float-float; e FP32):
+#   inner_init  the call's p (FP64) -> w, q:                8 + 8 + 8
+#   solve_init  increments, w -> r (the call's first step reads u too): 3*4 + 8 + 8
+#   direct_xy   a plane's values through an axis or both:   4 + 4
+#   direct_z    spectral columns in place:                  4 + 4
+#   refine      r, e -> r (from the fourth application of a solve on also the
+#               oldest one apart into the base):            8 + 4 + 8
+#   correct     see direct_correct_bytes
+BYTES_DIRECT_FP32 = {"predict": 24, "inner_init": 24, "solve_init": 28, "direct_xy": 8,
+                     "direct_z": 8, "refine": 20}
+# Direct path, FP64 (all FP64; mixed: the transforms, columns and e in FP32):
+#   predict u, v, w -> F*: 48; divergence F* -> b: 32; solve_init b, w -> b, x, r, r_hat: 48;
+#   refine x, r, e -> x, r: 40; correct F*, x, p -> u, p, w: 80
+BYTES_DIRECT_FP64 = {"predict": 48, "divergence": 32, "solve_init": 48, "direct_xy": 16,
+                     "direct_z": 16, "refine": 40, "correct": 80}
+BYTES_DIRECT_MIXED = dict(BYTES_DIRECT_FP64, direct_xy=10, direct_z=8, refine=36)
+MIXED_CELLS = 3 << 17  # FP64 grids of this many cells over all states: FP32 corrections
 
 KERNEL_NAMES = {"krylov_A": "k_mg_src_pair<SRC_P> / k_mg_src<SRC_P> / k_bicg_A",
                 "krylov_B": "k_mg_src_pair<SRC_S> / k_mg_src<SRC_S> / k_bicg_B",
-                "krylov_C": "k_mg_update_pair / k_mg_update / k_bicg_C", "mg_lap_v": "k_mg_lapdot_pair<0> / k_mg_lapdot_v",
+                "krylov_C": "k_mg_update_pair / k_mg_update / k_bicg_C",
+                "mg_lap_v": "k_mg_lapdot_pair<0> / k_mg_lapdot_v",
                 "mg_lap_t": "k_mg_lapdot_pair<1> / k_mg_lapdot_t",
                 "mg_restrict0": "k_mg_restrict (finest)",
-                "mg_prolong0": "k_mg_prolong_pair / k_mg_prolong (finest)", "predict": "k_predict_tile",
-                "divergence": "k_divergence", "correct": "k_correct_ff",
-                "direct_xy": "k_dir_xy", "direct_z": "k_dir_z",
-                "solve_init": "k_mg_refine_init_ff", "refine": "k_mg_refine_update_ff"}
+                "mg_prolong0": "k_mg_prolong_pair / k_mg_prolong (finest)",
+                "predict": "k_predict_tile", "divergence": "k_divergence",
+                "correct": "k_correct_ff", "solve_init": "k_mg_refine_init_ff",
+                "refine": "k_mg_refine_update_ff"}
+KERNEL_NAMES_DIRECT = {"predict": "k_predict_tile", "direct_xy": "k_dir_xy / k_dir_x, k_dir_y",
+                       "direct_z": "k_dir_z"}
+KERNEL_NAMES_DIRECT_FP32 = dict(KERNEL_NAMES_DIRECT, inner_init="k_dir_load_p",
+                                solve_init="k_dir_start", refine="k_dir_refine",
+                                correct="k_dir_correct")
+KERNEL_NAMES_DIRECT_FP64 = dict(KERNEL_NAMES_DIRECT, divergence="k_divergence",
+                                solve_init="k_mg_init_warm", refine="k_dir_update",
+                                correct="k_correct")
+
+
+def direct_correct_bytes(prof, share):
+    """k_dir_correct, bytes per cell (share: of the applications launched, those
+    made): reads u, the increment, the base of p and
+    the applications still apart (three at most), writes u; every step but a
+    call's last also reads q and writes w and q, the last one writes p (FP64)."""
+    steps = max(1, prof["correct"]["launches"])
+    apart = min(3.0, share * prof["refine"]["launches"] / steps)
+    last = min(1.0, prof["inner_init"]["launches"] / steps)
+    return 12 + 12 + 8 + 4 * apart + 12 + (1.0 - last) * 24 + last * 8
+
+
+# launches that a state which has converged leaves at once
+ITERATION_KINDS = ("krylov_A", "mg_restrict0", "mg_prolong0", "mg_lap_v", "krylov_B", "mg_lap_t",
+                   "krylov_C", "mg_coarse", "mg_block", "mg_cluster", "direct_xy", "direct_z",
+                   "refine")
+
+
+def active_share(g, slices):
+    """The share of the states that an iteration's launches of the sweep find
+    iterating: iterations made over those launched, in one more sweep."""
+    state = type(slices)(*[t[:N_SLICES].clone() for t in slices.fields()])
+    before = g.stats()["krylov_iters"]
+    g.profile(True, min_batch=2)
+    g.step_fine(state, DT_FINE, FINE_STEPS)
+    prof = g.profile_read()
+    g.profile(False)
+    return share_of(g.stats()["krylov_iters"] - before, prof, N_SLICES)
+
+
+def share_of(iterations, prof, batch):
+    direct = prof["direct_xy"]["launches"] > 0
+    launched = prof["refine" if direct else "krylov_C"]["launches"] * batch
+    return min(1.0, iterations / launched) if launched else 1.0
+
+
+def traffic_model(precision, preconditioner, prof, cells, share=1.0):
+    """(bytes per cell and launch, kernel names, solver) of the kernels that a
+    profile saw run; cells: of the grid, all states; share: as active_share."""
+    if preconditioner == "multigrid" and prof["direct_xy"]["launches"] > 0:
+        if precision == "fp32_refine":
+            return (dict(BYTES_DIRECT_FP32, correct=direct_correct_bytes(prof, share)),
+                    KERNEL_NAMES_DIRECT_FP32,
+                    "direct solve (dense transforms along x and y, three-point equations along "
+                    "z) in FP32 inside float-float refinement")
+        mixed = cells >= MIXED_CELLS
+        return (BYTES_DIRECT_MIXED if mixed else BYTES_DIRECT_FP64, KERNEL_NAMES_DIRECT_FP64,
+                "direct solve (dense transforms along x and y, three-point equations along z), "
+                + ("FP32 corrections of the FP64 residual" if mixed else "FP64"))
+    esz = 4 if precision == "fp32_refine" else 8
+    words = WORDS_MG if preconditioner == "multigrid" else WORDS_PLAIN
+    out = {k: w * esz for k, w in words.items()}
+    if precision == "fp32_refine" and preconditioner == "multigrid":
+        out.update(BYTES_MG_FP32)
+    return (out, KERNEL_NAMES, "BiCGStab + multigrid V(2,0) right preconditioner"
+            if preconditioner == "multigrid" else "BiCGStab")
 
 
 def parse():
@@ -466,22 +547,18 @@ def run_ours(args, world, rank, local, pg):
     ms_profiled = e0.elapsed_time(e1) / args.steps
     prof = g.profile_read()
     g.profile(False)
+    share = active_share(g, slices)
 
     # ---- roofline: dominant kernel and the whole sweep -----------------------
-    esz = 4 if prec == "fp32_refine" else 8
-    words = WORDS_MG if args.preconditioner == "multigrid" else WORDS_PLAIN
     peak = float(peaks["hbm_gbs"])
-    bpc = {k: wpc * esz for k, wpc in words.items()}
-    if prec == "fp32_refine" and args.preconditioner == "multigrid":
-        bpc.update(BYTES_STEP_FP32)
-    # the coarser levels count words moved (cell_units are words there)
-    bpc.update({"mg_coarse": esz, "mg_block": esz, "mg_cluster": esz})
+    bpc, names, solver = traffic_model(prec, args.preconditioner, prof,
+                                       N_SLICES * N_CELLS ** 3, share)
     per_kernel = {}
     for k, b in bpc.items():
         kp = prof[k]
         if kp["ms"] <= 0 or kp["launches"] == 0:
             continue
-        bytes_alg = kp["cell_units"] * b
+        bytes_alg = kp["cell_units"] * b * (share if k in ITERATION_KINDS else 1.0)
         per_kernel[k] = {"achieved_gbs": bytes_alg / (kp["ms"] / 1e3) / 1e9,
                          "frac": bytes_alg / (kp["ms"] / 1e3) / 1e9 / peak,
                          "ms_per_step": kp["ms"] / args.steps,
@@ -498,13 +575,15 @@ def run_ours(args, world, rank, local, pg):
     achieved = per_kernel[kern]["achieved_gbs"]
     traffic = traffic_for(kern, tiles["tile_z"] or 8)
     per_launch_units = kp["cell_units"] / max(kp["launches"], 1)
+    launch_bytes = per_kernel[kern]["bytes_per_step"] * args.steps / max(kp["launches"], 1)
     sweep_ms = sum(v["ms"] for v in prof.values()) / args.steps
     modelled_ms = sum(v["ms_per_step"] for v in per_kernel.values())
     sweep_bytes = sum(v["bytes_per_step"] for v in per_kernel.values())
-    roofline = {"bound": "hbm", "kernel": KERNEL_NAMES[kern], "achieved": achieved,
+    roofline = {"bound": "hbm", "kernel": names[kern], "achieved": achieved,
                 "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": f"{peak_kind} hbm_gbs",
-                "algorithmic_bytes_per_launch": per_launch_units * bpc[kern],
+                "algorithmic_bytes_per_launch": launch_bytes,
+                "active_share": share,
                 "avg_launch_us": 1e3 * kp["ms"] / max(kp["launches"], 1),
                 "traffic": (traffic * per_launch_units) if traffic else None,
                 "timing": "separate profiled pass of the same iterations (CUDA events "
@@ -567,8 +646,7 @@ def run_ours(args, world, rank, local, pg):
         "dtype": "f32+f64refine" if prec == "fp32_refine" else "f64",
         "data": "synthetic",
         "config": {"workload": WORKLOAD, "precision": prec, "slices": N_SLICES,
-                   "solver": "BiCGStab + multigrid V(2,0) right preconditioner"
-                   if args.preconditioner == "multigrid" else "BiCGStab",
+                   "solver": solver,
                    "fine_steps_per_slice": FINE_STEPS, "coarse_steps_per_slice": COARSE_STEPS,
                    "grid": [N_CELLS] * 3, "parallelism": f"replicas x{world}",
                    "schedule": schedule_text(args.parareal_chunk),
@@ -579,8 +657,9 @@ def run_ours(args, world, rank, local, pg):
                             "the iteration index (every fine and coarse solve starts from its "
                             "own warm start); the call's pipeline fill and drain are inside "
                             "the timed region",
-                   "l2": "working set > L2 (no flush needed): ~%.0f MB of Krylov vectors"
-                         % (N_SLICES * N_CELLS ** 3 * esz * 8 / 1e6)},
+                   "l2": "working set > L2 (no flush needed): ~%.0f MB of states, increments "
+                         "and pressures" % (N_SLICES * N_CELLS ** 3 *
+                                            (6 * (4 if prec == "fp32_refine" else 8) + 16) / 1e6)},
         "roofline": roofline,
         "cpu_baseline": cpu,
         "e2e": e2e,
@@ -637,13 +716,13 @@ def run_coarse_only(args):
     """The serial coarse chain alone (the G sweep of one Parareal iteration,
     without the update kernels), for profilers: `steps` repetitions, on a
     batch-1 grid tiled like Parareal's coarse grid (--coarse-tile-z cells per
-    thread in z; 0: 8, the library's default for it)."""
+    thread in z; 0: the library's default for one state)."""
     import torch
     from paper_1705_06149_gb300 import Grid
     init = initial_field_gpu(args.precision)
     g = Grid(N_CELLS, N_CELLS, N_CELLS, re=RE, precision=args.precision, batch=1,
              preconditioner=args.preconditioner, inner_rtol=args.inner_rtol,
-             tile_z=args.coarse_tile_z or 8)
+             tile_z=args.coarse_tile_z)
     st = g.state_from(init)
     g.project(st)
     dtc = DT_FINE * FINE_STEPS / COARSE_STEPS
@@ -723,12 +802,10 @@ def run_adjoint(args):
     peaks, peak_kind = measured_peaks()
     peak = float(peaks["hbm_gbs"])
     cells = n ** 3
-    # the adjoint kernels per adjoint step and cell, in values: (dR/du)^T mu
-    # reads u and mu and writes the result (3 + 3 + 3), the finishing update
-    # reads mu and acc and writes lambda and acc (4 per component), the copy
-    # mu <- lambda reads and writes 3 each; the terminal condition (once) is
-    # not counted
-    words_adj = 9 + 12 + 6
+    # the reverse step's kernel per step and cell, in values: it reads u and mu
+    # and writes lambda (3 + 3 + 3); the copies between them are no launches of
+    # the profile, the terminal condition (once) is not counted
+    words_adj = 9
     adj = prof["adjoint"]
     adj_bytes = nsteps * cells * words_adj * esz
     kernels = {k: {"ms": v["ms"], "launches": v["launches"]} for k, v in prof.items()
@@ -938,7 +1015,7 @@ def run_peaks(args):
 
 def fp64_comparators(init, start, ref):
     """Rates of the FP64 batched sweep and of the per-slice FP64 paths (one
-    slice per call, with the multigrid preconditioner and with plain
+    slice per call, with the library's default solver and with plain
     BiCGStab), each over a bounded sample of the same workload after a
     warm-up, every solve to the relative residual 1e-10 that the FP32+refine
     path's FP64 refinement reaches; with start/ref given (the oracle's start
@@ -986,8 +1063,8 @@ def fp64_comparators(init, start, ref):
         t = timed(per_slice)
         out[name] = {"value": len(one) * steps * N_CELLS ** 3 / t, "unit": UNIT,
                      "sample": f"{len(one)} slices x {steps} fine steps, one slice per call, "
-                               f"{'multigrid-preconditioned' if pc == 'multigrid' else 'plain'} "
-                               f"BiCGStab, Poisson rtol {rtol:g}",
+                               + ("the library's default solver" if pc == "multigrid" else
+                                  "plain BiCGStab") + f", Poisson rtol {rtol:g}",
                      "krylov_iters_per_solve": (g1.stats()["krylov_iters"] - it0)
                      / (len(one) * steps)}
         if start is not None:
