@@ -55,10 +55,9 @@ def test_tile_z_changes_results_only_at_rounding_level(prec, tol):
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32_refine"])
 def test_predictor_tiles_agree_to_rounding(prec):
-    """Every face is evaluated from the same operands whatever the tile, so
-    every predictor tile the autotuner may choose gives the same predictor
-    and steps up to rounding (the compiler may fuse products into
-    multiply-adds differently per instantiated shape)."""
+    """Every face takes the same operations whatever the tile: every predictor
+    tile the autotuner may choose gives the same predictor and the same steps
+    bit for bit (rounding included)."""
     from paper_1705_06149_gb300.autotune import PREDICT_TILES
     dims = (40, 24, 20)  # ragged against every tile
     init = inputs.random_state(*dims, seed=5, sigma=0.3)
@@ -73,13 +72,27 @@ def test_predictor_tiles_agree_to_rounding(prec):
         if ref is None:
             ref = got
         else:
-            # the predictor alone agrees to a few ulps; two steps carry those
-            # through the pressure solves (conditioning ~1e3)
-            tol = 1e-11 if prec == "fp64" else 1e-5
             for a, b in zip(got, ref):
-                a, b = a.double(), b.double()
-                assert float((a - b).norm()) <= tol * float(b.norm()), tile
+                assert torch.equal(a, b), tile
         g.close()
+
+
+# sizes and batches whose automatic tile is 16 or 32 columns wide and one, two,
+# 8, 16 or 32 planes long
+@pytest.mark.parametrize("prec", ["fp64", "fp32_refine"])
+@pytest.mark.parametrize("dims,batch", [((40, 24, 20), 1), ((16, 16, 16), 1), ((13, 9, 40), 3),
+                                        ((31, 33, 37), 4), ((33, 64, 50), 24),
+                                        ((48, 40, 70), 40), ((64, 64, 64), 6)])
+def test_automatic_predictor_tiles_give_the_same_bits(dims, batch, prec):
+    init = inputs.random_state(*dims, seed=6, sigma=0.3)
+    out = []
+    for tile in ((0, 0), (8, 4)):
+        g = Grid(*dims, re=300.0, precision=prec, batch=batch, predict_tile=tile)
+        st = g.state_from(init)
+        out.append([t.clone() for t in g.predict(st, 1e-3)])
+        g.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
 
 
 def test_predictor_tile_outside_the_instantiated_set_is_rejected():

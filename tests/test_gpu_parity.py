@@ -403,16 +403,23 @@ def test_chunked_parareal_is_bit_identical(prec, pc):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32_refine"])
-def test_chunked_parareal_with_cluster_v_cycles_is_bit_identical(prec):
+def test_chunked_parareal_with_cluster_v_cycles_is_bit_identical(prec, monkeypatch):
     """On a 32^3 grid the V-cycle's coarse levels run as thread-block
     clusters (4 CTAs per state), launched for 24 slices at once by the
     unchunked sweep and for chunks of 12 by the pipelined schedule; the
     pipelined iterations give the unchunked ones bit for bit."""
+    # (boxes without solid cells take the direct solve by default)
+    monkeypatch.setenv("NS_DIRECT", "0")
     runs = {}
     for chunk in (-1, 0):
         g = Grid(32, 32, 32, re=400.0, precision=prec, batch=24, parareal_chunk=chunk)
         u0 = g.state_from(inputs.random_state(32, 32, 32, seed=13, sigma=0.2))
         g.project(u0)
+        g.profile(True)
+        g.step_fine(u0.clone(), 1e-3, 1)
+        prof = g.profile_read()
+        g.profile(False)
+        assert prof["mg_cluster"]["launches"] > 0 and prof["direct_xy"]["launches"] == 0
         slices = g.zeros(25)
         k, d = g.parareal(u0, slices, 24, 4, 1, 1e-3, kmax=2)
         assert k == 2
