@@ -75,22 +75,33 @@ typedef struct {
                                 step (<= 0: 3e-4)                                    */
     int refine_maxit;        /* FP32_REFINE: outer corrections per solve before
                                 NS_ERR_NOT_CONVERGED (<= 0: 40)                      */
-    int batch;               /* capacity: largest batch one call may advance (>= 1)  */
+    int batch;               /* capacity: largest batch one call may advance (>= 1).
+                                A state gets the same bits whatever the batch of a
+                                call and its place in it.  Grids of another capacity
+                                agree with it only at rounding level (FP64: within
+                                poisson_rtol): the march of FP32_REFINE's direct
+                                solve (tile_z = 0) and, in FP64, the precision of
+                                the corrections follow nx ny nz batch.             */
     int preconditioner;      /* ns_preconditioner: BiCGStab as in Section 2 without
                                 (NS_PC_NONE) or with one multigrid V-cycle as right
                                 preconditioner (NS_PC_MULTIGRID; falls back to
                                 NS_PC_NONE on grids it cannot coarsen far enough).
                                 With NS_PC_MULTIGRID, a box without solid cells
                                 whose planes, or the matrices of an axis, fit one
-                                SM's shared memory takes its corrections from a
-                                direct solve of L e = r instead (transforms along x
-                                and y, three-point equations along z; the same
-                                stopping tolerances, one application counted as one
-                                iteration; large FP64 calls apply it in FP32 to the
-                                FP64 residual), unless its tolerance is below 1e-14;
-                                with solid cells it preconditions conjugate
-                                gradients in FP32_REFINE's inner solves (one
-                                iteration counted as one).  NS_DIRECT=0 in the
+                                SM's shared memory (up to about 300 cells along x
+                                and y in FP32_REFINE, 200 in FP64; 512 and 256
+                                along z) takes its corrections from a direct solve
+                                of L e = r instead (transforms along x and y,
+                                three-point equations along z; the same stopping
+                                tolerances, one application counted as one
+                                iteration; FP64 grids of nx ny nz batch >= 393216
+                                apply it in FP32 to the FP64 residual), unless its
+                                tolerance is below 1e-14 or L's condition number
+                                above 1e7 (FP64: 1e12); with solid cells that leave
+                                one region of fluid and are not single cells
+                                scattered over large planes it preconditions
+                                conjugate gradients in FP32_REFINE's inner solves
+                                (one iteration counted as one).  NS_DIRECT=0 in the
                                 environment at ns_create_grid, or any of the
                                 multigrid's variables below, keeps the V-cycle.
                                 The levels with at most 4096 cells (FP32_REFINE;
@@ -105,9 +116,11 @@ typedef struct {
                                 NS_MG_CLUSTER=0 at ns_create_grid turns that off. */
     int tile_z;              /* cells each thread marches along z in the stencil and
                                 solver kernels: an even number >= 2 (clamped to nz);
-                                0: 8, less on small grids.  Results depend on it at
-                                rounding level (it fixes the order of the per-state
-                                reductions).                                        */
+                                0: 8, less on small grids; FP32_REFINE's direct
+                                solve then takes 4 to 64, the longest that leaves
+                                every SM eight CTAs with batch states.  Results
+                                depend on it at rounding level (it fixes the order
+                                of the per-state reductions).                       */
     int parareal_chunk;      /* ns_parareal_iterate: slices per chunk of the fine
                                 sweep (> 0).  With the multigrid solver the chunks'
                                 sweeps and coarse chains are graph launches

@@ -275,7 +275,7 @@ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 // eighth fewer columns idle than 32, and of the shapes below the longest march
 // that still gives the call about 1500 warps (ten per SM): a longer march
 // stages fewer halo planes per cell (64^3 x 32 states, FP32: 399 us with one
-// plane, 225 with 4, 156 with 32), too few warps leave SMs idle (one 16^3
+// plane, 225 with 4, 164 with 32), too few warps leave SMs idle (one 16^3
 // state, FP64: 16 us with one plane, 154 with 16).
 void predict_tile_auto(const int n[3], int cap, int& px, int& py, int& pz) {
     static const int shapes[2][7][2] = {
@@ -317,8 +317,8 @@ void setup_geo(ns_grid* g) {
         G.fih2[a] = (float)G.ih2[a];
     }
     G.finv_re = (float)G.inv_re;
-    // cells per thread along z: fixed per grid (not per batch) so that every
-    // state is reduced over the same CTAs whatever the batch size; an even
+    // cells per thread along z: fixed per grid (not per call) so that every
+    // state is reduced over the same CTAs whatever the batch of a call; an even
     // number so that the multigrid restriction pairs stay inside a CTA.  By
     // default 8, halved (to 2) while a state's tiles leave half of the SMs
     // without one: the march is a chain of latencies (a 16^3 FP64 step 126 ->
@@ -577,8 +577,9 @@ ns_status setup_direct_of(ns_grid* g, DirPlan<T>& P) {
 // FP64 grids of DIR_MIXED_CELLS cells or more (all states) take FP32 corrections
 // (DM_MIXED) of the FP64 iterate and residual, two or three in the place of
 // one: an FP64 application is bound by its pipe (64^3 x 4 states: 125 us per
-// transform against 8).  4 steps of 64^3 x 4 FP64 3.14 -> 2.47 ms, of one state
-// equal, of smaller ones slower by their launches (32^3 0.58 -> 0.73 ms).
+// transform against 14 forward and 11 inverse).  4 steps of 64^3 x 4 FP64 3.14 ->
+// 2.47 ms, of one state equal, of smaller ones slower by their launches (32^3 0.58
+// -> 0.73 ms).
 constexpr long long DIR_MIXED_CELLS = 3 << 17;
 
 // Whether conjugate gradients preconditioned by the box solve suit the solid
@@ -587,12 +588,12 @@ constexpr long long DIR_MIXED_CELLS = 3 << 17;
 // gather them and the rounding of r in them spoils alpha (a sealed room of 10^3
 // cells in 32 x 24 x 16: no convergence where BiCGStab takes 24 iterations).
 // (Single closed cells have no equation.)  And not on planes of more than 8192
-// cells with scattered solid cells, whose iterations then outweigh their price
-// (an iteration 562 us against 770, 128^3 x 8): 1 % single cells 11.7 iterations
-// a step against 6.3, 9.7 ms against 9.2; 3 % 12.3 against 9.8; 10 % 22.2 against
-// 16.6.  There, 0.3 % 8.8 against 8.9, 8 boxes 10.3 against 12.1, pillars of 3 x 3
-// cells 8 apart 11.2 against 13.4, a plate 39 against 51; on 64^2 planes 10 %
-// single cells 2.7 against 2.9.
+// cells with scattered solid cells, which take so many more iterations that their
+// price no longer pays: a step of 128^3 x 8 with 1 % single cells takes 11.7
+// iterations against BiCGStab's 6.3, 9.7 ms against 9.2; 3 % 12.3 ms against 9.8;
+// 10 % 22.2 against 16.6.  But 0.3 % 8.8 against 8.9, 8 boxes 10.3 against 12.1,
+// pillars of 3 x 3 cells 8 apart 11.2 against 13.4, a plate 39 against 51; on 64^2
+// planes 10 % single cells 2.7 against 2.9.
 bool cg_suits(const ns_grid* g) {
     const Geo& G = g->geo;
     const bool periodic[3] = {G.bc[0] == BC_PERIODIC, G.bc[1] == BC_PERIODIC,

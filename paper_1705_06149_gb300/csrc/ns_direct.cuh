@@ -5,8 +5,9 @@
 // a periodic one), so e is r transformed along x and y, a three-point equation
 // along z per (kx, ky), and transformed back.  One application in FP32 leaves
 // 1e-4 .. 5e-7 of the residual (its rounding times the conditioning of L), so
-// two applications inside the float-float refinement reach what five BiCGStab
-// iterations with two V-cycles each reach.
+// one to three applications inside the float-float refinement (64^3: one or two,
+// 256^3: two or three) reach what five BiCGStab iterations with two V-cycles each
+// reach.
 //
 // Transforms (k_dir_xy).  Both bases split into vectors even and odd under
 // j -> n-1-j, so a line folded into its sums and differences takes two
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(DIR_MAX_THREADS)
 // rows of DIR_LNC columns in both parities, so folding and unfolding need no
 // exchange.  256 x 256 planes, FP32: 128 products per value and axis, bound by
 // the FP32 pipe and the shared-memory reads that feed it (4 of each per 16
-// products): 485 us per axis for 67e6 cells, floor of the pipe alone 221 us
+// products): 483 to 518 us per axis for 67e6 cells, floor of the pipe alone 221 us
 // (16 rows per thread, half the warps: 545 to 919 us).
 constexpr int DIR_LRB = 8, DIR_LNC = 2;
 
@@ -1071,8 +1072,10 @@ __global__ void __launch_bounds__(NTHREADS)
 // obstacles' shapes and not on the grid (an extension of a fluid field into a
 // solid has at most a fixed multiple of its energy).  An iteration is one
 // application and three passes, 56 B/cell next to the transforms.  128^3 x 8
-// states, 8 boxes: 21 iterations of 392 us per step, where BiCGStab, whose
-// V-cycles know the solids on the finest level only, took 23 of 770 us.
+// states, 8 boxes, two steps: 21.5 working iterations of 553 us a step (transforms
+// 286, columns 49, the passes 218) and 8 launched for states that had converged,
+// 85 us each: 31.4 ms; with BiCGStab, whose V-cycles know the solids on the finest
+// level only, 47 ms.
 //
 // The direction survives the outer corrections, which replace r by the true
 // residual: beta = -(z, q) / (p, q) makes the next one conjugate to the last and
@@ -1411,7 +1414,9 @@ inline std::vector<T> dir_tables(const DirPlan<T>& P, const int bc[3], const dou
 // does not give it) the longest march of 64 cells or less that leaves the SMs
 // eight CTAs deep, 4 below that.  A CTA's sums end in FP64, which a longer march
 // pays less often: 64^3 x 32 states, 8 -> 32 cells: start 137 -> 115 us,
-// correction of r 73 -> 66, of u 143 -> 136 (then 120 by its loads' order).
+// correction of r 73 -> 66, of u 143 -> 136; with a warp per sum in the last CTA
+// and the loads before any condition 109, 60 and 120.  The capacity decides, so
+// grids of different capacity add a state's partials in different orders.
 inline DirTile dir_tile_of(const int n[3], int cap, int tile_z) {
     DirTile t;
     const int xt = (n[0] + 31) / 32;

@@ -78,11 +78,12 @@ struct KBuf {       // Krylov vectors of all states, [batch][cells]
 // face value is selected by integer comparisons and costs four FP64
 // operations); FP32, instruction issue (hence the march: staging a tile with
 // its z halo at once took half of all instructions) with 16 warps per SM (24
-// with a third of the registers less: 168 us against 156 below).
+// with a third of the registers less: 168 us against 156).
 // Measured against evaluating every y flux twice and the face value by
 // comparisons, from 32 x 8 x 4 tiles staged at once: 64^3 x 32 states FP32
-// 280 -> 156 us, 64^3 FP32 27 -> 12 us, 64^3 x 4 FP64 747 -> 294 us, 16^3 FP64
-// 121 -> 16 us.
+// 280 -> 159 us (164 with the low parts of the coefficients, 18 more multiply-adds
+// a cell), 64^3 FP32 27 -> 12 us, 64^3 x 4 FP64 747 -> 282 us, 16^3 FP64 121 -> 16
+// us.
 constexpr int PT_X = 32, PT_Y = 8, PT_Z = 4;
 constexpr int PT_THREADS = PT_X * PT_Y;
 constexpr int PH = 2;       // halo

@@ -190,3 +190,35 @@ def test_masks_that_keep_the_multigrid_solve(dims, mask, direct):
     # of 40 solves times 20 max(n) iterations
     assert g.stats()["krylov_iters"] <= 100
     g.close()
+
+
+# what include/ns.h says of the bits: one grid gives a state the same ones whatever
+# the batch of a call and its place in it; grids of another capacity agree at
+# rounding level (FP64 from 393216 cells on: FP32 corrections, so within the
+# solves' tolerance)
+@pytest.mark.parametrize("prec,dims,caps", [("fp32_refine", (64, 64, 32), (1, 5, 24)),
+                                            ("fp64", (64, 64, 48), (1, 3)),
+                                            ("fp64", (20, 12, 16), (1, 5))])
+def test_bits_of_a_state_belong_to_its_grid(prec, dims, caps):
+    inits = [inputs.random_state(*dims, seed=60 + s, sigma=0.2) for s in range(3)]
+    out = {}
+    for cap in caps:
+        g = Grid(*dims, re=500.0, precision=prec, batch=cap)
+        alone = [g.state_from(i) for i in inits]
+        for st in alone:
+            g.step_fine(st, 5e-4, 3)
+        if cap >= 3:
+            both = g.state_from([np.stack([i[c] for i in inits]) for c in range(4)])
+            g.step_fine(both, 5e-4, 3)
+            for c in range(4):
+                for s in range(3):
+                    assert torch.equal(both.fields()[c][s], alone[s].fields()[c][0]), (cap, c, s)
+        out[cap] = [torch.cat([st.fields()[c] for st in alone]).double() for c in range(4)]
+        g.close()
+    for cap in caps[1:]:
+        # FP32: a rounding of the stored velocity; its divergence over dt in p.
+        # FP64: residuals of 1e-12 through L's condition number (a few 1e3)
+        for c in range(4):
+            a, b = out[cap][c], out[caps[0]][c]
+            tol = 1e-8 if prec == "fp64" else (1e-6 if c < 3 else 1e-5)
+            assert float((a - b).norm()) <= tol * float(b.norm()), (cap, c)
