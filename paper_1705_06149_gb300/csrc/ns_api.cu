@@ -344,34 +344,6 @@ void setup_geo(ns_grid* g) {
     if (deflt) predict_tile_auto(G.n, g->cap, G.ptx, G.pty, G.ptz);
 }
 
-// Face codes of the finest level with solid cells (FC_FLUID and one bit per
-// face joining two fluid cells), by the same rules as the pressure operator.
-std::vector<uint8_t> face_codes(const Geo& G, const uint8_t* solid) {
-    const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
-    std::vector<uint8_t> code((size_t)nx * ny * nz, 0);
-    auto at = [&](int i, int j, int k) { return solid[((size_t)k * ny + j) * nx + i] == 0; };
-    for (int k = 0; k < nz; ++k)
-        for (int j = 0; j < ny; ++j)
-            for (int i = 0; i < nx; ++i) {
-                if (!at(i, j, k)) continue;
-                unsigned m = FC_FLUID;
-                const int c[3] = {i, j, k};
-                for (int a = 0; a < 3; ++a) {
-                    for (int dir = 0; dir < 2; ++dir) {
-                        int q[3] = {c[0], c[1], c[2]};
-                        q[a] += dir ? 1 : -1;
-                        if (q[a] < 0 || q[a] >= G.n[a]) {
-                            if (G.bc[a] != BC_PERIODIC) continue;
-                            q[a] = q[a] < 0 ? G.n[a] - 1 : 0;
-                        }
-                        if (at(q[0], q[1], q[2])) m |= 1u << (2 * a + dir);
-                    }
-                }
-                code[((size_t)k * ny + j) * nx + i] = (uint8_t)m;
-            }
-    return code;
-}
-
 // Multigrid hierarchy: halve every size while all are even and >= 4; the
 // levels from the first one with at most `block_cells` cells down run in one
 // CTA per state.  Returns false when the hierarchy is not usable (the block
@@ -2947,7 +2919,11 @@ ns_status ns_create_grid(const ns_grid_desc* desc, void* cuda_stream, ns_grid** 
         st = setup_direct(g);
         if (g->mg && d.solid_mask) {
             // solid cells enter the finest level through its face codes
-            const std::vector<uint8_t> code = face_codes(g->geo, d.solid_mask);
+            const int* bc = g->geo.bc;
+            const bool periodic[3] = {bc[0] == BC_PERIODIC, bc[1] == BC_PERIODIC,
+                                      bc[2] == BC_PERIODIC};
+            const std::vector<uint8_t> code =
+                mask_face_codes(g->geo.n, periodic, d.solid_mask, (uint8_t)FC_FLUID);
             void* fc = nullptr;
             A(&fc, ncell);
             if (st == NS_OK &&

@@ -1,5 +1,5 @@
-"""csrc/ns_mask.h (solid cells, solid surface and separate fluid regions of a
-mask) against plain numpy: random masks of every density, sealed rooms, rooms
+"""csrc/ns_mask.h (face codes, solid cells, solid surface and separate fluid
+regions of a mask) against plain numpy: random masks of every density, sealed rooms, rooms
 joined only through a periodic axis, walls and wraps, extents down to 2.  No GPU
 needed."""
 from __future__ import annotations
@@ -10,6 +10,8 @@ import subprocess
 
 import numpy as np
 import pytest
+
+from test_masked_mg_emulation import FC_FLUID, _codes
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1705_06149_gb300", "csrc")
@@ -26,6 +28,10 @@ int main(int, char** argv) {
     if (!f || fread(s.data(), 1, s.size(), f) != s.size()) return 2;
     const MaskShape m = mask_shape(n, per, s.data());
     printf("%lld %lld %lld\\n", m.solid, m.faces, m.rooms);
+    const std::vector<uint8_t> c = mask_face_codes(n, per, s.data(), 64);
+    f = fopen(argv[8], "wb");
+    fwrite(c.data(), 1, c.size(), f);
+    fclose(f);
     return 0;
 }
 """
@@ -101,6 +107,9 @@ def test_mask_shape_matches_numpy(driver, periodic):
     for solid in _masks():
         solid.tofile(d / "s.bin")
         r = subprocess.run([exe, *map(str, solid.shape[::-1]), *map(str, periodic),
-                            str(d / "s.bin")], capture_output=True, text=True)
+                            str(d / "s.bin"), str(d / "c.bin")], capture_output=True, text=True)
         assert r.returncode == 0, r.stderr[-2000:]
         assert tuple(map(int, r.stdout.split())) == _shape(solid, periodic), (solid.shape, periodic)
+        code = np.fromfile(d / "c.bin", dtype=np.uint8).reshape(solid.shape)
+        assert FC_FLUID == 64
+        assert (code == _codes(solid, ["periodic" if p else "wall" for p in periodic])).all()
