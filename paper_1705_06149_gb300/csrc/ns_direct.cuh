@@ -92,13 +92,17 @@ __device__ __forceinline__ int dir_slot(const SliceCtl* c, int mode) {
 // log2 of the scale that brings a residual of squared norm rr to an RMS of order
 // one, from the exponents of rr and of the cells (no FP64 root or quotient: one
 // thread computes it at the end of a kernel that everything waits for).  `top`
-// keeps the scale itself in range: 100 where it is an FP32 value, DIR_SHIFT64
-// where it is an FP64 one.
-constexpr int DIR_SHIFT64 = 500;
+// keeps the scale itself in range.
 __device__ __forceinline__ int dir_shift(double rr, int log2n, int top) {
     if (!(rr > 0.0) || !isfinite(rr)) return 0;
     const int e = (int)((__double_as_longlong(rr) >> 52) & 0x7ff) - 1023;
     return -max(-top, min(top, (e - log2n) / 2));
+}
+// The same for the FP64 residuals that FP32 corrections are made of: none where
+// the residual is within 2^24 of one, FP32's range having room for that.
+__device__ __forceinline__ int dir_shift64(double rr, int log2n) {
+    const int e = dir_shift(rr, log2n, 500);
+    return e >= -24 && e <= 24 ? 0 : e;
 }
 inline int dir_log2(long long n) {
     int l = 0;
@@ -109,7 +113,7 @@ template <typename T>
 __device__ __forceinline__ double dir_scale(const SliceCtl* c, bool inv, const DirPlan<T>& P) {
     if (sizeof(T) == 8 || P.mode == DM_PRECOND) return 1.0;
     // (an FP64 grid's e stays scaled: unscaled it may be out of FP32's range)
-    if (P.mode == DM_MIXED) return inv ? 1.0 : ldexp(1.0, dir_shift(c->rr, P.log2n, DIR_SHIFT64));
+    if (P.mode == DM_MIXED) return inv ? 1.0 : ldexp(1.0, dir_shift64(c->rr, P.log2n));
     return inv ? 1.0f / c->o_fsc : c->o_fsc;
 }
 
@@ -1016,8 +1020,7 @@ __global__ void __launch_bounds__(NTHREADS)
     int i, j, k0;
     lev_origin(L, blockIdx.x, i, j, k0);
     const double rmean = c->rmean;
-    const double unscale =
-        sizeof(E) == 4 ? ldexp(1.0, -dir_shift(c->rr, log2n, DIR_SHIFT64)) : 1.0;
+    const double unscale = sizeof(E) == 4 ? ldexp(1.0, -dir_shift64(c->rr, log2n)) : 1.0;
     double rr = 0.0, sx = 0.0, sr = 0.0;
     if (i < L.n[0] && j < L.n[1]) {
         const int k1 = min(k0 + L.tz, L.n[2]);
