@@ -1326,8 +1326,12 @@ inline bool dir_sizes(const int n[3], bool per_z, int planes, DirPlan<T>& P) {
     P.hxp = (P.hx + 3) / 4 * 4;
     // rows and columns per thread: shared-memory cycles of a block of 16 rows
     // (with the padded rows), (rows / 4 + columns) / columns; a call of about
-    // one plane per SM prefers more threads (153 planes of 45 x 37: 8.5 us
-    // against 11.1; 192 of 96 x 64: 22 against 19)
+    // one plane per SM prefers more threads.  FP32, us per transform with more
+    // threads / fewer: 152 planes of 45 x 37 9.8 / 12.2, of 64 x 64 11.7 / 12.2, of
+    // 96 x 64 14.5 / 15.5, of 96 x 96 20.9 / 18.3; 192 planes 10.9 / 12.2, 14.2 /
+    // 14.2, 20.4 / 18.3, 31.1 / 28.7: past one plane per SM the large planes, which
+    // hold most of the time, turn (planes below 64 x 64 do not; FP64 ones of 45 x 37
+    // take 59 / 77 there)
     const bool few = planes < 176;
     P.ncol = few ? 1 : 2;
     P.rb = 4;
