@@ -104,6 +104,8 @@ typedef struct {
                                 (one iteration counted as one).  NS_DIRECT=0 in the
                                 environment at ns_create_grid, or any of the
                                 multigrid's variables below, keeps the V-cycle.
+                                (The coarse propagator's companion grid is made by
+                                the first call that needs it and reads them then.)
                                 The levels with at most 4096 cells (FP32_REFINE;
                                 512 in FP64) run in one CTA per state; the
                                 environment variable NS_MG_BLOCK_CELLS, read at
